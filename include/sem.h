@@ -166,8 +166,8 @@ sem_status sem_mesh_weights(const sem_mesh* mesh, double* mult_dev, double* mask
  *   h1_eff(q) = h1 * h1_dev[q],  h2_eff(q) = h2 * h2_dev[q]
  * with the scalar h1, h2 that the call passes.  Both NULL restores the
  * constant-coefficient operator.  The factors are stored pre-multiplied
- * (h1 G, h2 B in FP64, FP32 and the FP32 pair form: 128 B per local point
- * with both), so the operator kernels read no more bytes than without.
+ * (h1 G, h2 B in the forms the chosen kernels read: at most 176 B per local
+ * point with both), so the operator kernels read no more bytes than without.
  * sem_mesh_geometry and sem_rhs keep using the plain G and B.
  * A projection space on the mesh drops its basis at its next solve.
  * Errors: SEM_ERR_INVALID (null mesh; an h1 value <= 0 or an h2 value < 0 or
@@ -633,13 +633,14 @@ sem_status sem_gs_halo(int64_t E, int N, const int64_t* vert, const int32_t* ele
 sem_status sem_mesh_vertices(const sem_mesh_desc* desc, int64_t* vert_host, int64_t* E_out);
 
 /* Which kernel FP64 requests on this mesh use, as chosen by the autotuner at
- * creation: 1 = double-float (FP32-pair) arithmetic, 0 = native FP64. */
+ * creation: 1 = double-float (FP32-pair) arithmetic, 0 = native FP64 (on the
+ * FP64 pipe or, as accurate, in 64-bit fixed point). */
 int sem_mesh_fp64_kernel(const sem_mesh* mesh);
 
 /* Local-operator kernel variant the autotuner chose for `prec` (SEM_FP64
  * or SEM_FP32): 0 / 1 register kernels with ~256 / ~128 threads per CTA,
  * 2 / 3 (FP32) persistent kernels fed by bulk copies into a shared-memory
- * ring.  -1 for a bad argument. */
+ * ring, 4 / 5 (FP64) the fixed-point kernels.  -1 for a bad argument. */
 int sem_mesh_ax_variant(const sem_mesh* mesh, sem_prec prec);
 
 /* Synchronise `stream` and report whether a local-operator kernel launched

@@ -1,12 +1,14 @@
 // C ABI: mesh construction and the operator entry points (sem_ax, sem_gs,
 // sem_rhs, sem_apply, sem_jacobi).  The solver lives in solver.cpp and the
 // server in server.cpp.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
 #include <memory>
 #include <string>
 
+#include "fixed.cuh"
 #include "kernels.h"
 #include "sem_internal.h"
 #include "solver.h"
@@ -54,6 +56,12 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->G32lo);
   dev_free(m->B32);
   dev_free(m->B32lo);
+  dev_free(m->Gfx);
+  dev_free(m->fx_sG);
+  dev_free(m->fx_eB);
+  dev_free(m->fx_tab);
+  dev_free(m->fx_ti);
+  dev_free(m->wq);
   dev_free(m->dK);
   dev_free(m->dB);
   dev_free(m->wm);
@@ -69,11 +77,14 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->cG64);
   dev_free(m->cG32);
   dev_free(m->cG32lo);
+  dev_free(m->cGfx);
+  dev_free(m->cfx_sG);
   dev_free(m->cdK);
   dev_free(m->cB64);
   dev_free(m->cB32);
   dev_free(m->cB32lo);
   dev_free(m->cdB);
+  dev_free(m->cfx_eB);
   dev_free(m->Fgl);
   dev_free(m->pdinv);
   dev_free(m->Igl);
@@ -96,28 +107,36 @@ struct CoefArrays {
   double* G64 = nullptr;
   float* G32 = nullptr;
   float* G32lo = nullptr;
+  int4* Gfx = nullptr;
+  int* fx_sG = nullptr;
   double* dK = nullptr;
   double* B64 = nullptr;
   float* B32 = nullptr;
   float* B32lo = nullptr;
   double* dB = nullptr;
+  int* fx_eB = nullptr;
   size_t bytes = 0;
   void release() {
     dev_free(G64);
     dev_free(G32);
     dev_free(G32lo);
+    dev_free(Gfx);
+    dev_free(fx_sG);
     dev_free(dK);
     dev_free(B64);
     dev_free(B32);
     dev_free(B32lo);
     dev_free(dB);
+    dev_free(fx_eB);
     bytes = 0;
   }
 };
 
-size_t coef_bytes(const sem_mesh* m) {
-  const size_t P = (size_t)m->n_local;
-  return (m->cG64 ? P * (6 * 8 + 6 * 4 + 6 * 4 + 8) : 0) + (m->cB64 ? P * (8 + 4 + 4 + 8) : 0);
+// Frees *p and takes its size off the tally.
+template <typename T>
+void dev_drop(T*& p, size_t count, size_t& tally) {
+  if (p) tally -= count * sizeof(T);
+  dev_free(p);
 }
 
 sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, CoefArrays& c, cudaStream_t s) {
@@ -126,21 +145,32 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
   if (h1) {
     SEM_TRY(dev_alloc(&c.G64, 6 * P, c.bytes));
     SEM_TRY(dev_alloc(&c.G32, 6 * P, c.bytes));
-    SEM_TRY(dev_alloc(&c.G32lo, 6 * P, c.bytes));
     SEM_TRY(dev_alloc(&c.dK, P, c.bytes));
+    if (m->fp64_df) SEM_TRY(dev_alloc(&c.G32lo, 6 * P, c.bytes));
+    if (m->Gfx) {
+      SEM_TRY(dev_alloc(&c.Gfx, 3 * P, c.bytes));
+      SEM_TRY(dev_alloc(&c.fx_sG, m->E, c.bytes));
+    }
   }
   if (h2) {
     SEM_TRY(dev_alloc(&c.B64, P, c.bytes));
     SEM_TRY(dev_alloc(&c.B32, P, c.bytes));
-    SEM_TRY(dev_alloc(&c.B32lo, P, c.bytes));
     SEM_TRY(dev_alloc(&c.dB, P, c.bytes));
+    if (m->fp64_df) SEM_TRY(dev_alloc(&c.B32lo, P, c.bytes));
+    if (m->Gfx) SEM_TRY(dev_alloc(&c.fx_eB, m->E, c.bytes));
   }
   size_t tmp = 0;
-  int* bad_d = nullptr;
-  SEM_TRY(dev_alloc(&bad_d, 1, tmp));
+  int* bad_d = nullptr;  // [2]: a bad coefficient; factors out of the fixed-point form's range
+  SEM_TRY(dev_alloc(&bad_d, 2, tmp));
   std::unique_ptr<int, void (*)(int*)> bad_guard(bad_d, [](int* p) { cudaFree(p); });
-  SEM_CUDA(cudaMemsetAsync(bad_d, 0, sizeof(int), s));
-  launch_fold_coef(m->G64, m->B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
+  SEM_CUDA(cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s));
+  const double* G = m->G64;
+  if (h1 && !G) {  // the plain factors once more
+    SEM_CUDA(launch_geometry(m->xyz, c.G64, nullptr, m->D64, m->wq, n, m->E, nullptr, s));
+    G = c.G64;
+    count_launches(1);
+  }
+  launch_fold_coef(G, m->B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
   if (h1) {
     launch_local_diag(c.G64, c.dK, m->D64, n, m->E, s);
     SEM_CUDA(launch_gs<double>(c.dK, gs_dev(m), 0, nullptr, s));
@@ -151,17 +181,82 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     SEM_CUDA(launch_gs<double>(c.dB, gs_dev(m), 0, nullptr, s));
     launch_split_f64(c.B64, c.B32, c.B32lo, P, s);
   }
+  if (m->Gfx && (h1 || h2)) {
+    SEM_CUDA(launch_fx_pack(c.G64, c.B64, m->fx_ti, n, m->E, c.Gfx, c.fx_sG, c.fx_eB, bad_d + 1, s));
+    count_launches(1);
+  }
   SEM_CUDA(cudaGetLastError());
   count_launches(1 + (h1 ? 3 : 0) + (h2 ? 2 : 0));
-  int bad = 0;
-  SEM_CUDA(cudaMemcpyAsync(&bad, bad_d, sizeof(int), cudaMemcpyDeviceToHost, s));
+  int bad[2] = {0, 0};
+  SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SEM_CUDA(cudaStreamSynchronize(s));
-  if (bad) {
-    set_error((bad & 1) ? "sem_mesh_set_coefficients: need finite h1 > 0 at every point"
-                        : "sem_mesh_set_coefficients: need finite h2 >= 0 at every point");
+  if (bad[0]) {
+    set_error((bad[0] & 1) ? "sem_mesh_set_coefficients: need finite h1 > 0 at every point"
+                           : "sem_mesh_set_coefficients: need finite h2 >= 0 at every point");
     return SEM_ERR_INVALID;
   }
+  if (bad[1]) {  // coefficients beyond 2^+-200: the kernels on the FP64 pipe take them
+    dev_drop(c.Gfx, 3 * P, c.bytes);
+    dev_drop(c.fx_sG, m->E, c.bytes);
+    dev_drop(c.fx_eB, m->E, c.bytes);
+  } else if (h1 && !m->G64) {
+    dev_drop(c.G64, 6 * P, c.bytes);  // as for the plain factors: no chosen kernel reads it
+  }
   return SEM_OK;
+}
+
+// The plain FP64 factors, where the tuning freed them (see drop_unused).
+sem_status restore_G64(sem_mesh* m, cudaStream_t s) {
+  if (m->G64) return SEM_OK;
+  SEM_TRY(dev_alloc(&m->G64, 6 * m->n_local, m->dev_bytes));
+  SEM_CUDA(launch_geometry(m->xyz, m->G64, nullptr, m->D64, m->wq, m->n, m->E, nullptr, s));
+  count_launches(1);
+  return SEM_OK;
+}
+
+// Once the kernels are chosen: the factors that none of them reads.
+void drop_unused(sem_mesh* m) {
+  const size_t P = (size_t)m->n_local;
+  if (!m->fp64_df) {
+    dev_drop(m->G32lo, 6 * P, m->dev_bytes);
+    dev_drop(m->B32lo, P, m->dev_bytes);
+  }
+  if (m->ax_var[0] >= kAxFixed && m->Gfx) dev_drop(m->G64, 6 * P, m->dev_bytes);
+}
+
+// D and D^T of the n GLL points as 64-bit integers (FxOp::tab), c 2^sc, split
+// for fixed.cuh.  Even n: for i, l < n/2 the pair (Ep, Em) = (D[i][l] +- D[i][n-1-l]) / 2;
+// odd n: the n x n entries.  sc makes the largest row sum at most 2^62, or 2^61 where six or
+// more terms meet: with inputs of 61 bits (even n) or 60 bits (odd n) that is the bound of fx::dot.
+void fx_tables(int n, const std::vector<double>& D, std::vector<int>& tab, int* sc) {
+  const bool even = n % 2 == 0;
+  const int h = even ? n / 2 : n;
+  tab.assign((size_t)2 * h * h * (even ? 4 : 2) + 2, 0);  // a multiple of 4 ints
+  tab.resize(tab.size() / 4 * 4);
+  for (int dir = 0; dir < 2; ++dir) {
+    auto at = [&](int i, int l) { return (long double)(dir == 0 ? D[i * n + l] : D[l * n + i]); };
+    auto coef = [&](int i, int l, int s) {
+      return even ? (s ? (at(i, l) - at(i, n - 1 - l)) / 2 : (at(i, l) + at(i, n - 1 - l)) / 2) : at(i, l);
+    };
+    long double top = 0;
+    for (int i = 0; i < h; ++i)
+      for (int s = 0; s < (even ? 2 : 1); ++s) {
+        long double sum = 0;
+        for (int l = 0; l < h; ++l) sum += std::fabs(coef(i, l, s));
+        top = std::max(top, sum);
+      }
+    int e = 0;
+    std::frexp(top, &e);  // top < 2^e
+    sc[dir] = (even ? (h >= 6 ? 61 : 62) : (h >= 10 ? 61 : 62)) - e;
+    size_t q = (size_t)dir * h * h * (even ? 4 : 2);
+    for (int i = 0; i < h; ++i)
+      for (int l = 0; l < h; ++l)
+        for (int s = 0; s < (even ? 2 : 1); ++s) {
+          const int2 v = fx::split(std::llround(std::ldexp(coef(i, l, s), sc[dir])));
+          tab[q++] = v.x;
+          tab[q++] = v.y;
+        }
+  }
 }
 
 sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
@@ -225,9 +320,10 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_TRY(dev_alloc(&m->G64, 6 * P, tb));
   SEM_TRY(dev_alloc(&m->B64, P, tb));
   SEM_TRY(dev_alloc(&m->G32, 6 * P, tb));
-  SEM_TRY(dev_alloc(&m->G32lo, 6 * P, tb));
   SEM_TRY(dev_alloc(&m->B32, P, tb));
-  SEM_TRY(dev_alloc(&m->B32lo, P, tb));
+  SEM_TRY(dev_alloc(&m->Gfx, 3 * P, tb));
+  SEM_TRY(dev_alloc(&m->fx_sG, E, tb));
+  SEM_TRY(dev_alloc(&m->fx_eB, E, tb));
   SEM_TRY(dev_alloc(&m->dK, P, tb));
   SEM_TRY(dev_alloc(&m->dB, P, tb));
   SEM_TRY(dev_alloc(&m->wm, P, tb));
@@ -244,27 +340,35 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_TRY(dev_alloc(&m->eodf, eodf.size(), tb));
   }
 
+  // fixed-point tables of D and D^T, and the weights' exponents
+  std::vector<int> tab, ti(n);
+  fx_tables(n, D, tab, m->fx_sc);
+  const double wmax = *std::max_element(w.begin(), w.end());
+  for (int i = 0; i < n; ++i) ti[i] = (int)std::lround(-std::log2(w[i] / wmax));
+  SEM_TRY(dev_alloc(&m->fx_tab, tab.size() / 4, tb));
+  SEM_TRY(dev_alloc(&m->fx_ti, n, tb));
+  SEM_TRY(dev_alloc(&m->wq, n, tb));
+
   size_t tmp_bytes = 0;
-  double *xi_d = nullptr, *w_d = nullptr, *tlev_d = nullptr;
-  int* bad_d = nullptr;
+  double *xi_d = nullptr, *tlev_d = nullptr;
+  int* bad_d = nullptr;  // [2]: det J <= 0; factors out of the fixed-point form's range
   struct Tmp {
     double** a;
-    double** b;
     double** c;
     int** f;
     ~Tmp() {
       if (*a) cudaFree(*a);
-      if (*b) cudaFree(*b);
       if (*c) cudaFree(*c);
       if (*f) cudaFree(*f);
     }
-  } tmp{&xi_d, &w_d, &tlev_d, &bad_d};
+  } tmp{&xi_d, &tlev_d, &bad_d};
   SEM_TRY(dev_alloc(&xi_d, n, tmp_bytes));
-  SEM_TRY(dev_alloc(&w_d, n, tmp_bytes));
-  SEM_TRY(dev_alloc(&bad_d, 1, tmp_bytes));
+  SEM_TRY(dev_alloc(&bad_d, 2, tmp_bytes));
 
   SEM_CUDA(cudaMemcpyAsync(xi_d, xi.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
-  SEM_CUDA(cudaMemcpyAsync(w_d, w.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->wq, w.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->fx_tab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->fx_ti, ti.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D64, D.data(), n * n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32, D32.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32lo, D32lo.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -272,7 +376,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_CUDA(cudaMemcpyAsync(m->eo64, eo64.data(), eo64.size() * sizeof(double), cudaMemcpyHostToDevice, s));
     SEM_CUDA(cudaMemcpyAsync(m->eodf, eodf.data(), eodf.size() * sizeof(float), cudaMemcpyHostToDevice, s));
   }
-  SEM_CUDA(cudaMemsetAsync(bad_d, 0, sizeof(int), s));
+  SEM_CUDA(cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s));
   SEM_CUDA(cudaMemsetAsync(m->dev_err, 0, sizeof(int), s));
   SEM_CUDA(cudaMemcpyAsync(m->wm, plan.wm.data(), P, cudaMemcpyHostToDevice, s));
   if (!plan.idx.empty())
@@ -294,22 +398,28 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_CUDA(cudaMemcpyAsync(m->xyz, d.xyz, 3 * P * sizeof(double), cudaMemcpyHostToDevice, s));
   }
   SEM_CUDA(cudaGetLastError());
-  SEM_CUDA(launch_geometry(m->xyz, m->G64, m->B64, m->D64, w_d, n, E, bad_d, s));
+  SEM_CUDA(launch_geometry(m->xyz, m->G64, m->B64, m->D64, m->wq, n, E, bad_d, s));
   // assembled diagonals for the Jacobi preconditioner: dK = QQ^T diag(stiffness), dB = QQ^T B
   launch_local_diag(m->G64, m->dK, m->D64, n, E, s);
   SEM_CUDA(launch_gs<double>(m->dK, gs_dev(m), 0, nullptr, s));
   SEM_CUDA(cudaMemcpyAsync(m->dB, m->B64, P * sizeof(double), cudaMemcpyDeviceToDevice, s));
   SEM_CUDA(launch_gs<double>(m->dB, gs_dev(m), 0, nullptr, s));
-  launch_split_f64(m->G64, m->G32, m->G32lo, 6 * P, s);
-  launch_split_f64(m->B64, m->B32, m->B32lo, P, s);
+  launch_split_f64(m->G64, m->G32, nullptr, 6 * P, s);  // the low parts: autotune_mesh, where they are needed
+  launch_split_f64(m->B64, m->B32, nullptr, P, s);
+  SEM_CUDA(launch_fx_pack(m->G64, m->B64, m->fx_ti, n, E, m->Gfx, m->fx_sG, m->fx_eB, bad_d + 1, s));
   SEM_CUDA(cudaGetLastError());
-  count_launches(7);
-  int bad = 0;
-  SEM_CUDA(cudaMemcpyAsync(&bad, bad_d, sizeof(int), cudaMemcpyDeviceToHost, s));
+  count_launches(8);
+  int bad[2] = {0, 0};
+  SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SEM_CUDA(cudaStreamSynchronize(s));
-  if (bad) {
+  if (bad[0]) {
     set_error("mesh has an element with det(J) <= 0");
     return SEM_ERR_BAD_MESH;
+  }
+  if (bad[1]) {
+    dev_drop(m->Gfx, 3 * P, tb);
+    dev_drop(m->fx_sG, E, tb);
+    dev_drop(m->fx_eB, E, tb);
   }
   m->glo = std::move(topo.glo);
   return SEM_OK;
@@ -395,6 +505,7 @@ sem_status sem_mesh_create(const sem_mesh_desc* desc, void* stream, sem_mesh** o
     delete m;
     return st;
   }
+  drop_unused(m);
   *out = m;
   return SEM_OK;
 }
@@ -424,6 +535,8 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   std::lock_guard<std::mutex> lk(m->ws_mutex);
   CoefArrays c;
   sem_status st = build_coef(m, h1_dev, h2_dev, c, s);
+  // h2 out of the fixed-point range: the kernels on the FP64 pipe read the plain factors
+  if (st == SEM_OK && h2_dev && !h1_dev && !c.fx_eB && m->Gfx) st = restore_G64(m, s);
   if (st != SEM_OK) {
     cudaStreamSynchronize(s);
     c.release();
@@ -432,7 +545,7 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   // the old arrays are freed below: cudaFree waits for kernels still reading
   // them (no device-wide synchronisation, see sem_mesh_destroy)
   if (m->ws) SEM_CUDA(cudaStreamSynchronize(m->ws->s));
-  m->dev_bytes -= coef_bytes(m);
+  m->dev_bytes -= m->coef_bytes;
   dev_free(m->cG64);
   dev_free(m->cG32);
   dev_free(m->cG32lo);
@@ -441,6 +554,9 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   dev_free(m->cB32);
   dev_free(m->cB32lo);
   dev_free(m->cdB);
+  dev_free(m->cGfx);
+  dev_free(m->cfx_sG);
+  dev_free(m->cfx_eB);
   m->cG64 = c.G64;
   m->cG32 = c.G32;
   m->cG32lo = c.G32lo;
@@ -449,7 +565,11 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   m->cB32 = c.B32;
   m->cB32lo = c.B32lo;
   m->cdB = c.dB;
-  m->dev_bytes += coef_bytes(m);
+  m->cGfx = c.Gfx;
+  m->cfx_sG = c.fx_sG;
+  m->cfx_eB = c.fx_eB;
+  m->coef_bytes = c.bytes;
+  m->dev_bytes += m->coef_bytes;
   m->coef_gen++;
   if (m->ws) m->ws->minv_h1 = NAN;  // the cached Jacobi inverse belongs to the old operator
   return SEM_OK;
@@ -494,9 +614,13 @@ sem_status sem_mesh_geometry(const sem_mesh* m, double* G_dev, double* B_dev, vo
     set_error("sem_mesh_geometry: null mesh");
     return SEM_ERR_INVALID;
   }
-  if (G_dev)
+  if (G_dev && m->G64)
     SEM_CUDA(cudaMemcpyAsync(G_dev, m->G64, 6 * m->n_local * sizeof(double), cudaMemcpyDeviceToDevice,
                              (cudaStream_t)stream));
+  if (G_dev && !m->G64) {  // not kept: the same kernel on the same coordinates gives the same factors
+    SEM_CUDA(launch_geometry(m->xyz, G_dev, nullptr, m->D64, m->wq, m->n, m->E, nullptr, (cudaStream_t)stream));
+    count_launches(1);
+  }
   if (B_dev)
     SEM_CUDA(cudaMemcpyAsync(B_dev, m->B64, m->n_local * sizeof(double), cudaMemcpyDeviceToDevice,
                              (cudaStream_t)stream));

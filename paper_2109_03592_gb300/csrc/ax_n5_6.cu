@@ -1,12 +1,13 @@
 // Local-operator kernels instantiated for polynomial orders 5, 6.
 // (One translation unit per order keeps the parallel build short.)
 #include "ax_eo_impl.cuh"
+#include "ax_fx_impl.cuh"
 #include "ax_impl.cuh"
 
 namespace sem {
 
 cudaError_t ax64_n5(int v, bool f, const AxParams<double>& p, cudaStream_t s, int* g) {
-  return dispatch_ax_n<double, 5>(v, f, p, s, g);
+  return dispatch_fp64_n<5>(v, f, p, s, g);
 }
 cudaError_t ax32_n5(int v, bool f, const AxParams<float>& p, cudaStream_t s, int* g) {
   return dispatch_ax_n<float, 5>(v, f, p, s, g);
@@ -16,7 +17,7 @@ cudaError_t axdf_n5(int v, bool f, const AxDFParams& p, cudaStream_t s, int* g) 
 }
 
 cudaError_t ax64_n6(int v, bool f, const AxParams<double>& p, cudaStream_t s, int* g) {
-  return dispatch_ax_n<double, 6>(v, f, p, s, g);
+  return dispatch_fp64_n<6>(v, f, p, s, g);
 }
 cudaError_t ax32_n6(int v, bool f, const AxParams<float>& p, cudaStream_t s, int* g) {
   return dispatch_ax_n<float, 6>(v, f, p, s, g);

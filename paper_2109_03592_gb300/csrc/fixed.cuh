@@ -1,0 +1,111 @@
+// 64-bit fixed-point arithmetic on the integer pipe, for the operators whose
+// results must be as accurate as FP64.
+//
+// GB300 issues 1.7 FP64 FMAs per clock and SM (measured), but 63 IMAD.WIDE
+// (32 x 32 + 64 -> 64 bits).  A contraction of fixed-point numbers v = vh 2^32 +
+// vl, c = ch 2^32 + cl (low halves signed) keeps the upper 64 bits of the
+// 128-bit products:
+//   sum_l c_l v_l / 2^64 = sum ch vh + (sum (ch vl + cl vh)) / 2^32 + O(1/4) per term,
+// three IMAD.WIDE per multiply-add (6 issue slots; an FP32 pair needs 12
+// instructions for 48 bits, a native FMA 60+ slots).  Values of one element share
+// one exponent and are kept left-aligned at 60 bits, so the rounding of each
+// stage is 2^-57 or less of the element's largest value.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+namespace sem {
+namespace fx {
+
+typedef long long ll;
+
+constexpr int kBits = 60;   // magnitudes of fields: at most 2^60
+constexpr int kOpExp = 200;  // exponents of G, B, h1, h2 on the integer path lie within 2^+-200
+
+// Where the pair (2f, 2f + 1) of a point's six factors lies within its element: for odd n by point,
+// for even n by (pair, octant point) and thread of the octant mapping, so that a warp reads 512 bytes.
+__host__ __device__ __forceinline__ int pair_index(int n, int f, int i, int j, int k) {
+  if (n & 1) return (f * n * n + k * n + j) * n + i;
+  const int h = n / 2, I = i >= h, J = j >= h, K = k >= h;
+  const int a = I ? n - 1 - i : i, b = J ? n - 1 - j : j, c = K ? n - 1 - k : k;
+  return (3 * (I + 2 * J + 4 * K) + f) * h * h * h + a + h * (b + h * c);
+}
+
+// A 64-bit value split with a signed low half: v = y 2^32 + x (the register order of v itself).
+__host__ __device__ __forceinline__ int2 split(ll v) {
+  const int l = (int)v;
+  return make_int2(l, (int)(v >> 32) + (int)((unsigned)l >> 31));
+}
+
+#ifdef __CUDACC__
+__device__ __forceinline__ ll mad(ll acc, int a, int b) { return acc + (ll)a * b; }
+
+// sum of c_l v_l / 2^64, rounded; the caller bounds sum |ch| + sum |vh| < 2^32 - 2^8
+template <int n>
+__device__ __forceinline__ ll dot(const int2 (&c)[n], const int2 (&v)[n]) {
+  ll m = 0x80000000ll;
+#pragma unroll
+  for (int l = 0; l < n; ++l) {
+    m = mad(m, c[l].x, v[l].y);
+    m = mad(m, c[l].y, v[l].x);
+  }
+  ll r = m >> 32;
+#pragma unroll
+  for (int l = 0; l < n; ++l) r = mad(r, c[l].y, v[l].y);
+  return r;
+}
+
+// The same sum, term by term.
+struct Dot {
+  ll h = 0, m = 0x80000000ll;
+  __device__ __forceinline__ void add(int2 c, int2 v) {
+    m = mad(mad(m, c.x, v.y), c.y, v.x);
+    h = mad(h, c.y, v.y);
+  }
+  __device__ __forceinline__ ll get() const { return h + (m >> 32); }
+};
+
+// Biased exponent (11 bits) of a double's high word.
+__device__ __forceinline__ int expo(int hi) { return (hi >> 20) & 0x7ff; }
+
+// x 2^(bits + 1022 - emax), truncated, for a finite x with biased exponent <= emax;
+// entries below 2^-bits of 2^(emax - 1022) and denormals give 0 (emax > 64).
+template <int bits = kBits>
+__device__ __forceinline__ ll from_double(double x, int emax) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | lo;
+  const int d = min(emax - expo(hi), 63);
+  const ll v = (ll)((m << (bits - 53)) >> d);
+  return hi < 0 ? -v : v;
+}
+
+// v 2^e, rounded to nearest; |e| small enough that the result is a normal number or 0.
+__device__ __forceinline__ double to_double(ll v, int e) {
+  const double d = __ll2double_rn(v);
+  const double s = __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
+  return v == 0 ? 0.0 : s;
+}
+
+__device__ __forceinline__ ll shl(ll v, int s) { return (ll)((unsigned long long)v << s); }
+// v 2^s for any s (arithmetic shift right for s < 0)
+__device__ __forceinline__ ll shift(ll v, int s) { return s >= 0 ? shl(v, min(s, 63)) : v >> min(-s, 63); }
+// bits that hold |hi word| of the largest value seen by `m` (m collects hi ^ (hi >> 31))
+__device__ __forceinline__ int mag(ll v) {
+  const int h = (int)(v >> 32);
+  return h ^ (h >> 31);
+}
+__device__ __forceinline__ int bits_of(int m) { return 64 - __clz(m); }
+
+// Factor f of point (i, j, k) of element e, back as a double.
+__device__ inline double factor(const int4* G, int sG, const int* ti, int n, int64_t e, int f, int i, int j, int k) {
+  const int4 x = G[e * 3 * n * n * n + pair_index(n, f >> 1, i, j, k)];
+  const int2 y = (f & 1) ? make_int2(x.z, x.w) : make_int2(x.x, x.y);
+  return ldexp(__ll2double_rn(shl(y.y, 32) + y.x), -(sG + ti[i] + ti[j] + ti[k]));
+}
+#endif
+
+}  // namespace fx
+}  // namespace sem

@@ -6,6 +6,7 @@
 // isoparametric reading): J_ab = dx_a/dr_b from D applied to the nodal
 // coordinates, G = w_i w_j w_k det(J) J^{-1} J^{-T} with g1..g6 = G_rr, G_ss,
 // G_tt, G_rs, G_rt, G_st, and B = w_i w_j w_k det(J).
+#include "fixed.cuh"
 #include "kernels.h"
 
 namespace sem {
@@ -105,7 +106,7 @@ __global__ void k_geometry(const double* __restrict__ xyz, double* __restrict__ 
     const double C21 = J[0][2] * J[1][0] - J[0][0] * J[1][2];
     const double C22 = J[0][0] * J[1][1] - J[0][1] * J[1][0];
     const double det = J[0][0] * C00 + J[0][1] * C01 + J[0][2] * C02;
-    if (!(det > 0.0)) atomicExch(bad, 1);
+    if (bad && !(det > 0.0)) atomicExch(bad, 1);
     // Jinv[b][a] = d r_b / d x_a = C[a][b] / det.  G = w3 det Jinv Jinv^T = w3 / det * C^T C
     const double w3 = wg[i] * wg[j] * wg[k];
     const double s = w3 / det;
@@ -122,7 +123,7 @@ __global__ void k_geometry(const double* __restrict__ xyz, double* __restrict__ 
     Ge[3 * n3] = g4;
     Ge[4 * n3] = g5;
     Ge[5 * n3] = g6;
-    B[e * n3 + p] = w3 * det;
+    if (B) B[e * n3 + p] = w3 * det;
   }
 }
 
@@ -164,9 +165,9 @@ __global__ void k_split_f64(const double* __restrict__ v, float* __restrict__ hi
 // point by h1 of that point, which is h1 G at the point; the mass term scales
 // B u by h2.  Bit 0 / 1 of *bad flags an h1 <= 0 / h2 < 0 or a non-finite
 // value.
-__global__ void k_fold_coef(const double* __restrict__ G, const double* __restrict__ B, const double* __restrict__ h1,
-                            const double* __restrict__ h2, double* __restrict__ cG, double* __restrict__ cB, int n3,
-                            int64_t P, int* bad) {
+__global__ void k_fold_coef(const double* G, const double* __restrict__ B, const double* __restrict__ h1,
+                            const double* __restrict__ h2, double* cG, double* __restrict__ cB, int n3, int64_t P,
+                            int* bad) {  // cG may be G
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < P; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = q / n3, r = q - e * n3;
     if (h1) {
@@ -190,7 +191,60 @@ __global__ void k_weights(const uint8_t* __restrict__ wm, double* mult, double* 
   }
 }
 
+// The fixed-point factors of the FP64 operator (FxOp): one CTA per element,
+// first the element's largest exponents of G 2^t and B 2^t, then the integers.
+// 62 bits for G: with fields of 60 bits the three terms of a point's product
+// meet the bound of fx::dot.  B stays as it is (its conversion is part of the
+// mass term); only its exponent is kept.
+__global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B,
+                                                 const int* __restrict__ ti, int n, int64_t E, int4* __restrict__ fG,
+                                                 int* __restrict__ sG, int* __restrict__ eB, int* bad) {
+  __shared__ int top[2];
+  const int n3 = n * n * n;
+  const int64_t e = blockIdx.x;
+  if (threadIdx.x < 2) top[threadIdx.x] = 0;
+  __syncthreads();
+  int mG = 0, mB = 0;
+  for (int p = threadIdx.x; p < n3; p += blockDim.x) {
+    const int t = ti[p % n] + ti[(p / n) % n] + ti[p / (n * n)];
+    if (G) {
+      int hi = 0;
+      for (int f = 0; f < 6; ++f) hi = max(hi, __double2hiint(G[(e * 6 + f) * n3 + p]) & 0x7fffffff);
+      mG = max(mG, fx::expo(hi) == 0x7ff ? 0x1000 : fx::expo(hi) + t);
+    }
+    if (B) {
+      const int hi = __double2hiint(B[e * n3 + p]) & 0x7fffffff;
+      mB = max(mB, fx::expo(hi) == 0x7ff ? 0x1000 : hi ? fx::expo(hi) + t : 0);
+    }
+  }
+  atomicMax(&top[0], mG);
+  atomicMax(&top[1], mB);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // an all-zero B (h2 = 0 at every point of the element) is in range
+    if ((G && abs(top[0] - 1023) > fx::kOpExp) || (B && top[1] != 0 && abs(top[1] - 1023) > fx::kOpExp))
+      atomicExch(bad, 1);
+    if (G) sG[e] = 62 + 1022 - top[0];
+    if (B) eB[e] = top[1] == 0 ? 1023 : top[1];
+  }
+  if (!G) return;
+  for (int q = threadIdx.x; q < 3 * n3; q += blockDim.x) {
+    const int p = q % n3, f = 2 * (q / n3);  // factors f and f + 1 of point p
+    const int i = p % n, j = (p / n) % n, k = p / (n * n);
+    const int t = ti[i] + ti[j] + ti[k];
+    const int2 x = fx::split(fx::from_double<62>(G[(e * 6 + f) * n3 + p], top[0] - t));
+    const int2 y = fx::split(fx::from_double<62>(G[(e * 6 + f + 1) * n3 + p], top[0] - t));
+    fG[e * 3 * n3 + fx::pair_index(n, f / 2, i, j, k)] = make_int4(x.x, x.y, y.x, y.y);
+  }
+}
+
 // ---- launchers ---------------------------------------------------------------
+
+cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, int n, int64_t E, int4* fG, int* sG,
+                           int* eB, int* bad, cudaStream_t s) {
+  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, ti, n, E, fG, sG, eB, bad);
+  return cudaGetLastError();
+}
 
 static int grid_for(int64_t m, int threads) {
   int64_t g = (m + threads - 1) / threads;

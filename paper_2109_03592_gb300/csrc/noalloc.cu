@@ -104,7 +104,7 @@ extern "C" sem_status sem_pcg_solve_noalloc(const sem_mesh* m, const double* b_d
   int var_native = 0, var_df = 0, use_df = 0;
   {
     std::lock_guard<std::mutex> lk(mm->ws_mutex);
-    var_native = m->ax_var[0];
+    var_native = ax64_variant(m);
     var_df = m->ax_var_dff;  // the fused form runs here
     use_df = m->fp64_df;
   }
@@ -134,9 +134,7 @@ extern "C" sem_status sem_pcg_solve_noalloc(const sem_mesh* m, const double* b_d
                    h2 != 0.0, m->E, z, p, dst, part_ax, m->eo64, m->eodf};
       return launch_ax_df(m->N, var_df, true, a, s, nullptr);
     }
-    AxParams<double> a{nullptr, w, m->opG64(), m->opB64(), m->D64, h1, h2, h2 != 0.0, m->E, z, p, dst, part_ax,
-                       m->dev_err};
-    return launch_ax_f64(m->N, var_native, true, a, s, nullptr);
+    return launch_ax_f64(m->N, var_native, true, ax64_params(m, nullptr, w, h1, h2, z, p, dst, part_ax), s, nullptr);
   };
 
   // The same rule as sem_pcg_solve's FP64 solve: CG runs on its recurrences;

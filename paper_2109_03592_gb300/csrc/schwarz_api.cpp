@@ -698,7 +698,7 @@ sem_status sem_schwarz_create(const sem_mesh* mesh, double h1, double h2, int fl
     return SEM_ERR_INVALID;
   }
   sem_mesh* m = const_cast<sem_mesh*>(mesh);
-  if (m->cG64 || m->cB64) {
+  if (m->cG32 || m->cB64) {
     set_error("sem_schwarz_create: the separable local solves take scalar h1, h2 (the mesh has per-point "
               "coefficients)");
     return SEM_ERR_INVALID;

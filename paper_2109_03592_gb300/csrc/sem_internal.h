@@ -102,12 +102,19 @@ struct sem_mesh {
 
   // device arrays (library-owned)
   double* xyz = nullptr;     // [E][3][n3]
-  double* G64 = nullptr;     // [E][6][n3]
+  double* G64 = nullptr;     // [E][6][n3]; freed after the tuning where no chosen kernel reads it
   double* B64 = nullptr;     // [E][n3]
   float* G32 = nullptr;      // [E][6][n3] round-to-nearest of G64 (the "hi" part)
-  float* G32lo = nullptr;    // [E][6][n3] float(G64 - G32): G64 ~ G32 + G32lo to 2^-48
+  float* G32lo = nullptr;    // [E][6][n3] float(G64 - G32): G64 ~ G32 + G32lo to 2^-48 (double-float only)
   float* B32 = nullptr;      // [E][n3] round-to-nearest of B64
-  float* B32lo = nullptr;    // [E][n3] float(B64 - B32)
+  float* B32lo = nullptr;    // [E][n3] float(B64 - B32) (double-float only)
+  int4* Gfx = nullptr;       // [E][3 n3] the factors in fixed point (FxOp); null where their exponents are out of range
+  int* fx_sG = nullptr;      // [E] FxOp::sG
+  int* fx_eB = nullptr;      // [E] FxOp::eB
+  int4* fx_tab = nullptr;    // D and D^T in fixed point (FxOp::tab)
+  int* fx_ti = nullptr;      // [n] (FxOp::ti)
+  int fx_sc[2] = {0, 0};     // FxOp::sc
+  double* wq = nullptr;      // [n] GLL weights
   double* dK = nullptr;      // [n_local] QQ^T diag of the stiffness (h1 = 1, h2 = 0)
   double* dB = nullptr;      // [n_local] QQ^T B
   uint8_t* wm = nullptr;     // [n_local] multiplicity | 0x80 Dirichlet
@@ -133,18 +140,36 @@ struct sem_mesh {
   double* cG64 = nullptr;
   float* cG32 = nullptr;
   float* cG32lo = nullptr;
+  int4* cGfx = nullptr;
+  int* cfx_sG = nullptr;
   double* cdK = nullptr;
   double* cB64 = nullptr;
   float* cB32 = nullptr;
   float* cB32lo = nullptr;
   double* cdB = nullptr;
+  int* cfx_eB = nullptr;
   uint64_t coef_gen = 0;
+  size_t coef_bytes = 0;
 
   // the operator's arrays: the plain geometry, or its per-point copies
-  const double* opG64() const { return cG64 ? cG64 : G64; }
-  const float* opG32() const { return cG64 ? cG32 : G32; }
-  const float* opG32lo() const { return cG64 ? cG32lo : G32lo; }
-  const double* opdK() const { return cG64 ? cdK : dK; }
+  const double* opG64() const { return cG32 ? cG64 : G64; }
+  const float* opG32() const { return cG32 ? cG32 : G32; }
+  const float* opG32lo() const { return cG32 ? cG32lo : G32lo; }
+  const double* opdK() const { return cG32 ? cdK : dK; }
+  // the fixed-point operator's data; G null where a point's coefficient takes it out of range
+  sem::FxOp opfx() const {
+    sem::FxOp f;
+    const int4* g = cG32 ? cGfx : Gfx;
+    const int* b = cB64 ? cfx_eB : fx_eB;
+    f.G = b ? g : nullptr;
+    f.sG = cG32 ? cfx_sG : fx_sG;
+    f.eB = b;
+    f.tab = fx_tab;
+    f.ti = fx_ti;
+    f.sc[0] = fx_sc[0];
+    f.sc[1] = fx_sc[1];
+    return f;
+  }
   const double* opB64() const { return cB64 ? cB64 : B64; }
   const float* opB32() const { return cB64 ? cB32 : B32; }
   const float* opB32lo() const { return cB64 ? cB32lo : B32lo; }
@@ -156,7 +181,7 @@ struct sem_mesh {
   int ax_var[3] = {0, 0, 0};
   int ax_var_dff = 0;           // double-float variant of the fused form (the FP64 CG's operator)
   int fp64_df = 0;
-  float ax_ms[3][4] = {{0}};
+  float ax_ms[3][sem::kAxVariants] = {{0}};
 
   // P_N - P_{N-2} pressure operators (pressure_api.cpp), built on first use
   // under p_mutex: GL-point factors F [E][9][m^3] (rho^3 adj(J)_{ba}, index

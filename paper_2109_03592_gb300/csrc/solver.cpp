@@ -23,6 +23,7 @@
 #include <cstring>
 #include <functional>
 
+#include "fixed.cuh"
 #include "kernels.h"
 #include "sem_internal.h"
 #include "solver.h"
@@ -94,6 +95,21 @@ sem_status alloc_ws(sem_mesh* m, Workspace** out) {
 
 // ---- local operator dispatch ---------------------------------------------------
 
+AxParams<double> ax64_params(const sem_mesh* m, const double* u, double* w, double h1, double h2, const double* z,
+                             double* p, PcgState* st, double* part, double* pout) {
+  AxParams<double> a{u, w, m->opG64(), m->opB64(), m->D64, h1, h2, h2 != 0.0, m->E, z, p, st, part, m->dev_err,
+                     pout, m->opfx()};
+  const double top = std::ldexp(1.0, fx::kOpExp / 2), low = 1.0 / top;  // NaN is out of range too
+  for (double h : {std::fabs(h1), std::fabs(h2)})
+    if (h != 0.0 && !(h >= low && h <= top)) a.fx.direct = 1;
+  return a;
+}
+
+int ax64_variant(const sem_mesh* m) {
+  if (m->ax_var[0] < kAxFixed || m->opfx().G) return m->ax_var[0];
+  return m->ax_ms[0][1] < m->ax_ms[0][0] ? 1 : 0;
+}
+
 cudaError_t ax64(const sem_mesh* m, const double* u, double* w, double h1, double h2, bool fused,
                         const double* z, double* p, PcgState* st, double* part, cudaStream_t s, double* pout) {
   if (m->fp64_df) {
@@ -101,9 +117,7 @@ cudaError_t ax64(const sem_mesh* m, const double* u, double* w, double h1, doubl
                  h2 != 0.0, m->E, z, p, st, part, m->eo64, m->eodf, pout};
     return launch_ax_df(m->N, fused ? m->ax_var_dff : m->ax_var[2], fused, a, s, nullptr);
   }
-  AxParams<double> a{u, w, m->opG64(), m->opB64(), m->D64, h1, h2, h2 != 0.0, m->E, z, p, st, part, m->dev_err,
-                     pout};
-  return launch_ax_f64(m->N, m->ax_var[0], fused, a, s, nullptr);
+  return launch_ax_f64(m->N, ax64_variant(m), fused, ax64_params(m, u, w, h1, h2, z, p, st, part, pout), s, nullptr);
 }
 
 // The native FP64 operator.  The residuals b - A x that decide convergence
@@ -113,9 +127,8 @@ cudaError_t ax64(const sem_mesh* m, const double* u, double* w, double h1, doubl
 // than FP64's, would set the attainable residual (measured: the E = 262,144
 // pipe stalled above 1e-10 with a 2^-46 input split).
 cudaError_t ax64_exact(const sem_mesh* m, const double* u, double* w, double h1, double h2, cudaStream_t s) {
-  AxParams<double> a{u, w, m->opG64(), m->opB64(), m->D64, h1, h2, h2 != 0.0, m->E, nullptr, nullptr, nullptr, nullptr,
-                     m->dev_err};
-  return launch_ax_f64(m->N, m->ax_var[0], false, a, s, nullptr);
+  return launch_ax_f64(m->N, ax64_variant(m), false, ax64_params(m, u, w, h1, h2, nullptr, nullptr, nullptr, nullptr),
+                       s, nullptr);
 }
 
 cudaError_t ax32(const sem_mesh* m, const float* u, float* w, double h1, double h2, bool fused, const float* z,
@@ -162,14 +175,39 @@ struct TuneVal {
   int var[3];
   int var_dff;
   int df;
-  float ms[3][4];
+  float ms[3][kAxVariants];
 };
 std::mutex g_tune_mutex;
 std::vector<std::pair<TuneKey, TuneVal>> g_tune;
 }  // namespace
 
+// The low parts of G and B that the double-float kernels read (28 B per local
+// point).  They are not part of a new mesh: the fixed-point kernels serve FP64
+// where they are faster, and then nothing reads them.  false: no memory.
+static bool ensure_lo(sem_mesh* m, cudaStream_t s) {
+  if (m->G32lo) return true;
+  const size_t P = (size_t)m->n_local;
+  if (!m->G64 || cudaMalloc((void**)&m->G32lo, 6 * P * sizeof(float)) != cudaSuccess) {
+    m->G32lo = nullptr;
+    cudaGetLastError();
+    return false;
+  }
+  if (cudaMalloc((void**)&m->B32lo, P * sizeof(float)) != cudaSuccess) {
+    cudaGetLastError();
+    cudaFree(m->G32lo);
+    m->G32lo = m->B32lo = nullptr;
+    return false;
+  }
+  m->dev_bytes += 7 * P * sizeof(float);
+  launch_split_f64(m->G64, m->G32, m->G32lo, 6 * P, s);
+  launch_split_f64(m->B64, m->B32, m->B32lo, P, s);
+  count_launches(2);
+  return true;
+}
+
 static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
   const size_t n = (size_t)m->n_local;
+  const bool df = ax_df_available(m->N) && ensure_lo(m, s);
   double* w = nullptr;
   SEM_CUDA(cudaMalloc((void**)&w, n * sizeof(double)));
   cudaEvent_t a, b;
@@ -179,15 +217,14 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
   sem_status status = SEM_OK;
   const int reps = m->E >= 65536 ? 2 : 3;
   for (int kind = 0; kind < 3 && status == SEM_OK; ++kind) {
-    if (kind == 2 && !ax_df_available(m->N)) continue;
+    if (kind == 2 && !df) continue;
     for (int v = 0; v < ax_num_variants(); ++v) {
       cudaError_t err = cudaSuccess;
       float total = 0.f;
       for (int rep = 0; rep <= reps && err == cudaSuccess; ++rep) {
         cudaEventRecord(a, s);
         if (kind == 0) {
-          AxParams<double> pa{m->B64, w, m->G64, m->B64, m->D64, 1.0, 0.0, 0, m->E, nullptr, nullptr, nullptr, nullptr,
-                              m->dev_err};
+          const AxParams<double> pa = ax64_params(m, m->B64, w, 1.0, 0.0, nullptr, nullptr, nullptr, nullptr);
           err = launch_ax_f64(m->N, v, false, pa, s, nullptr);
         } else if (kind == 1) {
           AxParams<float> pa{m->B32, (float*)w, m->G32, m->B32, m->D32, 1.f, 0.f, 0, m->E,
@@ -218,13 +255,14 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
       }
     }
   }
-  m->fp64_df = ax_df_available(m->N) && best[2] < best[0];
+  // the native operator is the more accurate one, so the double-float one has to be clearly faster
+  m->fp64_df = df && best[2] < 0.9f * best[0];
   m->ax_var_dff = m->ax_var[2];
   // The fused double-float form (p = z + beta p, A_L p, <p, A_L p>: the FP64
   // CG's operator) is timed on its own: its fastest variant need not be the
   // plain form's.  z is the mass, beta 0, and the state is cleared before
   // every run, so each run does the same work.
-  if (status == SEM_OK && ax_df_available(m->N)) {
+  if (status == SEM_OK && df) {
     double* p = nullptr;
     double* part = nullptr;
     PcgState* st = nullptr;
@@ -275,7 +313,8 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
 // Times every elements-per-block variant of the FP64, FP32 and double-float
 // local operator on this mesh (the mesh's own factors as input) and keeps
 // the fastest; FP64 requests use the double-float kernel when it is faster.
-// SEM_FP64_KERNEL=native|df forces the FP64 choice, SEM_FP32_VARIANT=v an
+// SEM_FP64_KERNEL=native|df forces the FP64 choice, SEM_FP64_VARIANT=v a variant
+// of the native operator (0, 1: FP64 pipe; 4, 5: fixed point), SEM_FP32_VARIANT=v an
 // FP32 variant and SEM_FP64_DF_VARIANT=v a double-float variant (which then
 // serves FP64 requests) that exists for this order.
 sem_status autotune_mesh(sem_mesh* m, cudaStream_t s) {
@@ -309,6 +348,13 @@ forced:
     if (!std::strcmp(f, "native")) m->fp64_df = 0;
     if (!std::strcmp(f, "df") && ax_df_available(m->N)) m->fp64_df = 1;
   }
+  if (const char* f = std::getenv("SEM_FP64_VARIANT")) {  // of the native operator; 4 and 5 are fixed point
+    const int v = std::atoi(f);
+    if (v >= 0 && v < ax_num_variants() && m->ax_ms[0][v] > 0.f && (v < kAxFixed || m->Gfx)) {
+      m->ax_var[0] = v;
+      m->fp64_df = 0;
+    }
+  }
   if (const char* f = std::getenv("SEM_FP32_VARIANT")) {
     const int v = std::atoi(f);
     if (v >= 0 && v < ax_num_variants() && m->ax_ms[1][v] > 0.f) m->ax_var[1] = v;
@@ -320,6 +366,10 @@ forced:
       m->ax_var_dff = v;
       m->fp64_df = 1;
     }
+  }
+  if (m->fp64_df && !ensure_lo(m, s)) {
+    set_error("out of memory for the double-float factors");
+    return SEM_ERR_OOM;
   }
   return SEM_OK;
 }

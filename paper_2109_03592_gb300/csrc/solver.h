@@ -38,6 +38,11 @@ cudaError_t ax64_exact(const sem_mesh* m, const double* u, double* w, double h1,
 // pout, when given, receives the new direction z + beta p instead of p).
 cudaError_t ax32(const sem_mesh* m, const float* u, float* w, double h1, double h2, bool fused, const float* z,
                  float* p, PcgState* st, double* part, cudaStream_t s, float* pout = nullptr);
+// The native FP64 operator's parameters and its variant on this mesh (an FP64-pipe
+// kernel where the fixed-point form does not cover the operator).
+AxParams<double> ax64_params(const sem_mesh* m, const double* u, double* w, double h1, double h2, const double* z,
+                             double* p, PcgState* st, double* part, double* pout = nullptr);
+int ax64_variant(const sem_mesh* m);
 cudaError_t ax64(const sem_mesh* m, const double* u, double* w, double h1, double h2, bool fused, const double* z,
                  double* p, PcgState* st, double* part, cudaStream_t s, double* pout = nullptr);
 // Write a fresh PcgState (tol, maxit, done) to ws->st / read it back (both synchronise ws->s).
