@@ -89,9 +89,10 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->pdinv);
   dev_free(m->Igl);
   dev_free(m->DIgl);
+  dev_free(m->Ffx);
+  dev_free(m->Ffx_s);
+  dev_free(m->invB);
   dev_free(m->Fgl32);
-  dev_free(m->Igl32);
-  dev_free(m->DIgl32);
   dev_free(m->invB32);
 }
 

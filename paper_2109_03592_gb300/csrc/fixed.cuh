@@ -40,7 +40,13 @@ __host__ __device__ __forceinline__ int2 split(ll v) {
 }
 
 #ifdef __CUDACC__
-__device__ __forceinline__ ll mad(ll acc, int a, int b) { return acc + (ll)a * b; }
+// acc + a b.  As PTX: from the plain expression the compiler made two multiplies and a sign extension where an
+// operand comes from constant memory (twice the instructions in the pressure kernels).
+__device__ __forceinline__ ll mad(ll acc, int a, int b) {
+  ll r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(acc));
+  return r;
+}
 
 // sum of c_l v_l / 2^64, rounded; the caller bounds sum |ch| + sum |vh| < 2^32 - 2^8
 template <int n>

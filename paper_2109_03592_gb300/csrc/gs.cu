@@ -127,6 +127,66 @@ __global__ void __launch_bounds__(kGsThreads / 2) k_gs(T* __restrict__ v, const 
   }
 }
 
+// Three vectors with the same numbering (a velocity's components, `stride`
+// apart): one node per thread, its tuple read once, the three components' copies
+// loaded together.  Bound like k_gs by the 32-byte sectors that L2 moves for
+// single values; whole pressure operator with it / with three launches of k_gs:
+// N = 7, E = 32,768: FP64 1365 / 1381 us, FP32 351 / 370; E = 4096: 201 / 219, 62 / 73.
+template <typename T, int M>
+__device__ __forceinline__ void gs_tuple_x3(T* __restrict__ v, int64_t stride, const int32_t* __restrict__ id,
+                                            int apply_mask) {
+  int32_t x[M];
+  load_tuple<M>(id, x);
+  const bool live = !(apply_mask && x[0] < 0);
+  x[0] &= 0x7fffffff;
+  T val[3][M];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int c = 0; c < M; ++c) val[a][c] = live ? v[a * stride + x[c]] : T(0);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    T s = val[a][0];
+#pragma unroll
+    for (int c = 1; c < M; ++c) s = add_rn(s, val[a][c]);
+#pragma unroll
+    for (int c = 0; c < M; ++c) v[a * stride + x[c]] = live ? s : T(0);
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kGsThreads) k_gs3(T* __restrict__ v, int64_t stride, const GsDev g, int apply_mask) {
+  const int4 w = g.units[blockIdx.x];
+  const int c = w.x;
+  if ((int)threadIdx.x >= w.z) return;
+  const int64_t t = (int64_t)w.y + threadIdx.x;  // node within class c
+  const int32_t* base = g.idx + g.off[c];
+  switch (c) {
+    case 0: gs_tuple_x3<T, 2>(v, stride, base + t * 2, apply_mask); break;
+    case 1: gs_tuple_x3<T, 3>(v, stride, base + t * 3, apply_mask); break;
+    case 2: gs_tuple_x3<T, 4>(v, stride, base + t * 4, apply_mask); break;
+    case 3: gs_tuple_x3<T, 5>(v, stride, base + t * 5, apply_mask); break;
+    case 4: gs_tuple_x3<T, 6>(v, stride, base + t * 6, apply_mask); break;
+    case 5: gs_tuple_x3<T, 7>(v, stride, base + t * 7, apply_mask); break;
+    case 6: gs_tuple_x3<T, 8>(v, stride, base + t * 8, apply_mask); break;
+    default:
+      for (int a = 0; a < 3; ++a) {
+        T* va = v + a * stride;
+        if (c == 7) {
+          const int32_t b0 = g.gptr[t], e0 = g.gptr[t + 1];
+          const bool live = !(apply_mask && base[b0] < 0);
+          T acc = va[base[b0] & 0x7fffffff];
+          for (int32_t q = b0 + 1; q < e0; ++q) acc = add_rn(acc, va[base[q]]);
+          if (!live) acc = T(0);
+          va[base[b0] & 0x7fffffff] = acc;
+          for (int32_t q = b0 + 1; q < e0; ++q) va[base[q]] = acc;
+        } else if (apply_mask) {
+          va[base[t] & 0x7fffffff] = T(0);
+        }
+      }
+  }
+}
+
 template <typename T>
 cudaError_t launch_gs(T* v, const GsDev& g, int apply_mask, const PcgState* st, cudaStream_t s) {
   if (g.nunits == 0) return cudaSuccess;
@@ -134,6 +194,15 @@ cudaError_t launch_gs(T* v, const GsDev& g, int apply_mask, const PcgState* st, 
   return cudaGetLastError();
 }
 
+template <typename T>
+cudaError_t launch_gs3(T* v, int64_t stride, const GsDev& g, int apply_mask, cudaStream_t s) {
+  if (g.nunits == 0) return cudaSuccess;
+  k_gs3<T><<<(unsigned)g.nunits, kGsThreads, 0, s>>>(v, stride, g, apply_mask);
+  return cudaGetLastError();
+}
+
+template cudaError_t launch_gs3<double>(double*, int64_t, const GsDev&, int, cudaStream_t);
+template cudaError_t launch_gs3<float>(float*, int64_t, const GsDev&, int, cudaStream_t);
 template cudaError_t launch_gs<double>(double*, const GsDev&, int, const PcgState*, cudaStream_t);
 template cudaError_t launch_gs<float>(float*, const GsDev&, int, const PcgState*, cudaStream_t);
 

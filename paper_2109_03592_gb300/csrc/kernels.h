@@ -112,6 +112,9 @@ struct GsDev {
 };
 template <typename T>
 cudaError_t launch_gs(T* v, const GsDev& g, int apply_mask, const PcgState* st, cudaStream_t s);
+// the same for three vectors, `stride` values apart (the velocity components of the pressure operator)
+template <typename T>
+cudaError_t launch_gs3(T* v, int64_t stride, const GsDev& g, int apply_mask, cudaStream_t s);
 
 // ---- PCG vector kernels (pcg.cu) ----
 template <typename T>
@@ -172,14 +175,25 @@ cudaError_t launch_pap_finish(const double* partial, int count, PcgState* st, cu
 size_t gl_factors_smem(int n, int m);
 cudaError_t launch_gl_factors(const double* xyz, const double* Ig, const double* DIg, const double* rho, int n, int m,
                               int64_t E, double* F, int* bad, cudaStream_t s);
-// T = double, or float for the FP32 operator (factors and basis rounded from FP64)
+// What the weak gradient and divergence read (pressure_eo.cuh).  FP64: the factors in fixed point (Ffx, sF; direct: out
+// of its range) and the plain data for the elements that are evaluated in FP64; FP32: F32, in the same order.
+struct PressureOp {
+  const double *F, *Ig, *DIg, *invB;
+  const int2* Ffx;
+  const int* sF;
+  int direct;
+  const float *F32, *invB32;
+};
+cudaError_t launch_pressure_pack(const double* F, int N, int64_t E, int2* Ffx, int* sF, int* bad, cudaStream_t s);
+cudaError_t launch_pressure_pack32(const double* F, int N, int64_t E, float* F32, cudaStream_t s);
+void launch_recip(const double* a, double* out, int64_t n, cudaStream_t s);
+// T = double or float
 template <typename T>
-cudaError_t launch_pgrad(const T* p, const T* F, const T* Ig, const T* DIg, int n, int m, int64_t E, T* u,
-                         int64_t n_local, cudaStream_t s);
-// v_a = u_a / dB (dB given), u_a invB (invB given), or u_a
+cudaError_t launch_pgrad(int N, const PressureOp& op, const T* p, int64_t E, T* u, int64_t n_local, cudaStream_t s);
+// v_a = u_a / (QQ^T B) (scaled), or u_a
 template <typename T>
-cudaError_t launch_pdiv(const T* u, const T* dB, const T* invB, const T* F, const T* Ig, const T* DIg, int n, int m,
-                        int64_t E, T* out, int64_t n_local, cudaStream_t s);
+cudaError_t launch_pdiv(int N, const PressureOp& op, const T* u, bool scaled, int64_t E, T* out, int64_t n_local,
+                        cudaStream_t s);
 void launch_to_f32(const double* a, float* b, int64_t n, cudaStream_t s);
 void launch_to_f64(const float* a, double* b, int64_t n, cudaStream_t s);
 void launch_recip_f32(const double* a, float* b, int64_t n, cudaStream_t s);

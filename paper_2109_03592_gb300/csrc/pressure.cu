@@ -11,11 +11,10 @@
 //     (DIg along b, Ig elsewhere);
 //   * weak gradient    u_a = sum_b C_b^T (F[b][a] p), the transpose of D.
 // The factors and the diagonal run one CTA per element in FP64; the weak
-// gradient and divergence (pressure_line.cuh) apply each C_b as 1D
+// gradient and divergence (pressure_eo.cuh) apply each C_b as 1D
 // contractions of whole lines held in registers, several elements per CTA,
-// in FP64 or FP32.
+// in FP32 or in fixed point.
 #include "kernels.h"
-#include "pressure_line.cuh"
 
 namespace sem {
 
@@ -92,8 +91,7 @@ __global__ void k_gl_factors(const double* __restrict__ xyz, const double* __res
   }
 }
 
-// The weak gradient and divergence (k_pgrad_line, k_pdiv_line) are in
-// pressure_line.cuh.
+// The weak gradient and divergence (k_pgrad, k_pdiv) are in pressure_eo.cuh.
 
 // ---- vector kernels of the pressure CG (pressure values, Euclidean products) ----
 // Reductions are deterministic: block b sums its grid-stride slice in a fixed
@@ -338,6 +336,10 @@ __global__ void k_to_f64(const float* __restrict__ a, double* __restrict__ b, in
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     b[i] = (double)a[i];
 }
+__global__ void k_recip(const double* __restrict__ a, double* __restrict__ b, int64_t n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    b[i] = 1.0 / a[i];
+}
 __global__ void k_recip_f32(const double* __restrict__ a, float* __restrict__ b, int64_t n) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     b[i] = (float)(1.0 / a[i]);
@@ -452,74 +454,9 @@ cudaError_t launch_gl_factors(const double* xyz, const double* Ig, const double*
   return cudaGetLastError();
 }
 
-template <typename T, int N>
-cudaError_t launch_pgrad_n(const T* p, const T* F, const T* Ig, const T* DIg, int64_t E, T* u, int64_t n_local,
-                           cudaStream_t s) {
-  using S = pline::Shape<T, N>;
-  static DeviceOnce once;
-  cudaError_t err = once.get([&](int, int*) {
-    return cudaFuncSetAttribute(pline::k_pgrad_line<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
-  });
-  if (err != cudaSuccess) return err;
-  if (E == 0) return cudaSuccess;
-  pline::k_pgrad_line<T, N><<<(unsigned)((E + S::EPB - 1) / S::EPB), pline::kThreads, S::smem, s>>>(p, F, Ig, DIg, E,
-                                                                                                  u, n_local);
-  return cudaGetLastError();
+void launch_recip(const double* a, double* out, int64_t n, cudaStream_t s) {
+  k_recip<<<kPressureRedBlocks, kRedThreads, 0, s>>>(a, out, n);
 }
-
-template <typename T, int N>
-cudaError_t launch_pdiv_n(const T* u, const T* dB, const T* invB, const T* F, const T* Ig, const T* DIg, int64_t E,
-                          T* out, int64_t n_local, cudaStream_t s) {
-  using S = pline::Shape<T, N>;
-  static DeviceOnce once;
-  cudaError_t err = once.get([&](int, int*) {
-    return cudaFuncSetAttribute(pline::k_pdiv_line<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem);
-  });
-  if (err != cudaSuccess) return err;
-  if (E == 0) return cudaSuccess;
-  pline::k_pdiv_line<T, N><<<(unsigned)((E + S::EPB - 1) / S::EPB), pline::kThreads, S::smem, s>>>(
-      u, dB, invB, F, Ig, DIg, E, out, n_local);
-  return cudaGetLastError();
-}
-
-#define SEM_PRESSURE_ORDERS(X) X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11)
-
-template <typename T>
-cudaError_t launch_pgrad(const T* p, const T* F, const T* Ig, const T* DIg, int n, int m, int64_t E, T* u,
-                         int64_t n_local, cudaStream_t s) {
-  if (m != n - 2) return cudaErrorInvalidValue;
-  switch (n - 1) {
-#define SEM_CASE(N) \
-  case N:           \
-    return launch_pgrad_n<T, N>(p, F, Ig, DIg, E, u, n_local, s);
-    SEM_PRESSURE_ORDERS(SEM_CASE)
-#undef SEM_CASE
-    default: return cudaErrorNotSupported;
-  }
-}
-template cudaError_t launch_pgrad<double>(const double*, const double*, const double*, const double*, int, int, int64_t,
-                                          double*, int64_t, cudaStream_t);
-template cudaError_t launch_pgrad<float>(const float*, const float*, const float*, const float*, int, int, int64_t,
-                                         float*, int64_t, cudaStream_t);
-
-template <typename T>
-cudaError_t launch_pdiv(const T* u, const T* dB, const T* invB, const T* F, const T* Ig, const T* DIg, int n, int m,
-                        int64_t E, T* out, int64_t n_local, cudaStream_t s) {
-  if (m != n - 2) return cudaErrorInvalidValue;
-  switch (n - 1) {
-#define SEM_CASE(N) \
-  case N:           \
-    return launch_pdiv_n<T, N>(u, dB, invB, F, Ig, DIg, E, out, n_local, s);
-    SEM_PRESSURE_ORDERS(SEM_CASE)
-#undef SEM_CASE
-    default: return cudaErrorNotSupported;
-  }
-}
-template cudaError_t launch_pdiv<double>(const double*, const double*, const double*, const double*, const double*,
-                                         const double*, int, int, int64_t, double*, int64_t, cudaStream_t);
-template cudaError_t launch_pdiv<float>(const float*, const float*, const float*, const float*, const float*,
-                                        const float*, int, int, int64_t, float*, int64_t, cudaStream_t);
-
 void launch_to_f32(const double* a, float* b, int64_t n, cudaStream_t s) {
   k_to_f32<<<kPressureRedBlocks, kRedThreads, 0, s>>>(a, b, n);
 }

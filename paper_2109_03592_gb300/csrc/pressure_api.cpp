@@ -17,6 +17,67 @@
 #include "sem_internal.h"
 
 namespace sem {
+
+// The same quantities as gl_matrices below in long double: the GLL and GL points by Newton (from the FP64 GLL
+// points and from cos(pi (i + 3/4) / (m + 1/2))), made symmetric, and the basis by its products.
+void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double>& DIg) {
+  typedef long double ld;
+  const int n = N + 1, m = N - 1;
+  auto legendre = [](int k, ld x, ld& pk, ld& pk1) {  // P_k and P_{k-1}, k >= 1
+    pk1 = 1;
+    pk = x;
+    for (int j = 1; j < k; ++j) {
+      const ld p = ((2 * j + 1) * x * pk - j * pk1) / (j + 1);
+      pk1 = pk;
+      pk = p;
+    }
+  };
+  std::vector<double> xd, wd, Dd;
+  gll(N, xd, wd, Dd);
+  std::vector<ld> x(xd.begin(), xd.end()), z(m);
+  ld p, q;
+  for (int i = 1; i < N; ++i)  // roots of P_{N-1} - x P_N, whose derivative is -(N + 1) P_N
+    for (int it = 0; it < 4; ++it) {
+      legendre(N, x[i], p, q);
+      x[i] += (q - x[i] * p) / ((N + 1) * p);
+    }
+  for (int i = 0; i < m; ++i) {
+    z[i] = -std::cos(M_PI * (i + 0.75) / (m + 0.5));
+    for (int it = 0; it < 8; ++it) {  // P_m' = m (P_{m-1} - x P_m) / (1 - x^2)
+      legendre(m, z[i], p, q);
+      z[i] -= p * (1 - z[i] * z[i]) / (m * (q - z[i] * p));
+    }
+  }
+  auto symmetric = [](std::vector<ld>& v) {
+    const int k = (int)v.size();
+    for (int i = 0; i < k - 1 - i; ++i) {
+      const ld a = (v[k - 1 - i] - v[i]) / 2;
+      v[i] = -a;
+      v[k - 1 - i] = a;
+    }
+    if (k & 1) v[k / 2] = 0;
+  };
+  symmetric(x);
+  symmetric(z);
+  Ig.assign((size_t)m * n, 0);
+  DIg.assign((size_t)m * n, 0);
+  for (int i = 0; i < m; ++i)
+    for (int l = 0; l < n; ++l) {
+      ld v = 1, d = 0;
+      for (int k = 0; k < n; ++k)
+        if (k != l) v *= (z[i] - x[k]) / (x[l] - x[k]);
+      for (int r = 0; r < n; ++r) {
+        if (r == l) continue;
+        ld w = 1 / (x[l] - x[r]);
+        for (int k = 0; k < n; ++k)
+          if (k != l && k != r) w *= (z[i] - x[k]) / (x[l] - x[k]);
+        d += w;
+      }
+      Ig[i * n + l] = v;
+      DIg[i * n + l] = d;
+    }
+}
+
 namespace {
 
 // Legendre P_m(x) and P_{m-1}(x) by the three-term recurrence.
@@ -105,6 +166,10 @@ void gl_matrices(int N, std::vector<double>& Ig, std::vector<double>& DIg, std::
     }
 }
 
+PressureOp pressure_op(const sem_mesh* m) {
+  return {m->Fgl, m->Igl, m->DIgl, m->invB, m->Ffx, m->Ffx_s, m->Ffx_direct, m->Fgl32, m->invB32};
+}
+
 #define SEM_TRY_STATUS(expr)          \
   do {                                \
     sem_status _s = (expr);           \
@@ -132,13 +197,17 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   const int64_t m3 = (int64_t)mm * mm * mm;
   std::vector<double> Ig, DIg, rho;
   gl_matrices(N, Ig, DIg, rho);
-  double *F = nullptr, *I_d = nullptr, *DI_d = nullptr, *rho_d = nullptr;
-  int* bad_d = nullptr;
+  double *F = nullptr, *I_d = nullptr, *DI_d = nullptr, *rho_d = nullptr, *iB = nullptr;
+  int2* Ffx = nullptr;
+  int *sF = nullptr, *bad_d = nullptr;  // bad: det(J) <= 0; factors out of the fixed-point form's range
   auto release = [&]() {
     if (F) cudaFree(F);
     if (I_d) cudaFree(I_d);
     if (DI_d) cudaFree(DI_d);
     if (rho_d) cudaFree(rho_d);
+    if (iB) cudaFree(iB);
+    if (Ffx) cudaFree(Ffx);
+    if (sF) cudaFree(sF);
     if (bad_d) cudaFree(bad_d);
   };
   auto fail = [&](cudaError_t e, const char* what) {
@@ -151,32 +220,41 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   if ((e = cudaMalloc((void**)&I_d, sizeof(double) * mm * n)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&DI_d, sizeof(double) * mm * n)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&rho_d, sizeof(double) * mm)) != cudaSuccess) return fail(e, "cudaMalloc");
-  if ((e = cudaMalloc((void**)&bad_d, sizeof(int))) != cudaSuccess) return fail(e, "cudaMalloc");
+  if ((e = cudaMalloc((void**)&bad_d, 2 * sizeof(int))) != cudaSuccess) return fail(e, "cudaMalloc");
+  if ((e = cudaMalloc((void**)&Ffx, sizeof(int2) * 9 * m3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
+  if ((e = cudaMalloc((void**)&sF, sizeof(int) * 3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
+  if ((e = cudaMalloc((void**)&iB, sizeof(double) * m->n_local)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMemcpyAsync(I_d, Ig.data(), sizeof(double) * mm * n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
   if ((e = cudaMemcpyAsync(DI_d, DIg.data(), sizeof(double) * mm * n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
   if ((e = cudaMemcpyAsync(rho_d, rho.data(), sizeof(double) * mm, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
-  if ((e = cudaMemsetAsync(bad_d, 0, sizeof(int), s)) != cudaSuccess) return fail(e, "cudaMemsetAsync");
+  if ((e = cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s)) != cudaSuccess) return fail(e, "cudaMemsetAsync");
   if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
     return fail(e, "k_gl_factors");
-  count_launches(1);
-  int bad = 0;
-  if ((e = cudaMemcpyAsync(&bad, bad_d, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+  if ((e = launch_pressure_pack(F, N, m->E, Ffx, sF, bad_d + 1, s)) != cudaSuccess) return fail(e, "k_pack_fx");
+  launch_recip(m->dB, iB, m->n_local, s);
+  count_launches(3);
+  int bad[2] = {0, 0};
+  if ((e = cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "cudaStreamSynchronize");
   cudaFree(rho_d);
   rho_d = nullptr;
   cudaFree(bad_d);
   bad_d = nullptr;
-  if (bad) {
+  if (bad[0]) {
     release();
     set_error("mesh has an element with det(J) <= 0 at a GL point");
     return SEM_ERR_BAD_MESH;
   }
   sem_mesh* mut = const_cast<sem_mesh*>(m);
-  mut->dev_bytes += sizeof(double) * (9 * m3 * m->E + 2 * mm * n);
+  mut->dev_bytes += sizeof(double) * (18 * m3 * m->E + 2 * mm * n + m->n_local) + sizeof(int) * 3 * m->E;
+  m->Ffx = Ffx;
+  m->Ffx_s = sF;
+  m->Ffx_direct = bad[1];
+  m->invB = iB;
   m->Igl = I_d;
   m->DIgl = DI_d;
   m->Fgl = F;
@@ -190,11 +268,11 @@ sem_status ensure_pressure32(const sem_mesh* m, cudaStream_t s) {
   SEM_TRY_STATUS(ensure_pressure(m, s));
   std::lock_guard<std::mutex> lk(m->p_mutex);
   if (m->Fgl32) return SEM_OK;
-  const int N = m->N, n = N + 1, mm = N - 1;
+  const int N = m->N, mm = N - 1;
   const int64_t nF = (int64_t)9 * mm * mm * mm * m->E;
-  float *F = nullptr, *I = nullptr, *DI = nullptr, *iB = nullptr;
+  float *F = nullptr, *iB = nullptr;
   auto release = [&]() {
-    for (float* q : {F, I, DI, iB})
+    for (float* q : {F, iB})
       if (q) cudaFree(q);
   };
   auto fail = [&](cudaError_t e, const char* what) {
@@ -204,19 +282,13 @@ sem_status ensure_pressure32(const sem_mesh* m, cudaStream_t s) {
   };
   cudaError_t e;
   if ((e = cudaMalloc((void**)&F, sizeof(float) * nF)) != cudaSuccess) return fail(e, "cudaMalloc");
-  if ((e = cudaMalloc((void**)&I, sizeof(float) * mm * n)) != cudaSuccess) return fail(e, "cudaMalloc");
-  if ((e = cudaMalloc((void**)&DI, sizeof(float) * mm * n)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&iB, sizeof(float) * m->n_local)) != cudaSuccess) return fail(e, "cudaMalloc");
-  launch_to_f32(m->Fgl, F, nF, s);
-  launch_to_f32(m->Igl, I, (int64_t)mm * n, s);
-  launch_to_f32(m->DIgl, DI, (int64_t)mm * n, s);
+  if ((e = launch_pressure_pack32(m->Fgl, N, m->E, F, s)) != cudaSuccess) return fail(e, "k_pack_f32");
   launch_recip_f32(m->dB, iB, m->n_local, s);
-  count_launches(4);
+  count_launches(2);
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "pressure FP32 copies");
   sem_mesh* mut = const_cast<sem_mesh*>(m);
-  mut->dev_bytes += sizeof(float) * (nF + 2 * mm * n + m->n_local);
-  m->Igl32 = I;
-  m->DIgl32 = DI;
+  mut->dev_bytes += sizeof(float) * (nF + m->n_local);
   m->invB32 = iB;
   m->Fgl32 = F;
   return SEM_OK;
@@ -248,13 +320,11 @@ sem_status ensure_pdiag(const sem_mesh* m, cudaStream_t s) {
 
 // q = E p in FP32: weak gradient, masked QQ^T of each component, reciprocal mass, weak divergence.
 sem_status apply_E32(const sem_mesh* m, const float* p, float* q, float* work, cudaStream_t s) {
-  const int mm = m->N - 1;
-  const GsDev g = gs_dev(m);
-  SEM_CUDA(launch_pgrad<float>(p, m->Fgl32, m->Igl32, m->DIgl32, m->n, mm, m->E, work, m->n_local, s));
-  for (int a = 0; a < 3; ++a) SEM_CUDA(launch_gs<float>(work + a * m->n_local, g, 1, nullptr, s));
-  SEM_CUDA(launch_pdiv<float>(work, nullptr, m->invB32, m->Fgl32, m->Igl32, m->DIgl32, m->n, mm, m->E, q, m->n_local,
-                              s));
-  count_launches(5);
+  const PressureOp op = pressure_op(m);
+  SEM_CUDA(launch_pgrad<float>(m->N, op, p, m->E, work, m->n_local, s));
+  SEM_CUDA(launch_gs3<float>(work, m->n_local, gs_dev(m), 1, s));
+  SEM_CUDA(launch_pdiv<float>(m->N, op, work, true, m->E, q, m->n_local, s));
+  count_launches(3);
   return SEM_OK;
 }
 
@@ -345,6 +415,7 @@ sem_status pressure_cg(const sem_mesh* m, const double* g_dev, double* p_dev, do
   float* w32 = mixed ? q32 + np : nullptr;
   float* work32 = mixed ? w32 + np : nullptr;
   const GsDev g = gs_dev(m);
+  const PressureOp op = pressure_op(m);
   auto read = [&](double& v) -> sem_status {
     SEM_CUDA(cudaMemcpyAsync(&v, sum_d, sizeof(double), cudaMemcpyDeviceToHost, s));
     SEM_CUDA(cudaStreamSynchronize(s));
@@ -363,10 +434,10 @@ sem_status pressure_cg(const sem_mesh* m, const double* g_dev, double* p_dev, do
   uint64_t launches = 0;
   // out = E v in FP64: weak gradient, QQ^T with mask on each component, inverse mass, weak divergence
   auto apply_E = [&](const double* v, double* out) -> sem_status {
-    SEM_CUDA(launch_pgrad<double>(v, m->Fgl, m->Igl, m->DIgl, m->n, (int)mm, m->E, work, nl, s));
-    for (int a = 0; a < 3; ++a) SEM_CUDA(launch_gs<double>(work + a * nl, g, 1, nullptr, s));
-    SEM_CUDA(launch_pdiv<double>(work, m->dB, nullptr, m->Fgl, m->Igl, m->DIgl, m->n, (int)mm, m->E, out, nl, s));
-    launches += 5;
+    SEM_CUDA(launch_pgrad<double>(m->N, op, v, m->E, work, nl, s));
+    SEM_CUDA(launch_gs3<double>(work, nl, g, 1, s));
+    SEM_CUDA(launch_pdiv<double>(m->N, op, work, true, m->E, out, nl, s));
+    launches += 3;
     return SEM_OK;
   };
   // z = Pm (dinv r) in place and <r, z>, host-synchronous (start and after replacements)
@@ -433,7 +504,7 @@ sem_status pressure_cg(const sem_mesh* m, const double* g_dev, double* p_dev, do
       SEM_CUDA(launch_pcg_pdir(q, zdir, np, st, s));
       return SEM_OK;
     };
-    const int per_iter = mixed ? 10 : 8;
+    const int per_iter = mixed ? 8 : 6;
     {
       cudaGraph_t graph = nullptr;
       SEM_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
@@ -567,7 +638,7 @@ sem_status sem_pressure_grad(const sem_mesh* m, const double* p_dev, double* u_d
   cudaStream_t s = (cudaStream_t)stream;
   st = ensure_pressure(m, s);
   if (st != SEM_OK) return st;
-  SEM_CUDA(launch_pgrad<double>(p_dev, m->Fgl, m->Igl, m->DIgl, m->n, m->N - 1, m->E, u_dev, m->n_local, s));
+  SEM_CUDA(launch_pgrad<double>(m->N, pressure_op(m), p_dev, m->E, u_dev, m->n_local, s));
   count_launches(1);
   return SEM_OK;
 }
@@ -582,7 +653,7 @@ sem_status sem_pressure_div(const sem_mesh* m, const double* u_dev, double* q_de
   cudaStream_t s = (cudaStream_t)stream;
   st = ensure_pressure(m, s);
   if (st != SEM_OK) return st;
-  SEM_CUDA(launch_pdiv<double>(u_dev, nullptr, nullptr, m->Fgl, m->Igl, m->DIgl, m->n, m->N - 1, m->E, q_dev, m->n_local, s));
+  SEM_CUDA(launch_pdiv<double>(m->N, pressure_op(m), u_dev, false, m->E, q_dev, m->n_local, s));
   count_launches(1);
   return SEM_OK;
 }
@@ -606,11 +677,11 @@ sem_status sem_pressure_apply(const sem_mesh* m, const double* p_dev, double* q_
   cudaStream_t s = (cudaStream_t)stream;
   st = ensure_pressure(m, s);
   if (st != SEM_OK) return st;
-  const GsDev g = gs_dev(m);
-  SEM_CUDA(launch_pgrad<double>(p_dev, m->Fgl, m->Igl, m->DIgl, m->n, m->N - 1, m->E, work_dev, m->n_local, s));
-  for (int a = 0; a < 3; ++a) SEM_CUDA(launch_gs<double>(work_dev + a * m->n_local, g, 1, nullptr, s));
-  SEM_CUDA(launch_pdiv<double>(work_dev, m->dB, nullptr, m->Fgl, m->Igl, m->DIgl, m->n, m->N - 1, m->E, q_dev, m->n_local, s));
-  count_launches(5);
+  const PressureOp op = pressure_op(m);
+  SEM_CUDA(launch_pgrad<double>(m->N, op, p_dev, m->E, work_dev, m->n_local, s));
+  SEM_CUDA(launch_gs3<double>(work_dev, m->n_local, gs_dev(m), 1, s));
+  SEM_CUDA(launch_pdiv<double>(m->N, op, work_dev, true, m->E, q_dev, m->n_local, s));
+  count_launches(3);
   return SEM_OK;
 }
 

@@ -55,6 +55,9 @@ struct Topology {
   int64_t n_global = 0;
   std::vector<int64_t> glo;  // [n_local] first-touch global ids
 };
+// Ig and DIg (pressure_api.cpp) [m][n] in long double, from long-double GLL and GL points.
+void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double>& DIg);
+
 sem_status build_numbering(int64_t E, int N, const int64_t* vert, Topology& t);
 
 // Gather-scatter plan.  Nodes with m > 1 copies, in ascending global id,
@@ -191,11 +194,13 @@ struct sem_mesh {
   mutable double* Fgl = nullptr;
   mutable double* Igl = nullptr;
   mutable double* DIgl = nullptr;
-  // their FP32 copies and the reciprocal assembled mass [n_local], for the
-  // FP32 operator of the mixed-precision pressure solve (built on first use)
+  mutable int2* Ffx = nullptr;      // F in fixed point and its exponents (PressureOp)
+  mutable int* Ffx_s = nullptr;
+  mutable int Ffx_direct = 0;
+  mutable double* invB = nullptr;   // [n_local] 1 / (QQ^T B)
+  // FP32 copies of F and invB, for the FP32 operator of the mixed-precision
+  // pressure solve (built on first use)
   mutable float* Fgl32 = nullptr;
-  mutable float* Igl32 = nullptr;
-  mutable float* DIgl32 = nullptr;
   mutable float* invB32 = nullptr;
 
   std::mutex ws_mutex;
