@@ -8,7 +8,7 @@
 #include <memory>
 #include <string>
 
-#include "fixed.cuh"
+#include "fx_tables.h"
 #include "kernels.h"
 #include "sem_internal.h"
 #include "solver.h"
@@ -59,7 +59,6 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->Gfx);
   dev_free(m->fx_sG);
   dev_free(m->fx_eB);
-  dev_free(m->fx_tab);
   dev_free(m->fx_ti);
   dev_free(m->wq);
   dev_free(m->dK);
@@ -183,7 +182,7 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     launch_split_f64(c.B64, c.B32, c.B32lo, P, s);
   }
   if (m->Gfx && (h1 || h2)) {
-    SEM_CUDA(launch_fx_pack(c.G64, c.B64, m->fx_ti, n, m->E, c.Gfx, c.fx_sG, c.fx_eB, bad_d + 1, s));
+    SEM_CUDA(launch_fx_pack(c.G64, c.B64, m->fx_ti, fx_scale(m->N).K, n, m->E, c.Gfx, c.fx_sG, c.fx_eB, bad_d + 1, s));
     count_launches(1);
   }
   SEM_CUDA(cudaGetLastError());
@@ -223,41 +222,6 @@ void drop_unused(sem_mesh* m) {
     dev_drop(m->B32lo, P, m->dev_bytes);
   }
   if (m->ax_var[0] >= kAxFixed && m->Gfx) dev_drop(m->G64, 6 * P, m->dev_bytes);
-}
-
-// D and D^T of the n GLL points as 64-bit integers (FxOp::tab), c 2^sc, split
-// for fixed.cuh.  Even n: for i, l < n/2 the pair (Ep, Em) = (D[i][l] +- D[i][n-1-l]) / 2;
-// odd n: the n x n entries.  sc makes the largest row sum at most 2^62, or 2^61 where six or
-// more terms meet: with inputs of 61 bits (even n) or 60 bits (odd n) that is the bound of fx::dot.
-void fx_tables(int n, const std::vector<double>& D, std::vector<int>& tab, int* sc) {
-  const bool even = n % 2 == 0;
-  const int h = even ? n / 2 : n;
-  tab.assign((size_t)2 * h * h * (even ? 4 : 2) + 2, 0);  // a multiple of 4 ints
-  tab.resize(tab.size() / 4 * 4);
-  for (int dir = 0; dir < 2; ++dir) {
-    auto at = [&](int i, int l) { return (long double)(dir == 0 ? D[i * n + l] : D[l * n + i]); };
-    auto coef = [&](int i, int l, int s) {
-      return even ? (s ? (at(i, l) - at(i, n - 1 - l)) / 2 : (at(i, l) + at(i, n - 1 - l)) / 2) : at(i, l);
-    };
-    long double top = 0;
-    for (int i = 0; i < h; ++i)
-      for (int s = 0; s < (even ? 2 : 1); ++s) {
-        long double sum = 0;
-        for (int l = 0; l < h; ++l) sum += std::fabs(coef(i, l, s));
-        top = std::max(top, sum);
-      }
-    int e = 0;
-    std::frexp(top, &e);  // top < 2^e
-    sc[dir] = (even ? (h >= 6 ? 61 : 62) : (h >= 10 ? 61 : 62)) - e;
-    size_t q = (size_t)dir * h * h * (even ? 4 : 2);
-    for (int i = 0; i < h; ++i)
-      for (int l = 0; l < h; ++l)
-        for (int s = 0; s < (even ? 2 : 1); ++s) {
-          const int2 v = fx::split(std::llround(std::ldexp(coef(i, l, s), sc[dir])));
-          tab[q++] = v.x;
-          tab[q++] = v.y;
-        }
-  }
 }
 
 sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
@@ -341,12 +305,9 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_TRY(dev_alloc(&m->eodf, eodf.size(), tb));
   }
 
-  // fixed-point tables of D and D^T, and the weights' exponents
-  std::vector<int> tab, ti(n);
-  fx_tables(n, D, tab, m->fx_sc);
+  std::vector<int> ti(n);  // the weights' exponents (FxOp)
   const double wmax = *std::max_element(w.begin(), w.end());
   for (int i = 0; i < n; ++i) ti[i] = (int)std::lround(-std::log2(w[i] / wmax));
-  SEM_TRY(dev_alloc(&m->fx_tab, tab.size() / 4, tb));
   SEM_TRY(dev_alloc(&m->fx_ti, n, tb));
   SEM_TRY(dev_alloc(&m->wq, n, tb));
 
@@ -368,7 +329,6 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
 
   SEM_CUDA(cudaMemcpyAsync(xi_d, xi.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->wq, w.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
-  SEM_CUDA(cudaMemcpyAsync(m->fx_tab, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->fx_ti, ti.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D64, D.data(), n * n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32, D32.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -407,7 +367,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_CUDA(launch_gs<double>(m->dB, gs_dev(m), 0, nullptr, s));
   launch_split_f64(m->G64, m->G32, nullptr, 6 * P, s);  // the low parts: autotune_mesh, where they are needed
   launch_split_f64(m->B64, m->B32, nullptr, P, s);
-  SEM_CUDA(launch_fx_pack(m->G64, m->B64, m->fx_ti, n, E, m->Gfx, m->fx_sG, m->fx_eB, bad_d + 1, s));
+  SEM_CUDA(launch_fx_pack(m->G64, m->B64, m->fx_ti, fx_scale(N).K, n, E, m->Gfx, m->fx_sG, m->fx_eB, bad_d + 1, s));
   SEM_CUDA(cudaGetLastError());
   count_launches(8);
   int bad[2] = {0, 0};

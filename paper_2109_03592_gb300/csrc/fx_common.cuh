@@ -1,5 +1,4 @@
-// Parts shared by the two fixed-point forms of the FP64 local operator
-// (ax_fx_impl.cuh, ax_fxd_impl.cuh).
+// Parts of the fixed-point FP64 operators (ax_fx_impl.cuh, pressure_eo.cuh).
 #pragma once
 
 #include "fixed.cuh"
@@ -50,11 +49,16 @@ struct ElemMax {
 // w at one point of an element in FP64, straight from memory (Alg. 1, with the factors taken back from their
 // fixed-point form): for the rare element that the integer path does not cover.
 template <int N>
-__device__ __forceinline__ double slow_point(const AxParams<double>& P, const double* v, int64_t e, int i, int j, int k) {
+__device__ __forceinline__ double slow_point(const AxParams<double>& P, double kappa, const double* v, int64_t e, int i,
+                                             int j, int k) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
   const double* ue = v + e * n3;
   const int sG = P.fx.sG[e];
-  auto G = [&](int f, int a, int b, int c) { return factor(P.fx.G, sG, P.fx.ti, n, e, f, a, b, c); };
+  auto G = [&](int f, int a, int b, int c) {
+    const int4 x = P.fx.G[(e * 3 + (f >> 1)) * n3 + a + n * b + n2 * c];
+    const int2 y = (f & 1) ? make_int2(x.z, x.w) : make_int2(x.x, x.y);
+    return ldexp(__ll2double_rn(shl(y.y, 32) + y.x) / kappa, -sG);
+  };
   double out = 0.0;
 #pragma unroll 1
   for (int d = 0; d < 3; ++d) {

@@ -192,13 +192,14 @@ __global__ void k_weights(const uint8_t* __restrict__ wm, double* mult, double* 
 }
 
 // The fixed-point factors of the FP64 operator (FxOp): one CTA per element,
-// first the element's largest exponents of G 2^t and B 2^t, then the integers.
+// first the element's largest exponents of G and B 2^t, then the integers.
 // 62 bits for G: with fields of 60 bits the three terms of a point's product
 // meet the bound of fx::dot.  B stays as it is (its conversion is part of the
 // mass term); only its exponent is kept.
 __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B,
-                                                 const int* __restrict__ ti, int n, int64_t E, int4* __restrict__ fG,
-                                                 int* __restrict__ sG, int* __restrict__ eB, int* bad) {
+                                                 const int* __restrict__ ti, unsigned long long K, int n,
+                                                 int64_t E, int4* __restrict__ fG, int* __restrict__ sG,
+                                                 int* __restrict__ eB, int* bad) {
   __shared__ int top[2];
   const int n3 = n * n * n;
   const int64_t e = blockIdx.x;
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
     if (G) {
       int hi = 0;
       for (int f = 0; f < 6; ++f) hi = max(hi, __double2hiint(G[(e * 6 + f) * n3 + p]) & 0x7fffffff);
-      mG = max(mG, fx::expo(hi) == 0x7ff ? 0x1000 : fx::expo(hi) + t);
+      mG = max(mG, fx::expo(hi) == 0x7ff ? 0x1000 : fx::expo(hi));
     }
     if (B) {
       const int hi = __double2hiint(B[e * n3 + p]) & 0x7fffffff;
@@ -224,25 +225,23 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
     // an all-zero B (h2 = 0 at every point of the element) is in range
     if ((G && abs(top[0] - 1023) > fx::kOpExp) || (B && top[1] != 0 && abs(top[1] - 1023) > fx::kOpExp))
       atomicExch(bad, 1);
-    if (G) sG[e] = 62 + 1022 - top[0];
+    if (G) sG[e] = 1083 - top[0];
     if (B) eB[e] = top[1] == 0 ? 1023 : top[1];
   }
   if (!G) return;
   for (int q = threadIdx.x; q < 3 * n3; q += blockDim.x) {
     const int p = q % n3, f = 2 * (q / n3);  // factors f and f + 1 of point p
-    const int i = p % n, j = (p / n) % n, k = p / (n * n);
-    const int t = ti[i] + ti[j] + ti[k];
-    const int2 x = fx::split(fx::from_double<62>(G[(e * 6 + f) * n3 + p], top[0] - t));
-    const int2 y = fx::split(fx::from_double<62>(G[(e * 6 + f + 1) * n3 + p], top[0] - t));
-    fG[e * 3 * n3 + fx::pair_index(n, f / 2, i, j, k)] = make_int4(x.x, x.y, y.x, y.y);
+    const int2 x = fx::split(fx::scaled_factor(G[(e * 6 + f) * n3 + p], K, top[0]));
+    const int2 y = fx::split(fx::scaled_factor(G[(e * 6 + f + 1) * n3 + p], K, top[0]));
+    fG[e * 3 * n3 + q] = make_int4(x.x, x.y, y.x, y.y);
   }
 }
 
 // ---- launchers ---------------------------------------------------------------
 
-cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, int n, int64_t E, int4* fG, int* sG,
-                           int* eB, int* bad, cudaStream_t s) {
-  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, ti, n, E, fG, sG, eB, bad);
+cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, unsigned long long K, int n, int64_t E,
+                           int4* fG, int* sG, int* eB, int* bad, cudaStream_t s) {
+  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, ti, K, n, E, fG, sG, eB, bad);
   return cudaGetLastError();
 }
 

@@ -21,9 +21,10 @@ void launch_coords_pipe(double* xyz, const double* xi, const double* tlev, int n
 // B and bad may be null
 cudaError_t launch_geometry(const double* xyz, double* G, double* B, const double* D, const double* w, int n,
                             int64_t E, int* bad, cudaStream_t s);
-// FxOp's G and sG from G (not null), its eB from B (not null); *bad is set if an element's exponents are out of range.
-cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, int n, int64_t E, int4* fG, int* sG,
-                           int* eB, int* bad, cudaStream_t s);
+// FxOp's G and sG from G (not null) and K (FxScale), its eB from B (not null); *bad is set if an element's exponents
+// are out of range.
+cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, unsigned long long K, int n, int64_t E,
+                           int4* fG, int* sG, int* eB, int* bad, cudaStream_t s);
 void launch_local_diag(const double* G, double* dK, const double* D, int n, int64_t E, cudaStream_t s);
 void launch_fold_coef(const double* G, const double* B, const double* h1, const double* h2, double* cG, double* cB,
                       int n, int64_t P, int* bad, cudaStream_t s);
@@ -31,14 +32,12 @@ void launch_split_f64(const double* v, float* hi, float* lo, int64_t m, cudaStre
 void launch_weights(const uint8_t* wm, double* mult, double* mask, int64_t m, cudaStream_t s);
 
 // ---- local operator (ax_*.cu) ----
-// Data of the fixed-point FP64 operator (ax_fx_impl.cuh, ax_fxd_impl.cuh); G null: not available.
+// Data of the fixed-point FP64 operator (ax_fx_impl.cuh); G null: not available.
 struct FxOp {
-  const int4* G = nullptr;       // G 2^(t + sG) as split 64-bit integers, two per int4 (layout: fx_index)
+  const int4* G = nullptr;       // [E][3][n^3]: factors (2f, 2f + 1) of a point, G kappa 2^sG (FxScale) as split integers
   const int* sG = nullptr;       // [E]
   const int* eB = nullptr;       // [E]: biased exponent of the element's largest B 2^t
-  const int4* tab = nullptr;     // D, then D^T: even-odd pairs [h][h] (even n), or [n][n] int2 (odd n)
-  const int* ti = nullptr;       // [n]: t of point (i, j, k) is ti[i] + ti[j] + ti[k]
-  int sc[2] = {0, 0};            // the tables hold D 2^sc[0] and D^T 2^sc[1]
+  const int* ti = nullptr;       // [n]: t of point (i, j, k) is ti[i] + ti[j] + ti[k], 2^-ti ~ w_i / max w
   int direct = 0;                // h1 or h2 outside the exponent range of the integer path
 };
 
@@ -90,7 +89,7 @@ struct AxDFParams {
 // 3 (FP32, even n only) the persistent bulk-copy pipelined kernels with
 // ~128 threads x 3 stages / ~256 threads x 2 stages; for the double-float
 // FP64 operator 2 and 3 are the even-odd kernels (even n only); 4 and 5 are the
-// fixed-point kernels of the native FP64 operator, with ~128 / ~256 threads.  A launch of a variant
+// fixed-point kernel of the native FP64 operator, with ~128 / ~256 threads.  A launch of a variant
 // that does not exist for (N, precision) returns cudaErrorNotSupported.
 constexpr int kAxVariants = 6, kAxFixed = 4;  // kAxFixed: the first fixed-point variant
 int ax_num_variants();

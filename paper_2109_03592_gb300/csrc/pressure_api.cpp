@@ -13,6 +13,7 @@
 #include <mutex>
 #include <vector>
 
+#include "fx_tables.h"
 #include "kernels.h"
 #include "sem_internal.h"
 
@@ -32,15 +33,9 @@ void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double
       pk = p;
     }
   };
-  std::vector<double> xd, wd, Dd;
-  gll(N, xd, wd, Dd);
-  std::vector<ld> x(xd.begin(), xd.end()), z(m);
+  std::vector<ld> x, z(m);
+  gll_points_ld(N, x);
   ld p, q;
-  for (int i = 1; i < N; ++i)  // roots of P_{N-1} - x P_N, whose derivative is -(N + 1) P_N
-    for (int it = 0; it < 4; ++it) {
-      legendre(N, x[i], p, q);
-      x[i] += (q - x[i] * p) / ((N + 1) * p);
-    }
   for (int i = 0; i < m; ++i) {
     z[i] = -std::cos(M_PI * (i + 0.75) / (m + 0.5));
     for (int it = 0; it < 8; ++it) {  // P_m' = m (P_{m-1} - x P_m) / (1 - x^2)
@@ -57,7 +52,6 @@ void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double
     }
     if (k & 1) v[k / 2] = 0;
   };
-  symmetric(x);
   symmetric(z);
   Ig.assign((size_t)m * n, 0);
   DIg.assign((size_t)m * n, 0);

@@ -163,10 +163,10 @@ __device__ __forceinline__ typename A::V dot(const typename A::C (&c)[K], const 
 #pragma unroll
     for (int l = 0; l < K; ++l)
       if (l < count) m = fx::mad(fx::mad(m, c[l].x, v[l].y), c[l].y, v[l].x);
-    ll r = m >> 32;
+    ll r = m >> 32;  // the upper products: see fx::dot
 #pragma unroll
     for (int l = 0; l < K; ++l)
-      if (l < count) r = fx::mad(r, c[l].y, v[l].y);
+      if (l < count) r = r + (ll)c[l].y * v[l].y;
     return r;
   } else {
     float s = 0.f;
@@ -191,10 +191,10 @@ __device__ __forceinline__ ll dot2(const int2 (&c)[K], const int2 (&v)[K], int n
   ll r = (m >> 32) + (k >> 32);
 #pragma unroll
   for (int l = 0; l < K; ++l)
-    if (l < nc) r = fx::mad(r, c[l].y, v[l].y);
+    if (l < nc) r = r + (ll)c[l].y * v[l].y;
 #pragma unroll
   for (int l = 0; l < L; ++l)
-    if (l < nd) r = fx::mad(r, d[l].y, w[l].y);
+    if (l < nd) r = r + (ll)d[l].y * w[l].y;
   return r;
 }
 
@@ -726,10 +726,7 @@ static __global__ void __launch_bounds__(256) k_pack_fx(const double* __restrict
   for (int r = threadIdx.x; r < 9 * m3; r += blockDim.x) {
     const int KJ = r % m2, b = r / m2 % 3, I = r / (3 * m2) % m, a = r / (3 * m3);
     const double f = F[(e * 9 + 3 * b + a) * m3 + KJ * m + I];
-    const int hi = __double2hiint(f), d = fx::expo(top[a]) - fx::expo(hi);
-    const unsigned long long x = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(f)) << 10;
-    const ll v = d > 61 || fx::expo(hi) == 0 ? 0 : (ll)(__umul64hi(x, K) >> (d + 1));
-    out[e * 9 * m3 + r] = fx::split(hi < 0 ? -v : v);
+    out[e * 9 * m3 + r] = fx::split(fx::scaled_factor(f, K, fx::expo(top[a])));
   }
 }
 

@@ -114,9 +114,7 @@ struct sem_mesh {
   int4* Gfx = nullptr;       // [E][3 n3] the factors in fixed point (FxOp); null where their exponents are out of range
   int* fx_sG = nullptr;      // [E] FxOp::sG
   int* fx_eB = nullptr;      // [E] FxOp::eB
-  int4* fx_tab = nullptr;    // D and D^T in fixed point (FxOp::tab)
   int* fx_ti = nullptr;      // [n] (FxOp::ti)
-  int fx_sc[2] = {0, 0};     // FxOp::sc
   double* wq = nullptr;      // [n] GLL weights
   double* dK = nullptr;      // [n_local] QQ^T diag of the stiffness (h1 = 1, h2 = 0)
   double* dB = nullptr;      // [n_local] QQ^T B
@@ -167,10 +165,7 @@ struct sem_mesh {
     f.G = b ? g : nullptr;
     f.sG = cG32 ? cfx_sG : fx_sG;
     f.eB = b;
-    f.tab = fx_tab;
     f.ti = fx_ti;
-    f.sc[0] = fx_sc[0];
-    f.sc[1] = fx_sc[1];
     return f;
   }
   const double* opB64() const { return cB64 ? cB64 : B64; }
