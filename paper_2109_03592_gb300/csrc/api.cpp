@@ -58,7 +58,8 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->B32lo);
   dev_free(m->Gfx);
   dev_free(m->fx_sG);
-  dev_free(m->fx_eB);
+  dev_free(m->Bfx);
+  dev_free(m->fx_sB);
   dev_free(m->fx_ti);
   dev_free(m->wq);
   dev_free(m->dK);
@@ -83,7 +84,8 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->cB32);
   dev_free(m->cB32lo);
   dev_free(m->cdB);
-  dev_free(m->cfx_eB);
+  dev_free(m->cBfx);
+  dev_free(m->cfx_sB);
   dev_free(m->Fgl);
   dev_free(m->pdinv);
   dev_free(m->Igl);
@@ -114,7 +116,8 @@ struct CoefArrays {
   float* B32 = nullptr;
   float* B32lo = nullptr;
   double* dB = nullptr;
-  int* fx_eB = nullptr;
+  int2* Bfx = nullptr;
+  int* fx_sB = nullptr;
   size_t bytes = 0;
   void release() {
     dev_free(G64);
@@ -127,7 +130,8 @@ struct CoefArrays {
     dev_free(B32);
     dev_free(B32lo);
     dev_free(dB);
-    dev_free(fx_eB);
+    dev_free(Bfx);
+    dev_free(fx_sB);
     bytes = 0;
   }
 };
@@ -157,7 +161,10 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     SEM_TRY(dev_alloc(&c.B32, P, c.bytes));
     SEM_TRY(dev_alloc(&c.dB, P, c.bytes));
     if (m->fp64_df) SEM_TRY(dev_alloc(&c.B32lo, P, c.bytes));
-    if (m->Gfx) SEM_TRY(dev_alloc(&c.fx_eB, m->E, c.bytes));
+    if (m->Gfx) {
+      SEM_TRY(dev_alloc(&c.Bfx, P, c.bytes));
+      SEM_TRY(dev_alloc(&c.fx_sB, m->E, c.bytes));
+    }
   }
   size_t tmp = 0;
   int* bad_d = nullptr;  // [2]: a bad coefficient; factors out of the fixed-point form's range
@@ -182,7 +189,8 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     launch_split_f64(c.B64, c.B32, c.B32lo, P, s);
   }
   if (m->Gfx && (h1 || h2)) {
-    SEM_CUDA(launch_fx_pack(c.G64, c.B64, m->fx_ti, fx_scale(m->N).K, n, m->E, c.Gfx, c.fx_sG, c.fx_eB, bad_d + 1, s));
+    SEM_CUDA(launch_fx_pack(c.G64, c.B64, m->fx_ti, fx_scale(m->N).K, n, m->E, c.Gfx, c.fx_sG, c.Bfx, c.fx_sB,
+                            bad_d + 1, s));
     count_launches(1);
   }
   SEM_CUDA(cudaGetLastError());
@@ -198,7 +206,8 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
   if (bad[1]) {  // coefficients beyond 2^+-200: the kernels on the FP64 pipe take them
     dev_drop(c.Gfx, 3 * P, c.bytes);
     dev_drop(c.fx_sG, m->E, c.bytes);
-    dev_drop(c.fx_eB, m->E, c.bytes);
+    dev_drop(c.Bfx, P, c.bytes);
+    dev_drop(c.fx_sB, m->E, c.bytes);
   } else if (h1 && !m->G64) {
     dev_drop(c.G64, 6 * P, c.bytes);  // as for the plain factors: no chosen kernel reads it
   }
@@ -288,7 +297,8 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_TRY(dev_alloc(&m->B32, P, tb));
   SEM_TRY(dev_alloc(&m->Gfx, 3 * P, tb));
   SEM_TRY(dev_alloc(&m->fx_sG, E, tb));
-  SEM_TRY(dev_alloc(&m->fx_eB, E, tb));
+  SEM_TRY(dev_alloc(&m->Bfx, P, tb));
+  SEM_TRY(dev_alloc(&m->fx_sB, E, tb));
   SEM_TRY(dev_alloc(&m->dK, P, tb));
   SEM_TRY(dev_alloc(&m->dB, P, tb));
   SEM_TRY(dev_alloc(&m->wm, P, tb));
@@ -367,7 +377,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_CUDA(launch_gs<double>(m->dB, gs_dev(m), 0, nullptr, s));
   launch_split_f64(m->G64, m->G32, nullptr, 6 * P, s);  // the low parts: autotune_mesh, where they are needed
   launch_split_f64(m->B64, m->B32, nullptr, P, s);
-  SEM_CUDA(launch_fx_pack(m->G64, m->B64, m->fx_ti, fx_scale(N).K, n, E, m->Gfx, m->fx_sG, m->fx_eB, bad_d + 1, s));
+  SEM_CUDA(launch_fx_pack(m->G64, m->B64, m->fx_ti, fx_scale(N).K, n, E, m->Gfx, m->fx_sG, m->Bfx, m->fx_sB, bad_d + 1, s));
   SEM_CUDA(cudaGetLastError());
   count_launches(8);
   int bad[2] = {0, 0};
@@ -380,7 +390,8 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   if (bad[1]) {
     dev_drop(m->Gfx, 3 * P, tb);
     dev_drop(m->fx_sG, E, tb);
-    dev_drop(m->fx_eB, E, tb);
+    dev_drop(m->Bfx, P, tb);
+    dev_drop(m->fx_sB, E, tb);
   }
   m->glo = std::move(topo.glo);
   return SEM_OK;
@@ -497,7 +508,7 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   CoefArrays c;
   sem_status st = build_coef(m, h1_dev, h2_dev, c, s);
   // h2 out of the fixed-point range: the kernels on the FP64 pipe read the plain factors
-  if (st == SEM_OK && h2_dev && !h1_dev && !c.fx_eB && m->Gfx) st = restore_G64(m, s);
+  if (st == SEM_OK && h2_dev && !h1_dev && !c.Bfx && m->Gfx) st = restore_G64(m, s);
   if (st != SEM_OK) {
     cudaStreamSynchronize(s);
     c.release();
@@ -517,7 +528,8 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   dev_free(m->cdB);
   dev_free(m->cGfx);
   dev_free(m->cfx_sG);
-  dev_free(m->cfx_eB);
+  dev_free(m->cBfx);
+  dev_free(m->cfx_sB);
   m->cG64 = c.G64;
   m->cG32 = c.G32;
   m->cG32lo = c.G32lo;
@@ -528,7 +540,8 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   m->cdB = c.dB;
   m->cGfx = c.Gfx;
   m->cfx_sG = c.fx_sG;
-  m->cfx_eB = c.fx_eB;
+  m->cBfx = c.Bfx;
+  m->cfx_sB = c.fx_sB;
   m->coef_bytes = c.bytes;
   m->dev_bytes += m->coef_bytes;
   m->coef_gen++;

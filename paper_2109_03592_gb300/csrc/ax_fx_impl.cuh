@@ -24,7 +24,8 @@
 // What bounds it: issue, of multiply-adds and of the additions between them (integer pipe 57% busy, multiply pipe
 // 35%, DRAM 46%).  One thread per 2x2x2 octant instead of per line needed twice the shared-memory reads and splits
 // (N = 7, E = 32,768: 361 us; this kernel 274, 4.9 TB/s of u, G and w; even-odd FP32 pairs 407, the FP64 pipe 1900;
-// odd n, column threads without the fold, N = 8, E = 22,528: 660; this kernel 312).  Not kept: the r- and s-lines
+// odd n, column threads without the fold, N = 8, E = 22,528: 660; this kernel 312).  The Helmholtz term, from B in fixed point loaded ahead of the
+// stores of w, adds 12% (308 us; converted from FP64 at each use, 25%).  Not kept: the r- and s-lines
 // through one copy of the code in a loop (no faster at N = 7, 4 to 11% slower above).
 #pragma once
 
@@ -131,6 +132,8 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     const int64_t e0 = (int64_t)blockIdx.x * EPB;
     const uint32_t bytes = (uint32_t)(min((int64_t)EPB, P.E - e0) * 6 * n3 * sizeof(int2));
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.fx.G + e0 * 3 * n3), "r"(bytes) : "memory");
+    if (P.helm && n % 2 == 0)  // (16-byte ranges)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.fx.B + e0 * n3), "r"(bytes / 6) : "memory");
   }
   for (int q = 0; q < 3; ++q) Max::clear(smax[q]);
   if (!Max::whole) __syncthreads();
@@ -269,6 +272,9 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     for (int k = 0; k < n; ++k) v[k] = shl(park ? T[L::idx(x, y, k)] : wt[k], up);
     contract<n>(Q.d.te, Q.d.to, v, wt);
   }
+  int2 B[n];  // loaded together, ahead of the stores of w
+#pragma unroll
+  for (int k = 0; k < n; ++k) B[k] = P.helm && act ? __ldg(P.fx.B + base + k * n2) : make_int2(0, 0);
   __syncthreads();
 
   double pw = 0.0;  // this thread's part of <p, A_L p>
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     const int tij = P.helm ? P.fx.ti[x] + P.fx.ti[y] : 0;
     int ec = ex;  // the line's coarsest unit
     if (P.helm) {
-      mt.init(P.h2, P.fx.eB[e], expo(ehi));
+      mt.init(P.h2, P.fx.sB[e], expo(ehi));
       ec = max(ex, mt.em - tij);
     }
 #pragma unroll
@@ -288,7 +294,7 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
       const int at = L::idx(x, y, k);
       ll o = wt[k] + R[at] + S[at];
       int eo = ex;
-      if (P.helm) mt.add(o, eo, __ldg(P.B + base + k * n2), split(U[at]), tij + P.fx.ti[k]);
+      if (P.helm) mt.add(o, eo, B[k], split(U[at]), tij + P.fx.ti[k]);
       P.w[base + k * n2] = to_double(o, eo);
       if (FUSED) {
         const int2 a = split(U[at]), b = split((o >> 5) >> min(ec - eo, 58));

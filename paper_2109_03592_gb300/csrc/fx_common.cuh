@@ -83,26 +83,29 @@ __device__ __forceinline__ double slow_point(const AxParams<double>& P, double k
   return out;
 }
 
-// h2 B u of one point onto the stiffness part o 2^eo, in the coarser of the two
-// terms' units.  B 2^t has 60 bits below the element's largest, h2's
-// mantissa 62, u 60; their product is taken to 57 bits.
+// h2 B u of a thread's points onto the stiffness part, in the coarser of the two terms' units.  B 2^t has 62 bits
+// below the element's largest, h2's mantissa 62, u 60; their product is taken to 59 bits.
 struct MassTerm {
   int2 h2;
-  int eB, em;
-  __device__ __forceinline__ void init(double h2v, int eB_, int eu) {
+  int em;  // value of a point of t = 0
+  __device__ __forceinline__ void init(double h2v, int sB, int eu) {  // eu: biased exponent of the element's largest u
     int e2;
     h2 = split(__double2ll_rn(ldexp(frexp(h2v, &e2), 62)));
-    eB = eB_;  // biased exponents of the element's largest B 2^t and u
-    em = 61 + 2 - (kBits + 1022 - eB) + e2 + eu - 1022 - kBits;
+    em = 61 + 2 - sB + e2 + eu - 1022 - kBits;
   }
-  __device__ __forceinline__ void add(ll& o, int& eo, double B, int2 u, int t) const {
-    const int2 b[1] = {split(from_double(B, eB - t))}, hh[1] = {h2};
-    const int2 hb = split(dot<1>(b, hh));  // at most 2^58
+  // o 2^eo + the mass term of B (fixed) and u; eo becomes the coarser unit
+  __device__ __forceinline__ void add(ll& o, int& eo, int2 B, int2 u, int t) const {
+    const int2 b[1] = {B}, hh[1] = {h2};
+    const int2 hb = split(dot<1>(b, hh));  // at most 2^60
     const ll m = mad(mad(1ll << 28, hb.x, u.y), hb.y, u.x);
     const ll v = (((ll)hb.y * u.y) << 3) + (m >> 29);  // hb u / 2^61
     const int d = eo - (em - t);
-    o = d >= 0 ? o + (v >> min(d, 63)) : (o >> min(-d, 63)) + v;
-    eo = max(eo, em - t);
+    if (d >= 0) {
+      o += v >> min(d, 63);
+    } else {
+      o = (o >> min(-d, 63)) + v;
+      eo = em - t;
+    }
   }
 };
 

@@ -194,12 +194,11 @@ __global__ void k_weights(const uint8_t* __restrict__ wm, double* mult, double* 
 // The fixed-point factors of the FP64 operator (FxOp): one CTA per element,
 // first the element's largest exponents of G and B 2^t, then the integers.
 // 62 bits for G: with fields of 60 bits the three terms of a point's product
-// meet the bound of fx::dot.  B stays as it is (its conversion is part of the
-// mass term); only its exponent is kept.
+// meet the bound of fx::dot.
 __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B,
                                                  const int* __restrict__ ti, unsigned long long K, int n,
                                                  int64_t E, int4* __restrict__ fG, int* __restrict__ sG,
-                                                 int* __restrict__ eB, int* bad) {
+                                                 int2* __restrict__ fB, int* __restrict__ sB, int* bad) {
   __shared__ int top[2];
   const int n3 = n * n * n;
   const int64_t e = blockIdx.x;
@@ -226,8 +225,13 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
     if ((G && abs(top[0] - 1023) > fx::kOpExp) || (B && top[1] != 0 && abs(top[1] - 1023) > fx::kOpExp))
       atomicExch(bad, 1);
     if (G) sG[e] = 1083 - top[0];
-    if (B) eB[e] = top[1] == 0 ? 1023 : top[1];
+    if (B) sB[e] = 62 + 1022 - (top[1] == 0 ? 1023 : top[1]);
   }
+  if (B)
+    for (int p = threadIdx.x; p < n3; p += blockDim.x) {
+      const int t = ti[p % n] + ti[(p / n) % n] + ti[p / (n * n)];
+      fB[e * n3 + p] = fx::split(fx::from_double<62>(B[e * n3 + p], (top[1] == 0 ? 1023 : top[1]) - t));
+    }
   if (!G) return;
   for (int q = threadIdx.x; q < 3 * n3; q += blockDim.x) {
     const int p = q % n3, f = 2 * (q / n3);  // factors f and f + 1 of point p
@@ -240,8 +244,8 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
 // ---- launchers ---------------------------------------------------------------
 
 cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, unsigned long long K, int n, int64_t E,
-                           int4* fG, int* sG, int* eB, int* bad, cudaStream_t s) {
-  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, ti, K, n, E, fG, sG, eB, bad);
+                           int4* fG, int* sG, int2* fB, int* sB, int* bad, cudaStream_t s) {
+  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, ti, K, n, E, fG, sG, fB, sB, bad);
   return cudaGetLastError();
 }
 

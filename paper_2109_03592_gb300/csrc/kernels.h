@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "device_util.cuh"
 #include "launch_once.h"
@@ -21,10 +22,10 @@ void launch_coords_pipe(double* xyz, const double* xi, const double* tlev, int n
 // B and bad may be null
 cudaError_t launch_geometry(const double* xyz, double* G, double* B, const double* D, const double* w, int n,
                             int64_t E, int* bad, cudaStream_t s);
-// FxOp's G and sG from G (not null) and K (FxScale), its eB from B (not null); *bad is set if an element's exponents
-// are out of range.
+// FxOp's G and sG from G (not null) and K (FxScale), its B and sB from B (not null); *bad is set if an element's
+// exponents are out of range.
 cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, unsigned long long K, int n, int64_t E,
-                           int4* fG, int* sG, int* eB, int* bad, cudaStream_t s);
+                           int4* fG, int* sG, int2* fB, int* sB, int* bad, cudaStream_t s);
 void launch_local_diag(const double* G, double* dK, const double* D, int n, int64_t E, cudaStream_t s);
 void launch_fold_coef(const double* G, const double* B, const double* h1, const double* h2, double* cG, double* cB,
                       int n, int64_t P, int* bad, cudaStream_t s);
@@ -36,10 +37,13 @@ void launch_weights(const uint8_t* wm, double* mult, double* mask, int64_t m, cu
 struct FxOp {
   const int4* G = nullptr;       // [E][3][n^3]: factors (2f, 2f + 1) of a point, G kappa 2^sG (FxScale) as split integers
   const int* sG = nullptr;       // [E]
-  const int* eB = nullptr;       // [E]: biased exponent of the element's largest B 2^t
+  const int2* B = nullptr;       // [E][n^3]: B 2^(t + sB), 62 bits below the element's largest
+  const int* sB = nullptr;       // [E]
   const int* ti = nullptr;       // [n]: t of point (i, j, k) is ti[i] + ti[j] + ti[k], 2^-ti ~ w_i / max w
   int direct = 0;                // h1 or h2 outside the exponent range of the integer path
 };
+
+struct NoOp {};
 
 template <typename T>
 struct AxParams {
@@ -58,7 +62,7 @@ struct AxParams {
   double* partial;   // [gridDim.x]
   int* err;          // device error word (bounded-wait timeouts of the bulk-copy kernels)
   T* pout = nullptr;  // fused: the new direction goes here (nullptr: over p)
-  FxOp fx;            // T = double: the fixed-point variants
+  std::conditional_t<std::is_same<T, double>::value, FxOp, NoOp> fx;  // T = double: the fixed-point variants
 };
 
 // Double-float (FP32 pair) FP64-accurate variant: G = Ghi + Glo, D = Dhi + Dlo,

@@ -113,7 +113,8 @@ struct sem_mesh {
   float* B32lo = nullptr;    // [E][n3] float(B64 - B32) (double-float only)
   int4* Gfx = nullptr;       // [E][3 n3] the factors in fixed point (FxOp); null where their exponents are out of range
   int* fx_sG = nullptr;      // [E] FxOp::sG
-  int* fx_eB = nullptr;      // [E] FxOp::eB
+  int2* Bfx = nullptr;       // [E][n3] FxOp::B
+  int* fx_sB = nullptr;      // [E] FxOp::sB
   int* fx_ti = nullptr;      // [n] (FxOp::ti)
   double* wq = nullptr;      // [n] GLL weights
   double* dK = nullptr;      // [n_local] QQ^T diag of the stiffness (h1 = 1, h2 = 0)
@@ -148,7 +149,8 @@ struct sem_mesh {
   float* cB32 = nullptr;
   float* cB32lo = nullptr;
   double* cdB = nullptr;
-  int* cfx_eB = nullptr;
+  int2* cBfx = nullptr;
+  int* cfx_sB = nullptr;
   uint64_t coef_gen = 0;
   size_t coef_bytes = 0;
 
@@ -161,10 +163,11 @@ struct sem_mesh {
   sem::FxOp opfx() const {
     sem::FxOp f;
     const int4* g = cG32 ? cGfx : Gfx;
-    const int* b = cB64 ? cfx_eB : fx_eB;
+    const int2* b = cB64 ? cBfx : Bfx;
     f.G = b ? g : nullptr;
     f.sG = cG32 ? cfx_sG : fx_sG;
-    f.eB = b;
+    f.B = b;
+    f.sB = cB64 ? cfx_sB : fx_sB;
     f.ti = fx_ti;
     return f;
   }
