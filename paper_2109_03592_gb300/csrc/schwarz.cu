@@ -87,35 +87,51 @@ __device__ __forceinline__ void load_row(const T* __restrict__ S, int r, T (&row
 }
 
 // out[c] = sum_l S[l][c] x[l] (trans = false) or sum_l S[c][l] x[l] (trans =
-// true) for the n x n matrix S in shared memory, rows read as broadcasts.
-template <int n, typename T, bool TRANS>
-__device__ __forceinline__ void line_contract(const T* __restrict__ S, const T (&x)[n], T (&out)[n]) {
+// true) for the n x n matrix S in shared memory and Q lines x, rows read as broadcasts.
+template <int n, typename T, bool TRANS, int Q>
+__device__ __forceinline__ void line_contract(const T* __restrict__ S, const T (&x)[Q][n], T (&out)[Q][n]) {
 #pragma unroll
-  for (int c = 0; c < n; ++c) out[c] = T(0);
+  for (int h = 0; h < Q; ++h)
+#pragma unroll
+    for (int c = 0; c < n; ++c) out[h][c] = T(0);
   T row[n];
   if constexpr (!TRANS) {
 #pragma unroll
     for (int l = 0; l < n; ++l) {
       load_row<n, T>(S, l, row);
 #pragma unroll
-      for (int c = 0; c < n; ++c) out[c] += row[c] * x[l];
+      for (int h = 0; h < Q; ++h)
+#pragma unroll
+        for (int c = 0; c < n; ++c) out[h][c] += row[c] * x[h][l];
     }
   } else {
 #pragma unroll
     for (int c = 0; c < n; ++c) {
       load_row<n, T>(S, c, row);
 #pragma unroll
-      for (int l = 0; l < n; ++l) out[c] += row[l] * x[l];
+      for (int h = 0; h < Q; ++h)
+#pragma unroll
+        for (int l = 0; l < n; ++l) out[h][c] += row[l] * x[h][l];
     }
   }
+}
+
+// Lines per thread: two in FP32 where n is a multiple of 4 (vector row reads), (a, b) and
+// (a, b + n / 2), so that a matrix row read from shared memory serves both: the matrices'
+// rows were half of the shared-memory reads that bound the kernel.  One application at E =
+// 32,768, N = 7: 318 us, 326 with one line.  For other n the rows are scalar reads that the
+// compiler keeps in registers (168 at n = 10 with two lines).
+template <int N, typename T>
+__host__ __device__ constexpr int fdm_lines() {
+  return (N + 1) % 4 == 0 && sizeof(T) == 4 ? 2 : 1;
 }
 
 // (With the 1D matrices hoisted into registers, 110 registers at N = 7 in
 // FP32; forcing three CTAs per SM then spilled and measured slower, 1.43 ms
 // instead of 1.32 ms for one FP32 application at E = 262,144.)
 template <int N, typename T, int EPB>
-__global__ void __launch_bounds__(EPB*(N + 1) * (N + 1)) k_fdm(const FdmParams<T> P) {
-  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
+__global__ void __launch_bounds__(EPB*(N + 1) * (N + 1) / fdm_lines<N, T>()) k_fdm(const FdmParams<T> P) {
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, Q = fdm_lines<N, T>(), nt = n2 / Q, db = n / Q;
   using L = FdmLay<n, T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sS = reinterpret_cast<T*>(smem_raw);  // [EPB][3][n][n]: S_r, S_s, S_t (row l, column = eigenvector)
@@ -129,107 +145,124 @@ __global__ void __launch_bounds__(EPB*(N + 1) * (N + 1)) k_fdm(const FdmParams<T
     __syncthreads();
     if (sdone) return;
   }
-  const int le = tid / n2, q = tid - le * n2;
-  const int a = q % n, b = q / n;  // this thread's line: (a, b) = the two fixed indices
+  const int le = tid / nt, q = tid - le * nt;
+  const int a = q % n, b = q / n;  // this thread's lines: (a, b + h db) = the two fixed indices
   const int64_t e = (int64_t)blockIdx.x * EPB + le;
   const bool act = e < P.E;
   T* Se = sS + le * 3 * n2;
   T* Le = sL + le * 3 * n;
   T* X = sX + le * L::size;
   if (act) {
-    for (int t = q; t < 3 * n2; t += n2) {
+    for (int t = q; t < 3 * n2; t += nt) {
       const int d = t / n2;
       Se[t] = P.S[(int64_t)P.sidx[3 * e + d] * n2 + (t - d * n2)];
     }
-    for (int t = q; t < 3 * n; t += n2) {
+    for (int t = q; t < 3 * n; t += nt) {
       const int d = t / n;
       Le[t] = P.lam[(int64_t)P.sidx[3 * e + d] * n + (t - d * n)];
     }
   }
-  // W r, coalesced: thread q holds point (i, j) = (a, b) of every k-plane
+  // W r, coalesced: the thread holds points (i, j) = (a, b + h db) of every k-plane
   const int64_t base = e * n3 + q;
   if (act) {
-    T t0 = T(0), t1 = T(0);  // coarse restriction of this column: sum_k f_b(xi_k) r / mult
 #pragma unroll
-    for (int k = 0; k < n; ++k) {
-      const T wk = P.wtab[P.wm[base + k * n2] & 0x7f];
-      const T wr = wk * P.r[base + k * n2];
-      X[L::idx(a, b, k)] = wr;
-      if (P.rc) {
-        const T rm = wk * wr;  // r / mult
-        t0 += P.ftab[k] * rm;
-        t1 += P.ftab[n + k] * rm;
+    for (int h = 0; h < Q; ++h) {
+      const int bb = b + h * db, qq = q + h * nt;
+      T t0 = T(0), t1 = T(0);  // coarse restriction of this column: sum_k f_b(xi_k) r / mult
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        const T wk = P.wtab[P.wm[base + h * nt + k * n2] & 0x7f];
+        const T wr = wk * P.r[base + h * nt + k * n2];
+        X[L::idx(a, bb, k)] = wr;
+        if (P.rc) {
+          const T rm = wk * wr;  // r / mult
+          t0 += P.ftab[k] * rm;
+          t1 += P.ftab[n + k] * rm;
+        }
       }
-    }
-    if (P.rc) {
-      T* R = sR + le * 8 * n2;
-      const T fa[2] = {P.ftab[a], P.ftab[n + a]}, fb[2] = {P.ftab[b], P.ftab[n + b]};
+      if (P.rc) {
+        T* R = sR + le * 8 * n2;
+        const T fa[2] = {P.ftab[a], P.ftab[n + a]}, fb[2] = {P.ftab[bb], P.ftab[n + bb]};
 #pragma unroll
-      for (int v = 0; v < 8; ++v) R[v * n2 + q] = fa[v & 1] * fb[(v >> 1) & 1] * ((v >> 2) & 1 ? t1 : t0);
+        for (int v = 0; v < 8; ++v) R[v * n2 + qq] = fa[v & 1] * fb[(v >> 1) & 1] * ((v >> 2) & 1 ? t1 : t0);
+      }
     }
   }
   __syncthreads();
   if (P.rc && act) {  // one thread per element vertex: the element's columns in order
-    for (int v = q; v < 8; v += n2) {
+    for (int v = q; v < 8; v += nt) {
       const T* R = sR + le * 8 * n2 + v * n2;
       T sum = T(0);
       for (int c = 0; c < n2; ++c) sum += R[c];
       P.rc[8 * e + v] = (double)sum;
     }
   }
-  T x[n], y[n];
-  // forward r: line (j, k) = (a, b)
+  T x[Q][n], y[Q][n];
+  // lines of direction D (0: (j, k) = (a, b), 1: (i, k), 2: (i, j)) from and to X
+  auto idx = [&](int dir, int l, int h) {
+    const int bb = b + h * db;
+    return dir == 0 ? L::idx(l, a, bb) : dir == 1 ? L::idx(a, l, bb) : L::idx(a, bb, l);
+  };
+  auto get = [&](int dir, T (&v)[Q][n]) {
+#pragma unroll
+    for (int h = 0; h < Q; ++h)
+#pragma unroll
+      for (int l = 0; l < n; ++l) v[h][l] = X[idx(dir, l, h)];
+  };
+  auto put = [&](int dir, const T (&v)[Q][n]) {
+#pragma unroll
+    for (int h = 0; h < Q; ++h)
+#pragma unroll
+      for (int l = 0; l < n; ++l) X[idx(dir, l, h)] = v[h][l];
+  };
+  // forward r
   if (act) {
-#pragma unroll
-    for (int l = 0; l < n; ++l) x[l] = X[L::idx(l, a, b)];
-    line_contract<n, T, false>(Se, x, y);
-#pragma unroll
-    for (int l = 0; l < n; ++l) X[L::idx(l, a, b)] = y[l];
+    get(0, x);
+    line_contract<n, T, false, Q>(Se, x, y);
+    put(0, y);
   }
   __syncthreads();
-  // forward s: line (i, k) = (a, b)
+  // forward s
   if (act) {
-#pragma unroll
-    for (int l = 0; l < n; ++l) x[l] = X[L::idx(a, l, b)];
-    line_contract<n, T, false>(Se + n2, x, y);
-#pragma unroll
-    for (int l = 0; l < n; ++l) X[L::idx(a, l, b)] = y[l];
+    get(1, x);
+    line_contract<n, T, false, Q>(Se + n2, x, y);
+    put(1, y);
   }
   __syncthreads();
-  // t: line (i, j) = (a, b): forward, divide by h1 (lam_r + lam_s + lam_t) + h2, back
+  // t: forward, divide by h1 (lam_r + lam_s + lam_t) + h2, back
   if (act) {
+    get(2, x);
+    line_contract<n, T, false, Q>(Se + 2 * n2, x, y);
 #pragma unroll
-    for (int l = 0; l < n; ++l) x[l] = X[L::idx(a, b, l)];
-    line_contract<n, T, false>(Se + 2 * n2, x, y);
-    const T lab = Le[a] + Le[n + b];
+    for (int h = 0; h < Q; ++h) {
+      const T lab = Le[a] + Le[n + b + h * db];
 #pragma unroll
-    for (int l = 0; l < n; ++l) y[l] = y[l] / (P.h1 * (lab + Le[2 * n + l]) + P.h2);
-    line_contract<n, T, true>(Se + 2 * n2, y, x);
-#pragma unroll
-    for (int l = 0; l < n; ++l) X[L::idx(a, b, l)] = x[l];
+      for (int l = 0; l < n; ++l) y[h][l] = y[h][l] / (P.h1 * (lab + Le[2 * n + l]) + P.h2);
+    }
+    line_contract<n, T, true, Q>(Se + 2 * n2, y, x);
+    put(2, x);
   }
   __syncthreads();
-  // back s: line (i, k) = (a, b)
+  // back s
   if (act) {
-#pragma unroll
-    for (int l = 0; l < n; ++l) x[l] = X[L::idx(a, l, b)];
-    line_contract<n, T, true>(Se + n2, x, y);
-#pragma unroll
-    for (int l = 0; l < n; ++l) X[L::idx(a, l, b)] = y[l];
+    get(1, x);
+    line_contract<n, T, true, Q>(Se + n2, x, y);
+    put(1, y);
   }
   __syncthreads();
-  // back r: line (j, k) = (a, b)
+  // back r
   if (act) {
-#pragma unroll
-    for (int l = 0; l < n; ++l) x[l] = X[L::idx(l, a, b)];
-    line_contract<n, T, true>(Se, x, y);
-#pragma unroll
-    for (int l = 0; l < n; ++l) X[L::idx(l, a, b)] = y[l];
+    get(0, x);
+    line_contract<n, T, true, Q>(Se, x, y);
+    put(0, y);
   }
   __syncthreads();
   if (act) {
 #pragma unroll
-    for (int k = 0; k < n; ++k) P.z[base + k * n2] = P.wtab[P.wm[base + k * n2] & 0x7f] * X[L::idx(a, b, k)];
+    for (int h = 0; h < Q; ++h)
+#pragma unroll
+      for (int k = 0; k < n; ++k)
+        P.z[base + h * nt + k * n2] = P.wtab[P.wm[base + h * nt + k * n2] & 0x7f] * X[L::idx(a, b + h * db, k)];
   }
 }
 
@@ -242,7 +275,9 @@ size_t fdm_smem() {
 template <int N, typename T>
 cudaError_t launch_fdm_n(const FdmParams<T>& p, cudaStream_t s) {
   constexpr int n = N + 1;
-  constexpr int EPB = (256 / (n * n)) < 1 ? 1 : 256 / (n * n);
+  constexpr int per = n * n / fdm_lines<N, T>();
+  constexpr int threads = fdm_lines<N, T>() == 2 ? 128 : 256;
+  constexpr int EPB = threads / per < 1 ? 1 : threads / per;
   const size_t smem = fdm_smem<N, T, EPB>();
   static DeviceOnce once;
   cudaError_t err = once.get([&](int, int*) {
@@ -251,7 +286,7 @@ cudaError_t launch_fdm_n(const FdmParams<T>& p, cudaStream_t s) {
   if (err != cudaSuccess) return err;
   if (p.E == 0) return cudaSuccess;
   const int64_t grid = (p.E + EPB - 1) / EPB;
-  k_fdm<N, T, EPB><<<(unsigned)grid, EPB * n * n, smem, s>>>(p);
+  k_fdm<N, T, EPB><<<(unsigned)grid, EPB * per, smem, s>>>(p);
   return cudaGetLastError();
 }
 
