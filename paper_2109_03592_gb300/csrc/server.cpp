@@ -66,8 +66,8 @@ int64_t local_points(const sem_mesh_desc& d) {
   return E * n * n * n;
 }
 
-// Device bytes one request holds while it runs: mesh arrays (~129 B per
-// local point, ~220 B while they are built), solver workspace (~96 B), the request's f, b, x (24 B) and the
+// Device bytes one request holds while it runs: mesh arrays (~137 B per
+// local point, ~228 B while they are built), solver workspace (~96 B), the request's f, b, x (24 B) and the
 // set-up scratch (8 B), plus a fixed allowance.
 size_t estimate_bytes(const sem_mesh_desc& d) { return (size_t)local_points(d) * 272 + (64u << 20); }
 
