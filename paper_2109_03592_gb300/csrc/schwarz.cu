@@ -116,11 +116,14 @@ __device__ __forceinline__ void line_contract(const T* __restrict__ S, const T (
   }
 }
 
-// Lines per thread: two in FP32 where n is a multiple of 4 (vector row reads), (a, b) and
+// Lines per thread, Q: two in FP32 where n is a multiple of 4 (vector row reads), (a, b) and
 // (a, b + n / 2), so that a matrix row read from shared memory serves both: the matrices'
 // rows were half of the shared-memory reads that bound the kernel.  One application at E =
-// 32,768, N = 7: 318 us, 326 with one line.  For other n the rows are scalar reads that the
-// compiler keeps in registers (168 at n = 10 with two lines).
+// 32,768, N = 7: 315 us, 326 with one line.  For other n the rows are scalar reads that the
+// compiler keeps in registers (168 at n = 10 with two lines).  Meshes of fewer than
+// kFdmPairElements keep one line: they do not fill the GPU (32 elements per SM, twice), and
+// two lines are twice the chain (a whole application on a small mesh 28.7 us, 27.7 with one).
+constexpr int64_t kFdmPairElements = 2 * 32 * 152;
 template <int N, typename T>
 __host__ __device__ constexpr int fdm_lines() {
   return (N + 1) % 4 == 0 && sizeof(T) == 4 ? 2 : 1;
@@ -129,9 +132,9 @@ __host__ __device__ constexpr int fdm_lines() {
 // (With the 1D matrices hoisted into registers, 110 registers at N = 7 in
 // FP32; forcing three CTAs per SM then spilled and measured slower, 1.43 ms
 // instead of 1.32 ms for one FP32 application at E = 262,144.)
-template <int N, typename T, int EPB>
-__global__ void __launch_bounds__(EPB*(N + 1) * (N + 1) / fdm_lines<N, T>()) k_fdm(const FdmParams<T> P) {
-  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, Q = fdm_lines<N, T>(), nt = n2 / Q, db = n / Q;
+template <int N, typename T, int EPB, int Q>
+__global__ void __launch_bounds__(EPB*(N + 1) * (N + 1) / Q) k_fdm(const FdmParams<T> P) {
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, nt = n2 / Q, db = n / Q;
   using L = FdmLay<n, T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sS = reinterpret_cast<T*>(smem_raw);  // [EPB][3][n][n]: S_r, S_s, S_t (row l, column = eigenvector)
@@ -272,22 +275,27 @@ size_t fdm_smem() {
   return sizeof(T) * ((size_t)EPB * (3 * n * n + 3 * n) + (size_t)EPB * FdmLay<n, T>::size + 8ull * EPB * n * n);
 }
 
-template <int N, typename T>
-cudaError_t launch_fdm_n(const FdmParams<T>& p, cudaStream_t s) {
-  constexpr int n = N + 1;
-  constexpr int per = n * n / fdm_lines<N, T>();
-  constexpr int threads = fdm_lines<N, T>() == 2 ? 128 : 256;
+template <int N, typename T, int Q>
+cudaError_t launch_fdm_q(const FdmParams<T>& p, cudaStream_t s) {
+  constexpr int per = (N + 1) * (N + 1) / Q;
+  constexpr int threads = Q == 2 ? 128 : 256;
   constexpr int EPB = threads / per < 1 ? 1 : threads / per;
   const size_t smem = fdm_smem<N, T, EPB>();
   static DeviceOnce once;
   cudaError_t err = once.get([&](int, int*) {
-    return cudaFuncSetAttribute(k_fdm<N, T, EPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return cudaFuncSetAttribute(k_fdm<N, T, EPB, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   if (err != cudaSuccess) return err;
   if (p.E == 0) return cudaSuccess;
   const int64_t grid = (p.E + EPB - 1) / EPB;
-  k_fdm<N, T, EPB><<<(unsigned)grid, EPB * per, smem, s>>>(p);
+  k_fdm<N, T, EPB, Q><<<(unsigned)grid, EPB * per, smem, s>>>(p);
   return cudaGetLastError();
+}
+
+template <int N, typename T>
+cudaError_t launch_fdm_n(const FdmParams<T>& p, cudaStream_t s) {
+  if (fdm_lines<N, T>() == 2 && p.E >= kFdmPairElements) return launch_fdm_q<N, T, fdm_lines<N, T>()>(p, s);
+  return launch_fdm_q<N, T, 1>(p, s);
 }
 
 // ---- coarse space -------------------------------------------------------------
