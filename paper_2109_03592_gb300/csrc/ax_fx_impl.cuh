@@ -30,6 +30,8 @@
 #pragma once
 
 #include <cmath>
+#include <cstdlib>
+#include <iterator>
 
 #include "ax_eo_impl.cuh"
 #include "ax_impl.cuh"
@@ -338,14 +340,28 @@ LineTable<N> line_table() {
   return t;
 }
 
-// The forward table times h1 2^-(its exponent), to half a unit.
+// The forward table times mant 2^-shift (h1 without its exponent, or half of that), to half a unit.
 template <class T>
-void scale_table(T& t, long long mant) {  // mant 2^-53 in (-1, 1)
-  for (auto& row : t)
-    for (int2& c : row) {
-      const __int128 p = (__int128)(((long long)c.y << 32) + c.x) * mant + (1ll << 52);
-      c = split((long long)(p >> 53));
+void scale_table(const T& from, T& to, long long mant, int shift) {  // mant 2^-53 in (-1, 1)
+  for (size_t r = 0; r < std::size(from); ++r)
+    for (size_t l = 0; l < std::size(from[r]); ++l) {
+      const int2 c = from[r][l];
+      const __int128 p = (__int128)(((long long)c.y << 32) + c.x) * mant + ((__int128)1 << (shift - 1));
+      to[r][l] = split((long long)(p >> shift));
     }
+}
+
+// Whether fx::dot's middle sums of the table's rows stay below 2^63 for all folded values (up to 2^61, so |y| <= 2^29 and
+// |x| <= 2^31).
+template <class T>
+bool sums_fit(const T& t) {
+  for (auto& row : t) {
+    unsigned long long s = 1ull << 31;
+    for (const int2& c : row)
+      s += ((unsigned long long)std::llabs(c.x) << 29) + ((unsigned long long)std::llabs(c.y) << 31);
+    if (s >> 63) return false;
+  }
+  return true;
 }
 
 template <int N, int EPB, bool FUSED>
@@ -365,8 +381,15 @@ cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out
   if (p.h1 != 1.0 && !p.fx.direct) {
     int e1 = 0;
     const long long mant = (long long)std::ldexp(std::frexp(p.h1, &e1), 53);
-    scale_table(q.d.e, mant);
-    scale_table(q.d.o, mant);
+    // The plain tables keep the sums below 0.8 2^63; a mantissa gives the entries any low halves, and then the sums of
+    // N >= 9 can pass 2^63 (at worst 1.15 2^63 at N = 11, where about 4 mantissas in 10,000 allow it).  Half the mantissa
+    // keeps them below 0.96 2^63, at the cost of one bit.
+    for (int shift = 53; shift <= 54; ++shift) {
+      scale_table(plain.e, q.d.e, mant, shift);
+      scale_table(plain.o, q.d.o, mant, shift);
+      if (sums_fit(q.d.e) && sums_fit(q.d.o)) break;
+      ++e1;
+    }
     q.scale += p.h1 == 0.0 ? 0 : e1;
   }
   k_ax_fx<N, EPB, FUSED><<<(unsigned)grid, line_threads(N, EPB), smem, s>>>(q);

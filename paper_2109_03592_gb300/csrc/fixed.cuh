@@ -39,7 +39,7 @@ __device__ __forceinline__ ll mad(ll acc, int a, int b) {
   return r;
 }
 
-// sum of c_l v_l / 2^64, rounded; the caller bounds sum |ch| + sum |vh| < 2^32 - 2^8.  fma_pipe: the upper products
+// sum of c_l v_l / 2^64, rounded; the caller bounds 2^31 + sum (|cl vh| + |ch vl|) < 2^63.  fma_pipe: the upper products
 // accumulate in the multiply-adds themselves (half their rate, no additions on the busier integer pipe); as mad() does
 // it, the compiler adds them up apart.  Faster by 4 to 7% in kernels of even n, slower by 4% at n = 9.
 template <int n, bool fma_pipe = true>
