@@ -11,8 +11,9 @@ using namespace fx;
 
 constexpr int kExpMin = 1023 - 500, kExpMax = 1023 + 500;  // biased exponents of u on the integer path
 
-// Maximum of v over an element's threads.  put() by every thread of the CTA, a barrier, then get(); `s` is
-// one of the CTA's arrays, used once.  Where an element is whole warps each warp has a word of its own;
+// Maximum of v over an element's threads.  put() by every thread of the CTA, which is whole warps (so all 32 lanes meet
+// in its warp operations, also behind a branch that some of them took), a barrier, then get(); `s` is one of the CTA's
+// arrays, used once.  Where an element is whole warps each warp has a word of its own;
 // otherwise the elements' words are cleared beforehand (clear(), and a barrier).
 template <int T, int EPB>
 struct ElemMax {
@@ -25,12 +26,11 @@ struct ElemMax {
   }
   __device__ static __forceinline__ void put(int* s, int le, int v) {  // v >= 0
     if constexpr (whole) {
-      v = __reduce_max_sync(__activemask(), v);
+      v = __reduce_max_sync(0xffffffffu, v);
       if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = v;
     } else if constexpr (T < 32 && 32 % T == 0) {
-      const unsigned mask = __activemask();
 #pragma unroll
-      for (int o = T / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(mask, v, o));
+      for (int o = T / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
       if (threadIdx.x % T == 0) atomicMax(s + le, v);
     } else {
       atomicMax(s + le, v);
