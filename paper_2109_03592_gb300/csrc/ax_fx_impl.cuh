@@ -299,12 +299,14 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
       if (P.helm) mt.add(o, eo, B[k], split(U[at]), tij + P.fx.ti[k]);
       P.w[base + k * n2] = to_double(o, eo);
       if (FUSED) {
-        const int2 a = split(U[at]), b = split((o >> 5) >> min(ec - eo, 58));
+        const int down = 5 + min(ec - eo, 56);  // to nearest: a floor has the same sign in every line
+        const int2 a = split(U[at]), b = split((o + (1ll << (down - 1))) >> down);
         ph = mad(ph, a.y, b.y);
         pm = mad(mad(pm, a.x, b.y), a.y, b.x);
       }
     }
-    if (FUSED) pw = ldexp(__ll2double_rn(ph + (pm >> 32)), 64 + 5 + ec + eu);
+    // the lines' sums cancel in <p, A p> (smooth p: to 1e-4 of them and less), so their low halves count
+    if (FUSED) pw = ldexp(fma(__ll2double_rn(pm), 0x1p-32, __ll2double_rn(ph)), 64 + 5 + ec + eu);
   } else if (act) {
     const double* v = FUSED ? (P.pout ? P.pout : P.p) : P.u;
 #pragma unroll 1
