@@ -162,14 +162,16 @@ sem_status apply_local(const sem_mesh* m, const void* u, void* w, double h1, dou
 // local operator on this mesh (the mesh's own factors as input) and keeps
 // the fastest; FP64 requests use the double-float kernel when it is faster.
 // SEM_FP64_KERNEL=native|df forces the FP64 choice.
-// Choices are cached per process by (N, log2 E): the first mesh of a shape
-// times the variants, later ones reuse its choice, so two meshes of the same
-// shape in one process always run the same kernels (and give bitwise-equal
-// results).
+// Choices are cached per process by (N, log2 E) and by whether the mesh's
+// factors have a fixed-point form (a mesh without one is timed without those
+// kernels): the first mesh of a shape times the variants, later ones reuse its
+// choice, so two meshes of the same shape in one process always run the same
+// kernels (and give bitwise-equal results).
 namespace {
 struct TuneKey {
   int N, lg;
-  bool operator==(const TuneKey& o) const { return N == o.N && lg == o.lg; }
+  bool fixed;
+  bool operator==(const TuneKey& o) const { return N == o.N && lg == o.lg && fixed == o.fixed; }
 };
 struct TuneVal {
   int var[3];
@@ -320,7 +322,7 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
 sem_status autotune_mesh(sem_mesh* m, cudaStream_t s) {
   int lg = 0;
   while ((1LL << (lg + 1)) <= m->E) ++lg;
-  const TuneKey key{m->N, lg};
+  const TuneKey key{m->N, lg, m->Gfx != nullptr};
   {
     std::lock_guard<std::mutex> lk(g_tune_mutex);
     for (auto& kv : g_tune)
