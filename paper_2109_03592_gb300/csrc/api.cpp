@@ -8,6 +8,7 @@
 #include <memory>
 #include <string>
 
+#include "fixed.cuh"
 #include "fx_tables.h"
 #include "kernels.h"
 #include "sem_internal.h"
@@ -60,7 +61,9 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->fx_sG);
   dev_free(m->Bfx);
   dev_free(m->fx_sB);
-  dev_free(m->fx_ti);
+  dev_free(m->fx_W);
+  dev_free(m->fx_tw);
+  dev_free(m->fx_W64);
   dev_free(m->wq);
   dev_free(m->dK);
   dev_free(m->dB);
@@ -171,6 +174,12 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
   SEM_TRY(dev_alloc(&bad_d, 2, tmp));
   std::unique_ptr<int, void (*)(int*)> bad_guard(bad_d, [](int* p) { cudaFree(p); });
   SEM_CUDA(cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s));
+  if (m->Gfx && (h1 || h2)) {  // the fixed-point factors, from those without quadrature weights
+    SEM_CUDA(launch_geometry(m->xyz, c.G64, c.B64, m->D64, m->wq + n, n, m->E, nullptr, s));
+    launch_fold_coef(c.G64, c.B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
+    SEM_CUDA(launch_fx_pack(c.G64, c.B64, n, m->E, c.Gfx, c.fx_sG, c.Bfx, c.fx_sB, bad_d + 1, s));
+    count_launches(3);
+  }
   const double* G = m->G64;
   if (h1 && !G) {  // the plain factors once more
     SEM_CUDA(launch_geometry(m->xyz, c.G64, nullptr, m->D64, m->wq, n, m->E, nullptr, s));
@@ -187,11 +196,6 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     SEM_CUDA(cudaMemcpyAsync(c.dB, c.B64, P * sizeof(double), cudaMemcpyDeviceToDevice, s));
     SEM_CUDA(launch_gs<double>(c.dB, gs_dev(m), 0, nullptr, s));
     launch_split_f64(c.B64, c.B32, c.B32lo, P, s);
-  }
-  if (m->Gfx && (h1 || h2)) {
-    SEM_CUDA(launch_fx_pack(c.G64, c.B64, m->fx_ti, fx_scale(m->N).K, n, m->E, c.Gfx, c.fx_sG, c.Bfx, c.fx_sB,
-                            bad_d + 1, s));
-    count_launches(1);
   }
   SEM_CUDA(cudaGetLastError());
   count_launches(1 + (h1 ? 3 : 0) + (h2 ? 2 : 0));
@@ -315,11 +319,21 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_TRY(dev_alloc(&m->eodf, eodf.size(), tb));
   }
 
-  std::vector<int> ti(n);  // the weights' exponents (FxOp)
-  const double wmax = *std::max_element(w.begin(), w.end());
-  for (int i = 0; i < n; ++i) ti[i] = (int)std::lround(-std::log2(w[i] / wmax));
-  SEM_TRY(dev_alloc(&m->fx_ti, n, tb));
-  SEM_TRY(dev_alloc(&m->wq, n, tb));
+  std::vector<long long> W;
+  std::vector<int> tw;
+  fx_weights(N, W, tw);
+  std::vector<int2> Wsplit(W.size());
+  std::vector<double> W64(W.size());
+  for (size_t q = 0; q < W.size(); ++q) {
+    Wsplit[q] = fx::split(W[q]);
+    W64[q] = std::ldexp((double)W[q], -tw[q % (n * n)]);
+  }
+  std::vector<double> w1(w);
+  w1.resize(2 * n, 1.0);
+  SEM_TRY(dev_alloc(&m->fx_W, W.size(), tb));
+  SEM_TRY(dev_alloc(&m->fx_tw, tw.size(), tb));
+  SEM_TRY(dev_alloc(&m->fx_W64, W64.size(), tb));
+  SEM_TRY(dev_alloc(&m->wq, 2 * n, tb));
 
   size_t tmp_bytes = 0;
   double *xi_d = nullptr, *tlev_d = nullptr;
@@ -338,8 +352,10 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_TRY(dev_alloc(&bad_d, 2, tmp_bytes));
 
   SEM_CUDA(cudaMemcpyAsync(xi_d, xi.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
-  SEM_CUDA(cudaMemcpyAsync(m->wq, w.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
-  SEM_CUDA(cudaMemcpyAsync(m->fx_ti, ti.data(), n * sizeof(int), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->wq, w1.data(), 2 * n * sizeof(double), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->fx_W, Wsplit.data(), Wsplit.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->fx_W64, W64.data(), W64.size() * sizeof(double), cudaMemcpyHostToDevice, s));
+  SEM_CUDA(cudaMemcpyAsync(m->fx_tw, tw.data(), tw.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D64, D.data(), n * n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32, D32.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32lo, D32lo.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));
@@ -369,6 +385,9 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_CUDA(cudaMemcpyAsync(m->xyz, d.xyz, 3 * P * sizeof(double), cudaMemcpyHostToDevice, s));
   }
   SEM_CUDA(cudaGetLastError());
+  // the fixed-point factors, from those without quadrature weights
+  SEM_CUDA(launch_geometry(m->xyz, m->G64, m->B64, m->D64, m->wq + n, n, E, bad_d, s));
+  SEM_CUDA(launch_fx_pack(m->G64, m->B64, n, E, m->Gfx, m->fx_sG, m->Bfx, m->fx_sB, bad_d + 1, s));
   SEM_CUDA(launch_geometry(m->xyz, m->G64, m->B64, m->D64, m->wq, n, E, bad_d, s));
   // assembled diagonals for the Jacobi preconditioner: dK = QQ^T diag(stiffness), dB = QQ^T B
   launch_local_diag(m->G64, m->dK, m->D64, n, E, s);
@@ -377,9 +396,8 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_CUDA(launch_gs<double>(m->dB, gs_dev(m), 0, nullptr, s));
   launch_split_f64(m->G64, m->G32, nullptr, 6 * P, s);  // the low parts: autotune_mesh, where they are needed
   launch_split_f64(m->B64, m->B32, nullptr, P, s);
-  SEM_CUDA(launch_fx_pack(m->G64, m->B64, m->fx_ti, fx_scale(N).K, n, E, m->Gfx, m->fx_sG, m->Bfx, m->fx_sB, bad_d + 1, s));
   SEM_CUDA(cudaGetLastError());
-  count_launches(8);
+  count_launches(9);
   int bad[2] = {0, 0};
   SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SEM_CUDA(cudaStreamSynchronize(s));

@@ -10,10 +10,16 @@
 // folds serve n outputs, and the tables are kernel parameters under unrolled loops, so
 // they are constant operands of the multiply-adds (fx::mad); t-lines stay in registers.
 //
+// Quadrature weights: A = D^T W G D = W M G D with M = W^-1 D^T W, whose entries are as large as D's (off the diagonal
+// they are -D's).  So the factors are kept without the weights, which multiply the result of a point at the end: they
+// fall by up to 7000 (N = 11) from an element's middle to its corners, and all values that share an exponent would carry
+// that.  Error against 64 bits over FP64's own, by emulation, at the corners: 0.4 (N = 11, random u; 340 with D^T W G D);
+// inside elements 0.1 to 1.3 (0.2 to 1.8).  The weights take 2% more time at N = 7, E = 262,144, none or less elsewhere.
+//
 // Scaling: u is brought to 60 bits below the element's largest exponent, the
 // gradients once more (those of smooth fields are small against the terms of D that
 // cancel), and so is G grad u; each table is scaled, not by a power of two, so that its
-// largest row sum of magnitudes keeps 60 bits within 60 bits, and the stored factors
+// largest row sum of magnitudes keeps 60 bits within 60 bits, and the weights
 // carry the inverse of the scales, with 62 bits.  The tables come from long-double GLL
 // points (fx_tables.cpp).
 //
@@ -42,7 +48,7 @@
 namespace sem {
 namespace fxk {
 
-// Even-odd tables of D and D^T (rows of the first half).
+// Even-odd tables of D and of M = W^-1 D^T W (rows of the first half).
 template <int N>
 struct LineTable {
   static constexpr int n = N + 1, np = (n + 1) / 2, nm = n / 2;
@@ -52,8 +58,9 @@ struct LineTable {
 template <int N>
 struct LineParams {
   AxParams<double> a;
-  double kappa;  // FxScale::K / 2^63
-  int scale;     // FxScale::scale and the exponent of h1
+  int scale;  // FxScale::scale and the exponent of h1
+  int2 h2;    // the mantissa of h2 / kappa, 62 bits, and its exponent
+  int e2;
   LineTable<N> d;
 };
 
@@ -281,37 +288,44 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
 
   double pw = 0.0;  // this thread's part of <p, A_L p>
   if (act && !slow) {
-    const int eu = expo(ehi) - 1022 - kBits;          // u = value 2^eu
-    const int ex = eu + Q.scale - sG - s1 - up;       // the stiffness part
-    ll ph = 0, pm = 0;
-    MassTerm mt;
-    const int tij = P.helm ? P.fx.ti[x] + P.fx.ti[y] : 0;
-    int ec = ex;  // the line's coarsest unit
+    const int eu = expo(ehi) - 1022 - kBits;    // u = value 2^eu
+    int eo = eu + Q.scale - sG - s1 - up;       // the unit of a point's sum, without its weights
+    MassTerm mt{Q.h2, 0};
     if (P.helm) {
-      mt.init(P.h2, P.fx.sB[e], expo(ehi));
-      ec = max(ex, mt.em - tij);
+      const int em = eu + 63 + Q.e2 - P.fx.sB[e];
+      mt.down = eo - em;
+      eo = max(eo, em);
     }
+    if (FUSED) eo += 64 - P.fx.tw[line];
+    // The weights: in FP64, whose pipe is idle, or for <p, A p> in integers, o W kept to 2^(64 - wb): |o| < 3 g 2^60 + 2^59
+    // (g: fx_tables.cpp) and W <= 2^62, so that stays below 2^63.  (Integers for both: 2697 us a plain apply at N = 7,
+    // E = 262,144.)
+    constexpr int wb = n % 2 ? 4 : 3;
+    ll ph = 0, pm = 0;
 #pragma unroll
     for (int k = 0; k < n; ++k) {
       const int at = L::idx(x, y, k);
       ll o = wt[k] + R[at] + S[at];
-      int eo = ex;
-      if (P.helm) mt.add(o, eo, B[k], split(U[at]), tij + P.fx.ti[k]);
-      P.w[base + k * n2] = to_double(o, eo);
-      if (FUSED) {
-        const int down = 5 + min(ec - eo, 56);  // to nearest: a floor has the same sign in every line
-        const int2 a = split(U[at]), b = split((o + (1ll << (down - 1))) >> down);
+      if (P.helm) o = mt.add(o, B[k], split(U[at]));
+      if (!FUSED) {
+        P.w[base + k * n2] = to_double(o, eo) * __ldg(P.fx.W64 + line + k * n2);
+      } else {
+        const int2 c = __ldg(P.fx.W + line + k * n2), v = split(o);
+        const ll m = mad(mad(0, c.x, v.y), c.y, v.x), h = (ll)c.y * v.y;
+        P.w[base + k * n2] = to_double(shl(h, wb) + ((m + (1ll << (31 - wb))) >> (32 - wb)), eo - wb);
+        // o W / 2^64 to nearest (a floor has the same sign in every line); two bits of p, which only scale it
+        const int2 a = split(U[at] >> 2), b = split(h + ((m + (1ll << 31)) >> 32));
         ph = mad(ph, a.y, b.y);
-        pm = mad(mad(pm, a.x, b.y), a.y, b.x);
+        pm = mad(mad(pm + __mulhi(a.x, b.x), a.x, b.y), a.y, b.x);  // (inside an element b is small: 2^-10 of its bound)
       }
     }
     // the lines' sums cancel in <p, A p> (smooth p: to 1e-4 of them and less), so their low halves count
-    if (FUSED) pw = ldexp(fma(__ll2double_rn(pm), 0x1p-32, __ll2double_rn(ph)), 64 + 5 + ec + eu);
+    if (FUSED) pw = ldexp(fma(__ll2double_rn(pm), 0x1p-32, __ll2double_rn(ph)), 64 + 2 + eo + eu);
   } else if (act) {
     const double* v = FUSED ? (P.pout ? P.pout : P.p) : P.u;
 #pragma unroll 1
     for (int k = 0; k < n; ++k) {
-      const double r = slow_point<N>(P, Q.kappa, v, e, x, y, k);
+      const double r = slow_point<N>(P, v, e, x, y, k);
       P.w[base + k * n2] = r;
       if (FUSED) pw += v[base + k * n2] * r;
     }
@@ -338,7 +352,7 @@ LineTable<N> line_table() {
     }
   };
   fill([&](int r, int l) { return f.D[r * n + l]; }, f.d, t.e, t.o);
-  fill([&](int r, int l) { return f.D[l * n + r]; }, f.dt, t.te, t.to);
+  fill([&](int r, int l) { return f.M[r * n + l]; }, f.dt, t.te, t.to);
   return t;
 }
 
@@ -379,7 +393,9 @@ cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out
   if (grid_out) *grid_out = (int)grid;
   if (p.E == 0) return cudaSuccess;
   static const LineTable<N> plain = line_table<N>();
-  LineParams<N> q{p, std::ldexp((double)fx_scale(N).K, -63), fx_scale(N).scale, plain};
+  LineParams<N> q{p, fx_scale(N).scale, make_int2(0, 0), 0, plain};
+  if (p.helm && !p.fx.direct)
+    q.h2 = split(std::llround(std::ldexp(std::frexp((long double)p.h2 / fx_scale(N).kappa, &q.e2), 62)));
   if (p.h1 != 1.0 && !p.fx.direct) {
     int e1 = 0;
     const long long mant = (long long)std::ldexp(std::frexp(p.h1, &e1), 53);

@@ -49,15 +49,14 @@ struct ElemMax {
 // w at one point of an element in FP64, straight from memory (Alg. 1, with the factors taken back from their
 // fixed-point form): for the rare element that the integer path does not cover.
 template <int N>
-__device__ __forceinline__ double slow_point(const AxParams<double>& P, double kappa, const double* v, int64_t e, int i,
-                                             int j, int k) {
+__device__ __forceinline__ double slow_point(const AxParams<double>& P, const double* v, int64_t e, int i, int j, int k) {
   constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
   const double* ue = v + e * n3;
   const int sG = P.fx.sG[e];
   auto G = [&](int f, int a, int b, int c) {
     const int4 x = P.fx.G[(e * 3 + (f >> 1)) * n3 + a + n * b + n2 * c];
     const int2 y = (f & 1) ? make_int2(x.z, x.w) : make_int2(x.x, x.y);
-    return ldexp(__ll2double_rn(shl(y.y, 32) + y.x) / kappa, -sG);
+    return ldexp(__ll2double_rn(shl(y.y, 32) + y.x), -sG) * (P.fx.wq[a] * P.fx.wq[b] * P.fx.wq[c]);
   };
   double out = 0.0;
 #pragma unroll 1
@@ -83,29 +82,18 @@ __device__ __forceinline__ double slow_point(const AxParams<double>& P, double k
   return out;
 }
 
-// h2 B u of a thread's points onto the stiffness part, in the coarser of the two terms' units.  B 2^t has 62 bits
-// below the element's largest, h2's mantissa 62, u 60; their product is taken to 59 bits.
+// h2 B u of a point onto the stiffness part, both without the quadrature weights, in the coarser of the two terms' units.
+// B has 62 bits below the element's largest, h2's mantissa (over kappa) 62, u 60; their product is taken to 59 bits.
 struct MassTerm {
   int2 h2;
-  int em;  // value of a point of t = 0
-  __device__ __forceinline__ void init(double h2v, int sB, int eu) {  // eu: biased exponent of the element's largest u
-    int e2;
-    h2 = split(__double2ll_rn(ldexp(frexp(h2v, &e2), 62)));
-    em = 61 + 2 - sB + e2 + eu - 1022 - kBits;
-  }
-  // o 2^eo + the mass term of B (fixed) and u; eo becomes the coarser unit
-  __device__ __forceinline__ void add(ll& o, int& eo, int2 B, int2 u, int t) const {
+  int down;  // the mass term's unit over the stiffness part's is 2^-down
+  // o (the stiffness part) + the mass term of B (fixed) and u
+  __device__ __forceinline__ ll add(ll o, int2 B, int2 u) const {
     const int2 b[1] = {B}, hh[1] = {h2};
     const int2 hb = split(dot<1>(b, hh));  // at most 2^60
     const ll m = mad(mad(1ll << 28, hb.x, u.y), hb.y, u.x);
     const ll v = (((ll)hb.y * u.y) << 3) + (m >> 29);  // hb u / 2^61
-    const int d = eo - (em - t);
-    if (d >= 0) {
-      o += v >> min(d, 63);
-    } else {
-      o = (o >> min(-d, 63)) + v;
-      eo = em - t;
-    }
+    return down >= 0 ? o + (v >> min(down, 63)) : (o >> min(-down, 63)) + v;
   }
 };
 

@@ -53,22 +53,34 @@ FxScale build(int N) {
     for (int l = 0; l < n; ++l) s += f.D[i * n + l];
     f.D[i * n + i] = -s;
   }
-  long double rows = 0, cols = 0;
+  f.w.resize(n);
+  for (int i = 0; i < n; ++i) {  // w_i = 2 / (N (N + 1) P_N(x_i)^2)
+    long double q = 1, p = x[i];
+    for (int j = 1; j < N; ++j) {
+      const long double t = ((2 * j + 1) * x[i] * p - j * q) / (j + 1);
+      q = p;
+      p = t;
+    }
+    f.w[i] = 2 / (N * (N + 1) * p * p);
+  }
+  f.M.assign((size_t)n * n, 0);
+  long double rows = 0, rows_m = 0;
   for (int i = 0; i < n; ++i) {
     long double a = 0, b = 0;
     for (int l = 0; l < n; ++l) {
+      f.M[i * n + l] = f.D[l * n + i] * f.w[l] / f.w[i];
       a += std::fabs(f.D[i * n + l]);
-      b += std::fabs(f.D[l * n + i]);
+      b += std::fabs(f.M[i * n + l]);
     }
     rows = std::max(rows, a);
-    cols = std::max(cols, b);
+    rows_m = std::max(rows_m, b);
   }
   const long double g = std::ldexp(n % 2 ? 0.5L : 0.8L, 64);
   f.d = g / rows;
-  f.dt = g / cols;
+  f.dt = g / rows_m;
   int j = 0;
   const long double m = std::frexp(f.d * f.dt, &j);  // m in [1/2, 1)
-  f.K = (unsigned long long)std::min(std::ldexp(1 / m, 63), 0x1.fffffffffffffffep63L);
+  f.kappa = 1 / m;
   f.scale = 192 - j;
   return f;
 }
@@ -80,6 +92,21 @@ const FxScale& fx_scale(int N) {
   static FxScale table[kMaxN + 1];
   std::call_once(once[N], [N] { table[N] = build(N); });
   return table[N];
+}
+
+void fx_weights(int N, std::vector<long long>& W, std::vector<int>& tw) {
+  const FxScale& f = fx_scale(N);
+  const int n = N + 1;
+  const long double wmax = *std::max_element(f.w.begin(), f.w.end());
+  W.resize((size_t)n * n * n);
+  tw.resize((size_t)n * n);
+  for (int ij = 0; ij < n * n; ++ij) {
+    const long double c = f.w[ij % n] * f.w[ij / n] * f.kappa;
+    int top = 0;
+    std::frexp(c * wmax, &top);
+    tw[ij] = 62 - top;
+    for (int k = 0; k < n; ++k) W[(size_t)k * n * n + ij] = std::llround(std::ldexp(c * f.w[k], tw[ij]));
+  }
 }
 
 }  // namespace sem

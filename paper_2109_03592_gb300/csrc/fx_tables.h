@@ -5,15 +5,19 @@
 
 namespace sem {
 
-// D of order N in long double and the scales of its fixed-point tables: the tables are D d and D^T dt, the stored
-// factors G kappa 2^sG with kappa = K / 2^63 = 2^j / (d dt) in [1, 2], and scale = 192 - j.
+// D of order N in long double, M = W^-1 D^T W (W: the GLL weights w) and the scales of their fixed-point tables D d and
+// M dt, with 1 / (d dt) = kappa 2^-j, kappa in [1, 2], and scale = 192 - j.
 struct FxScale {
-  std::vector<long double> D;  // [n][n]
-  long double d, dt;
-  unsigned long long K;
+  std::vector<long double> D, M;  // [n][n]
+  std::vector<long double> w;     // [n]
+  long double d, dt, kappa;
   int scale;
 };
 const FxScale& fx_scale(int N);  // N = 1 .. 11; built once per order
+
+// w_i w_j w_k kappa of the points (FxOp::W) as integers of at most 62 bits, below the largest of their t-line (i, j) by
+// 2^-tw: W [n^3], tw [n^2].
+void fx_weights(int N, std::vector<long long>& W, std::vector<int>& tw);
 
 // GLL points of order N in long double.
 void gll_points_ld(int N, std::vector<long double>& x);

@@ -116,13 +116,15 @@ __global__ void k_geometry(const double* __restrict__ xyz, double* __restrict__ 
     const double g4 = s * (C00 * C01 + C10 * C11 + C20 * C21);
     const double g5 = s * (C00 * C02 + C10 * C12 + C20 * C22);
     const double g6 = s * (C01 * C02 + C11 * C12 + C21 * C22);
-    double* Ge = G + e * 6 * n3 + p;
-    Ge[0] = g1;
-    Ge[n3] = g2;
-    Ge[2 * n3] = g3;
-    Ge[3 * n3] = g4;
-    Ge[4 * n3] = g5;
-    Ge[5 * n3] = g6;
+    if (G) {
+      double* Ge = G + e * 6 * n3 + p;
+      Ge[0] = g1;
+      Ge[n3] = g2;
+      Ge[2 * n3] = g3;
+      Ge[3 * n3] = g4;
+      Ge[4 * n3] = g5;
+      Ge[5 * n3] = g6;
+    }
     if (B) B[e * n3 + p] = w3 * det;
   }
 }
@@ -165,9 +167,9 @@ __global__ void k_split_f64(const double* __restrict__ v, float* __restrict__ hi
 // point by h1 of that point, which is h1 G at the point; the mass term scales
 // B u by h2.  Bit 0 / 1 of *bad flags an h1 <= 0 / h2 < 0 or a non-finite
 // value.
-__global__ void k_fold_coef(const double* G, const double* __restrict__ B, const double* __restrict__ h1,
-                            const double* __restrict__ h2, double* cG, double* __restrict__ cB, int n3, int64_t P,
-                            int* bad) {  // cG may be G
+__global__ void k_fold_coef(const double* G, const double* B, const double* __restrict__ h1,
+                            const double* __restrict__ h2, double* cG, double* cB, int n3, int64_t P,
+                            int* bad) {  // cG may be G and cB B
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < P; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t e = q / n3, r = q - e * n3;
     if (h1) {
@@ -192,11 +194,10 @@ __global__ void k_weights(const uint8_t* __restrict__ wm, double* mult, double* 
 }
 
 // The fixed-point factors of the FP64 operator (FxOp): one CTA per element,
-// first the element's largest exponents of G and B 2^t, then the integers.
-// 62 bits for G: with fields of 60 bits the three terms of a point's product
+// first the element's largest exponents of G and B, then the integers.  62
+// bits for G: with fields of 60 bits the three terms of a point's product
 // meet the bound of fx::dot.
-__global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B,
-                                                 const int* __restrict__ ti, unsigned long long K, int n,
+__global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B, int n,
                                                  int64_t E, int4* __restrict__ fG, int* __restrict__ sG,
                                                  int2* __restrict__ fB, int* __restrict__ sB, int* bad) {
   __shared__ int top[2];
@@ -206,46 +207,36 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
   __syncthreads();
   int mG = 0, mB = 0;
   for (int p = threadIdx.x; p < n3; p += blockDim.x) {
-    const int t = ti[p % n] + ti[(p / n) % n] + ti[p / (n * n)];
-    if (G) {
-      int hi = 0;
-      for (int f = 0; f < 6; ++f) hi = max(hi, __double2hiint(G[(e * 6 + f) * n3 + p]) & 0x7fffffff);
-      mG = max(mG, fx::expo(hi) == 0x7ff ? 0x1000 : fx::expo(hi));
-    }
-    if (B) {
-      const int hi = __double2hiint(B[e * n3 + p]) & 0x7fffffff;
-      mB = max(mB, fx::expo(hi) == 0x7ff ? 0x1000 : hi ? fx::expo(hi) + t : 0);
-    }
+    if (G)
+      for (int f = 0; f < 6; ++f) mG = max(mG, __double2hiint(G[(e * 6 + f) * n3 + p]) & 0x7fffffff);
+    if (B) mB = max(mB, __double2hiint(B[e * n3 + p]) & 0x7fffffff);
   }
   atomicMax(&top[0], mG);
   atomicMax(&top[1], mB);
   __syncthreads();
+  // an all-zero B (h2 = 0 at every point of the element) is in range
+  const int tG = fx::expo(top[0]), tB = top[1] ? fx::expo(top[1]) : 1023;
   if (threadIdx.x == 0) {
-    // an all-zero B (h2 = 0 at every point of the element) is in range
-    if ((G && abs(top[0] - 1023) > fx::kOpExp) || (B && top[1] != 0 && abs(top[1] - 1023) > fx::kOpExp))
-      atomicExch(bad, 1);
-    if (G) sG[e] = 1083 - top[0];
-    if (B) sB[e] = 62 + 1022 - (top[1] == 0 ? 1023 : top[1]);
+    if ((G && abs(tG - 1023) > fx::kOpExp) || (B && abs(tB - 1023) > fx::kOpExp)) atomicExch(bad, 1);
+    if (G) sG[e] = 62 + 1022 - tG;
+    if (B) sB[e] = 62 + 1022 - tB;
   }
   if (B)
-    for (int p = threadIdx.x; p < n3; p += blockDim.x) {
-      const int t = ti[p % n] + ti[(p / n) % n] + ti[p / (n * n)];
-      fB[e * n3 + p] = fx::split(fx::from_double<62>(B[e * n3 + p], (top[1] == 0 ? 1023 : top[1]) - t));
-    }
+    for (int p = threadIdx.x; p < n3; p += blockDim.x) fB[e * n3 + p] = fx::split(fx::from_double<62>(B[e * n3 + p], tB));
   if (!G) return;
   for (int q = threadIdx.x; q < 3 * n3; q += blockDim.x) {
     const int p = q % n3, f = 2 * (q / n3);  // factors f and f + 1 of point p
-    const int2 x = fx::split(fx::scaled_factor(G[(e * 6 + f) * n3 + p], K, top[0]));
-    const int2 y = fx::split(fx::scaled_factor(G[(e * 6 + f + 1) * n3 + p], K, top[0]));
+    const int2 x = fx::split(fx::from_double<62>(G[(e * 6 + f) * n3 + p], tG));
+    const int2 y = fx::split(fx::from_double<62>(G[(e * 6 + f + 1) * n3 + p], tG));
     fG[e * 3 * n3 + q] = make_int4(x.x, x.y, y.x, y.y);
   }
 }
 
 // ---- launchers ---------------------------------------------------------------
 
-cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, unsigned long long K, int n, int64_t E,
-                           int4* fG, int* sG, int2* fB, int* sB, int* bad, cudaStream_t s) {
-  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, ti, K, n, E, fG, sG, fB, sB, bad);
+cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int* sG, int2* fB, int* sB,
+                           int* bad, cudaStream_t s) {
+  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, n, E, fG, sG, fB, sB, bad);
   return cudaGetLastError();
 }
 

@@ -19,13 +19,13 @@ void launch_coords_box(double* xyz, const double* xi, int n, int64_t E, int nx, 
                        double ly, double lz, cudaStream_t s);
 void launch_coords_pipe(double* xyz, const double* xi, const double* tlev, int n, int64_t E, int nc, int nr,
                         int nzp, double R, double L, double a, cudaStream_t s);
-// B and bad may be null
+// w: the quadrature weights, or ones; G, B and bad may be null
 cudaError_t launch_geometry(const double* xyz, double* G, double* B, const double* D, const double* w, int n,
                             int64_t E, int* bad, cudaStream_t s);
-// FxOp's G and sG from G (not null) and K (FxScale), its B and sB from B (not null); *bad is set if an element's
-// exponents are out of range.
-cudaError_t launch_fx_pack(const double* G, const double* B, const int* ti, unsigned long long K, int n, int64_t E,
-                           int4* fG, int* sG, int2* fB, int* sB, int* bad, cudaStream_t s);
+// FxOp's G and sG from G (not null), its B and sB from B (not null), both made with weights of 1; *bad is set if an
+// element's exponents are out of range.
+cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int* sG, int2* fB, int* sB,
+                           int* bad, cudaStream_t s);
 void launch_local_diag(const double* G, double* dK, const double* D, int n, int64_t E, cudaStream_t s);
 void launch_fold_coef(const double* G, const double* B, const double* h1, const double* h2, double* cG, double* cB,
                       int n, int64_t P, int* bad, cudaStream_t s);
@@ -35,12 +35,15 @@ void launch_weights(const uint8_t* wm, double* mult, double* mask, int64_t m, cu
 // ---- local operator (ax_*.cu) ----
 // Data of the fixed-point FP64 operator (ax_fx_impl.cuh); G null: not available.
 struct FxOp {
-  const int4* G = nullptr;       // [E][3][n^3]: factors (2f, 2f + 1) of a point, G kappa 2^sG (FxScale) as split integers
-  const int* sG = nullptr;       // [E]
-  const int2* B = nullptr;       // [E][n^3]: B 2^(t + sB), 62 bits below the element's largest
-  const int* sB = nullptr;       // [E]
-  const int* ti = nullptr;       // [n]: t of point (i, j, k) is ti[i] + ti[j] + ti[k], 2^-ti ~ w_i / max w
-  int direct = 0;                // h1 or h2 outside the exponent range of the integer path
+  const int4* G = nullptr;    // [E][3][n^3]: factors (2f, 2f + 1) of a point without the quadrature weights, times 2^sG
+  const int* sG = nullptr;    // [E]
+  const int2* B = nullptr;    // [E][n^3]: the mass without them, times 2^sB (both: 62 bits below the element's largest)
+  const int* sB = nullptr;    // [E]
+  const int2* W = nullptr;    // [n^3]: w_i w_j w_k kappa 2^tw (fx_weights)
+  const int* tw = nullptr;    // [n^2]: tw of the t-line (i, j)
+  const double* W64 = nullptr; // [n^3]: w_i w_j w_k kappa
+  const double* wq = nullptr; // [n]: the weights
+  int direct = 0;             // h1 or h2 outside the exponent range of the integer path
 };
 
 struct NoOp {};

@@ -115,8 +115,10 @@ struct sem_mesh {
   int* fx_sG = nullptr;      // [E] FxOp::sG
   int2* Bfx = nullptr;       // [E][n3] FxOp::B
   int* fx_sB = nullptr;      // [E] FxOp::sB
-  int* fx_ti = nullptr;      // [n] (FxOp::ti)
-  double* wq = nullptr;      // [n] GLL weights
+  int2* fx_W = nullptr;      // [n3] FxOp::W
+  int* fx_tw = nullptr;      // [n2] FxOp::tw
+  double* fx_W64 = nullptr;  // [n3] FxOp::W64
+  double* wq = nullptr;      // [2 n] GLL weights, then ones
   double* dK = nullptr;      // [n_local] QQ^T diag of the stiffness (h1 = 1, h2 = 0)
   double* dB = nullptr;      // [n_local] QQ^T B
   uint8_t* wm = nullptr;     // [n_local] multiplicity | 0x80 Dirichlet
@@ -168,7 +170,10 @@ struct sem_mesh {
     f.sG = cG32 ? cfx_sG : fx_sG;
     f.B = b;
     f.sB = cB64 ? cfx_sB : fx_sB;
-    f.ti = fx_ti;
+    f.W = fx_W;
+    f.tw = fx_tw;
+    f.W64 = fx_W64;
+    f.wq = wq;
     return f;
   }
   const double* opB64() const { return cB64 ? cB64 : B64; }
