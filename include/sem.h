@@ -180,7 +180,12 @@ sem_status sem_mesh_set_coefficients(sem_mesh* mesh, const double* h1_dev, const
  * h1 (scaling the stiffness after the G contraction) and h2 (scaling B u):
  * scalars, times the mesh's per-point coefficients if it has any.
  * No assembly and no mask.  u and w: local vectors of `prec` SEM_FP64 or
- * SEM_FP32 (SEM_FP32 uses the FP32 factors).  u and w must not overlap. */
+ * SEM_FP32 (SEM_FP32 uses the FP32 factors).  u and w must not overlap.
+ * FP64 results are as accurate as FP64 evaluation at every point: relative
+ * to the sum of the magnitudes of its terms, to 2^-51 where one of the three
+ * lines of points through it has values within 2^-6 of the element's largest,
+ * and to 2^-45 for any finite u with values above 2^-44 of the element's
+ * largest (smaller ones count as the rounding of zeros). */
 sem_status sem_ax(const sem_mesh* mesh, const void* u_dev, void* w_dev, double h1, double h2,
                   sem_prec prec, void* stream);
 

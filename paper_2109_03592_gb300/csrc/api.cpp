@@ -113,7 +113,8 @@ struct CoefArrays {
   float* G32 = nullptr;
   float* G32lo = nullptr;
   int4* Gfx = nullptr;
-  int* fx_sG = nullptr;
+  int2* fx_sG = nullptr;
+  int fx_range = 0;
   double* dK = nullptr;
   double* B64 = nullptr;
   float* B32 = nullptr;
@@ -170,10 +171,10 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     }
   }
   size_t tmp = 0;
-  int* bad_d = nullptr;  // [2]: a bad coefficient; factors out of the fixed-point form's range
-  SEM_TRY(dev_alloc(&bad_d, 2, tmp));
+  int* bad_d = nullptr;  // [3]: a bad coefficient; launch_fx_pack's two
+  SEM_TRY(dev_alloc(&bad_d, 3, tmp));
   std::unique_ptr<int, void (*)(int*)> bad_guard(bad_d, [](int* p) { cudaFree(p); });
-  SEM_CUDA(cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s));
+  SEM_CUDA(cudaMemsetAsync(bad_d, 0, 3 * sizeof(int), s));
   if (m->Gfx && (h1 || h2)) {  // the fixed-point factors, from those without quadrature weights
     SEM_CUDA(launch_geometry(m->xyz, c.G64, c.B64, m->D64, m->wq + n, n, m->E, nullptr, s));
     launch_fold_coef(c.G64, c.B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
@@ -199,14 +200,15 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
   }
   SEM_CUDA(cudaGetLastError());
   count_launches(1 + (h1 ? 3 : 0) + (h2 ? 2 : 0));
-  int bad[2] = {0, 0};
-  SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  int bad[3] = {0, 0, 0};
+  SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SEM_CUDA(cudaStreamSynchronize(s));
   if (bad[0]) {
     set_error((bad[0] & 1) ? "sem_mesh_set_coefficients: need finite h1 > 0 at every point"
                            : "sem_mesh_set_coefficients: need finite h2 >= 0 at every point");
     return SEM_ERR_INVALID;
   }
+  c.fx_range = bad[2];
   if (bad[1]) {  // coefficients beyond 2^+-200: the kernels on the FP64 pipe take them
     dev_drop(c.Gfx, 3 * P, c.bytes);
     dev_drop(c.fx_sG, m->E, c.bytes);
@@ -337,7 +339,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
 
   size_t tmp_bytes = 0;
   double *xi_d = nullptr, *tlev_d = nullptr;
-  int* bad_d = nullptr;  // [2]: det J <= 0; factors out of the fixed-point form's range
+  int* bad_d = nullptr;  // [3]: det J <= 0; launch_fx_pack's two
   struct Tmp {
     double** a;
     double** c;
@@ -349,7 +351,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     }
   } tmp{&xi_d, &tlev_d, &bad_d};
   SEM_TRY(dev_alloc(&xi_d, n, tmp_bytes));
-  SEM_TRY(dev_alloc(&bad_d, 2, tmp_bytes));
+  SEM_TRY(dev_alloc(&bad_d, 3, tmp_bytes));
 
   SEM_CUDA(cudaMemcpyAsync(xi_d, xi.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->wq, w1.data(), 2 * n * sizeof(double), cudaMemcpyHostToDevice, s));
@@ -363,7 +365,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_CUDA(cudaMemcpyAsync(m->eo64, eo64.data(), eo64.size() * sizeof(double), cudaMemcpyHostToDevice, s));
     SEM_CUDA(cudaMemcpyAsync(m->eodf, eodf.data(), eodf.size() * sizeof(float), cudaMemcpyHostToDevice, s));
   }
-  SEM_CUDA(cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s));
+  SEM_CUDA(cudaMemsetAsync(bad_d, 0, 3 * sizeof(int), s));
   SEM_CUDA(cudaMemsetAsync(m->dev_err, 0, sizeof(int), s));
   SEM_CUDA(cudaMemcpyAsync(m->wm, plan.wm.data(), P, cudaMemcpyHostToDevice, s));
   if (!plan.idx.empty())
@@ -398,13 +400,14 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   launch_split_f64(m->B64, m->B32, nullptr, P, s);
   SEM_CUDA(cudaGetLastError());
   count_launches(9);
-  int bad[2] = {0, 0};
-  SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  int bad[3] = {0, 0, 0};
+  SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SEM_CUDA(cudaStreamSynchronize(s));
   if (bad[0]) {
     set_error("mesh has an element with det(J) <= 0");
     return SEM_ERR_BAD_MESH;
   }
+  m->fx_range = bad[2];
   if (bad[1]) {
     dev_drop(m->Gfx, 3 * P, tb);
     dev_drop(m->fx_sG, E, tb);
@@ -558,6 +561,7 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   m->cdB = c.dB;
   m->cGfx = c.Gfx;
   m->cfx_sG = c.fx_sG;
+  m->cfx_range = c.fx_range;
   m->cBfx = c.Bfx;
   m->cfx_sB = c.fx_sB;
   m->coef_bytes = c.bytes;

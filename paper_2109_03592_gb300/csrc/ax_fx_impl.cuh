@@ -23,9 +23,9 @@
 // carry the inverse of the scales, with 62 bits.  The tables come from long-double GLL
 // points (fx_tables.cpp).
 //
-// An element whose values are not finite, or whose exponents lie outside the
-// range that the shifts are written for (2^-500 .. 2^500), is evaluated in FP64
-// directly from memory (slow_point).
+// An element whose values are not finite, whose exponents lie outside the range
+// that the shifts are written for (2^-500 .. 2^500), or whose small values stand
+// alone beside large ones (line_state) is evaluated in FP64 (element_fp64).
 //
 // What bounds it: issue, of multiply-adds and of the additions between them (integer pipe 57% busy, multiply pipe
 // 35%, DRAM 46%).  One thread per 2x2x2 octant instead of per line needed twice the shared-memory reads and splits
@@ -61,6 +61,7 @@ struct LineParams {
   int scale;  // FxScale::scale and the exponent of h1
   int2 h2;    // the mantissa of h2 / kappa, 62 bits, and its exponent
   int e2;
+  int mass_limit;  // sG - sB beyond which the mass term outweighs the stiffness and is added in FP64
   LineTable<N> d;
 };
 
@@ -107,6 +108,101 @@ __device__ __forceinline__ void contract(const int2 (&e)[(n + 1) / 2][(n + 1) / 
   }
 }
 
+// Whether a point of the t-line (x, y) of u has small lines and no good one (line_state); *alone tells whether any of the
+// element has.  By all threads of the CTA, one to a t-line.  rows (4 n words): the r-lines (j, k) that are not good in bit
+// k of row j, the small ones of these; the s-lines (i, k) in bit k of row i alike.
+template <int n>
+__device__ __noinline__ bool find_alone(const ll* U, int range, bool act, unsigned (&rows)[4][n], int* alone, int x, int y) {
+  using L = LineLayout<n>;
+  if (act) {
+    *alone = 0;
+    if (y == 0)
+      for (int q = 0; q < 4; ++q) rows[q][x] = 0;
+  }
+  __syncthreads();
+  int t = kGoodLine;
+  if (act) {
+    ll m[3] = {0, 0, 0};
+#pragma unroll 1
+    for (int l = 0; l < n; ++l) {
+      const ll a[3] = {U[L::idx(l, x, y)], U[L::idx(x, l, y)], U[L::idx(x, y, l)]};
+      for (int d = 0; d < 3; ++d) m[d] |= a[d] ^ (a[d] >> 63);
+    }
+    int st[3];
+    for (int d = 0; d < 3; ++d) st[d] = line_state(kBits - 64 + __clzll(m[d]), range);
+    for (int d = 0; d < 2; ++d) {
+      if (st[d] != kGoodLine) atomicOr(&rows[2 * d][x], 1u << y);
+      if (st[d] == kSmallLine) atomicOr(&rows[2 * d + 1][x], 1u << y);
+    }
+    t = st[2];
+  }
+  __syncthreads();
+  const bool a = t != kGoodLine && (rows[0][y] & rows[2][x] & (t == kSmallLine ? ~0u : rows[1][y] | rows[3][x])) != 0;
+  if (a) *alone = 1;
+  return a;
+}
+
+// The elements that the integer path does not cover, in FP64 (Alg. 1), by all threads of the CTA: those with `on`
+// evaluate the t-line (x, y) of element e from v into P.w and return its part of <v, A_L v>.  U: the element's shared
+// memory (three arrays).  FP64 multiply-adds bound it (1.7 per clock and SM), so the loops are left rolled.
+template <int N>
+__device__ __noinline__ double element_fp64(const AxParams<double>& P, const double* v, int64_t e, int x, int y, bool on,
+                                            double* U) {
+  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
+  using L = LineLayout<n>;
+  double *R = U + L::size, *S = R + L::size;
+  const int line = x + n * y;
+  const int64_t base = e * n3 + line;
+  double pw = 0.0;
+  __syncthreads();
+  if (on)
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) U[L::idx(x, y, k)] = v[base + k * n2];
+  __syncthreads();
+  if (on) {
+    const int s = P.fx.sG[e].x;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      double ur = 0.0, us = 0.0, ut = 0.0;
+#pragma unroll 1
+      for (int l = 0; l < n; ++l) {
+        ur += P.D[x * n + l] * U[L::idx(l, y, k)];
+        us += P.D[y * n + l] * U[L::idx(x, l, k)];
+        ut += P.D[k * n + l] * U[L::idx(x, y, l)];
+      }
+      const double w3 = P.fx.wq[x] * P.fx.wq[y] * P.fx.wq[k];
+      double g[6];
+#pragma unroll
+      for (int f = 0; f < 3; ++f) {
+        const int4 c = P.fx.G[(e * 3 + f) * n3 + line + k * n2];
+        g[2 * f] = ldexp(__ll2double_rn(shl(c.y, 32) + c.x), -s) * w3;
+        g[2 * f + 1] = ldexp(__ll2double_rn(shl(c.w, 32) + c.z), -s) * w3;
+      }
+      R[L::idx(x, y, k)] = g[0] * ur + g[3] * us + g[4] * ut;
+      S[L::idx(x, y, k)] = g[3] * ur + g[1] * us + g[5] * ut;
+      P.w[base + k * n2] = g[4] * ur + g[5] * us + g[2] * ut;  // until u has been read
+    }
+  }
+  __syncthreads();
+  if (on)
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) U[L::idx(x, y, k)] = P.w[base + k * n2];
+  __syncthreads();
+  if (on)
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {
+      double w = 0.0;
+#pragma unroll 1
+      for (int l = 0; l < n; ++l)
+        w += P.D[l * n + x] * R[L::idx(l, y, k)] + P.D[l * n + y] * S[L::idx(x, l, k)] + P.D[l * n + k] * U[L::idx(x, y, l)];
+      w *= P.h1;
+      if (P.helm) w += P.h2 * P.B[base + k * n2] * v[base + k * n2];
+      P.w[base + k * n2] = w;
+      pw += v[base + k * n2] * w;
+    }
+  return pw;
+}
+
 // Arrays of an element in shared memory: u, then the r- and s-lines' values, and for n >= 10 the t-line's while the
 // thread works on the other two (24 registers at n = 12).
 __host__ __device__ constexpr int line_arrays(int N) { return N >= 9 ? 4 : 3; }
@@ -129,6 +225,9 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
   __shared__ int sdone;
   using Max = ElemMax<n2, EPB>;
   __shared__ int smax[3][Max::size];
+  __shared__ unsigned srow[EPB][4][n];  // find_alone
+  __shared__ int alone[EPB];            // a point without a good line
+  __shared__ int slook, sfp64;          // in the CTA: a t-line that may not be good; elements in FP64
 
   const int tid = threadIdx.x;
   if (FUSED) {
@@ -145,6 +244,10 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(P.fx.B + e0 * n3), "r"(bytes / 6) : "memory");
   }
   for (int q = 0; q < 3; ++q) Max::clear(smax[q]);
+  if (tid == 0) {
+    slook = 0;
+    sfp64 = P.fx.direct;
+  }
   if (!Max::whole) __syncthreads();
 
   const int le = min(tid / n2, EPB - 1), line = tid - le * n2, x = line % n, y = line / n;
@@ -180,8 +283,13 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     for (int k = 0; k < n; ++k) ehi = max(ehi, __double2hiint(v[k]) & 0x7fffffff);
     Max::put(smax[0], le, ehi);
     __syncthreads();
+    const int lhi = ehi;
     ehi = Max::get(smax[0], le);
     if (ehi == 0) ehi = 1023 << 20;  // an element of zeros
+    if (act) {
+      if (expo(ehi) - expo(lhi) + P.fx.range > kLineBits) slook = 1;
+      if (expo(ehi) < kExpMin || expo(ehi) > kExpMax) sfp64 = 1;
+    }
     if (act) {
       ll u[n];
 #pragma unroll
@@ -198,9 +306,11 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     if (act) m |= mag(wt[k]);
     if (park && act) T[L::idx(x, y, k)] = wt[k];
   }
-  const int sG = act ? P.fx.sG[e] : 0;
-  const bool slow = P.fx.direct || expo(ehi) < kExpMin || expo(ehi) > kExpMax;
+  const int sG = act ? P.fx.sG[e].x : 0;
   __syncthreads();
+  if (slook) {  // the same for the whole CTA
+    if (find_alone<n>(U, act ? P.fx.sG[e].y : 0, act, srow[le], alone + le, x, y)) sfp64 = 1;
+  }
 
   if (act) {
     ll v[n], g[n];
@@ -287,14 +397,18 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
   __syncthreads();
 
   double pw = 0.0;  // this thread's part of <p, A_L p>
-  if (act && !slow) {
+  const bool fp64 = sfp64 && (P.fx.direct || (slook && alone[le]) || expo(ehi) < kExpMin || expo(ehi) > kExpMax);
+  if (act && !fp64) {
     const int eu = expo(ehi) - 1022 - kBits;    // u = value 2^eu
     int eo = eu + Q.scale - sG - s1 - up;       // the unit of a point's sum, without its weights
     MassTerm mt{Q.h2, 0};
-    if (P.helm) {
-      const int em = eu + 63 + Q.e2 - P.fx.sB[e];
+    bool helm = P.helm, mass64 = false;
+    if (helm) {
+      const int sB = P.fx.sB[e], em = eu + 63 + Q.e2 - sB;
+      mass64 = sG - sB > Q.mass_limit;
+      helm = !mass64;
       mt.down = eo - em;
-      eo = max(eo, em);
+      if (helm) eo = max(eo, em);
     }
     if (FUSED) eo += 64 - P.fx.tw[line];
     // The weights: in FP64, whose pipe is idle, or for <p, A p> in integers, o W kept to 2^(64 - wb): |o| < 3 g 2^60 + 2^59
@@ -306,7 +420,7 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     for (int k = 0; k < n; ++k) {
       const int at = L::idx(x, y, k);
       ll o = wt[k] + R[at] + S[at];
-      if (P.helm) o = mt.add(o, B[k], split(U[at]));
+      if (helm) o = mt.add(o, B[k], split(U[at]));
       if (!FUSED) {
         P.w[base + k * n2] = to_double(o, eo) * __ldg(P.fx.W64 + line + k * n2);
       } else {
@@ -321,14 +435,20 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
     }
     // the lines' sums cancel in <p, A p> (smooth p: to 1e-4 of them and less), so their low halves count
     if (FUSED) pw = ldexp(fma(__ll2double_rn(pm), 0x1p-32, __ll2double_rn(ph)), 64 + 2 + eo + eu);
-  } else if (act) {
-    const double* v = FUSED ? (P.pout ? P.pout : P.p) : P.u;
+    if (mass64) {
+      const double* v = FUSED ? (P.pout ? P.pout : P.p) : P.u;
 #pragma unroll 1
-    for (int k = 0; k < n; ++k) {
-      const double r = slow_point<N>(P, v, e, x, y, k);
-      P.w[base + k * n2] = r;
-      if (FUSED) pw += v[base + k * n2] * r;
+      for (int k = 0; k < n; ++k) {
+        const double u = v[base + k * n2], t = P.h2 * P.B[base + k * n2] * u;
+        P.w[base + k * n2] += t;
+        if (FUSED) pw += u * t;
+      }
     }
+  }
+  if (sfp64) {  // the same for the whole CTA
+    const double r = element_fp64<N>(P, FUSED ? (P.pout ? P.pout : P.p) : P.u, e, x, y, act && fp64,
+                                     reinterpret_cast<double*>(U));
+    if (act && fp64) pw = r;
   }
 
   if (FUSED) {  // this block's part of <p, A_L p>; k_pap_finish sums the parts in block order
@@ -393,11 +513,11 @@ cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out
   if (grid_out) *grid_out = (int)grid;
   if (p.E == 0) return cudaSuccess;
   static const LineTable<N> plain = line_table<N>();
-  LineParams<N> q{p, fx_scale(N).scale, make_int2(0, 0), 0, plain};
+  LineParams<N> q{p, fx_scale(N).scale, make_int2(0, 0), 0, 0, plain};
+  int e1 = 0;  // exponent of h1
   if (p.helm && !p.fx.direct)
     q.h2 = split(std::llround(std::ldexp(std::frexp((long double)p.h2 / fx_scale(N).kappa, &q.e2), 62)));
   if (p.h1 != 1.0 && !p.fx.direct) {
-    int e1 = 0;
     const long long mant = (long long)std::ldexp(std::frexp(p.h1, &e1), 53);
     // The plain tables keep the sums below 0.8 2^63; a mantissa gives the entries any low halves, and then the sums of
     // N >= 9 can pass 2^63 (at worst 1.15 2^63 at N = 11, where about 4 mantissas in 10,000 allow it).  Half the mantissa
@@ -405,10 +525,16 @@ cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out
     for (int shift = 53; shift <= 54; ++shift) {
       scale_table(plain.e, q.d.e, mant, shift);
       scale_table(plain.o, q.d.o, mant, shift);
+      q.scale = fx_scale(N).scale + e1 + shift - 53;
       if (sums_fit(q.d.e) && sums_fit(q.d.o)) break;
-      ++e1;
     }
-    q.scale += p.h1 == 0.0 ? 0 : e1;
+  }
+  // The mass term of a point where u is small is rounded like the element's largest; FP64 rounds it with the stiffness
+  // terms of the point's lines.  It is left in fixed point up to 2^4 times the bound of those, 2 D_00^2 h1 G: beyond that
+  // (h1 = 0 among them) the mass is most of the result.
+  if (p.helm) {
+    constexpr int d00 = N * n / 4 < 2 ? 0 : N * n / 4 < 4 ? 2 : N * n / 4 < 8 ? 4 : N * n / 4 < 16 ? 6 : N * n / 4 < 32 ? 8 : 10;
+    q.mass_limit = p.h1 == 0.0 ? -100000 : e1 + d00 + 1 + 4 - q.e2;
   }
   k_ax_fx<N, EPB, FUSED><<<(unsigned)grid, line_threads(N, EPB), smem, s>>>(q);
   cudaError_t err = cudaGetLastError();

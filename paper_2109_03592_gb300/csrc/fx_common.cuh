@@ -11,6 +11,21 @@ using namespace fx;
 
 constexpr int kExpMin = 1023 - 500, kExpMax = 1023 + 500;  // biased exponents of u on the integer path
 
+// The values of an element share one exponent, FP64's do not: an element whose small values stand alone is evaluated in
+// FP64.  w at a point is a sum over the three lines through it, so a small value does no harm where one of its lines has
+// a larger one; a line is
+//   good   its largest value lies at most kLineBits below the element's (less the factors' own range, FxOp::sG),
+//   zero   all its values are zero or more than kNoiseBits below (the rounding of zeros such as sin(pi)),
+//   small  otherwise,
+// and the element is taken in FP64 if a point has small lines and no good one.  The integer path's error is then at most
+// 2^(kLineBits - 7) of FP64's bound, which is reached at such points alone.  Emulated: no element of CG directions of
+// smooth right-hand sides is, at any order; a Gaussian of 0.5 element widths has a quarter of its elements taken.
+constexpr int kLineBits = 12, kNoiseBits = 44;
+enum { kZeroLine, kSmallLine, kGoodLine };
+__device__ __forceinline__ int line_state(int below, int range) {  // below: bits below the element's largest
+  return below + range <= kLineBits ? kGoodLine : below > kNoiseBits ? kZeroLine : kSmallLine;
+}
+
 // Maximum of v over an element's threads.  put() by every thread of the CTA, which is whole warps (so all 32 lanes meet
 // in its warp operations, also behind a branch that some of them took), a barrier, then get(); `s` is one of the CTA's
 // arrays, used once.  Where an element is whole warps each warp has a word of its own;
@@ -45,42 +60,6 @@ struct ElemMax {
     return v;
   }
 };
-
-// w at one point of an element in FP64, straight from memory (Alg. 1, with the factors taken back from their
-// fixed-point form): for the rare element that the integer path does not cover.
-template <int N>
-__device__ __forceinline__ double slow_point(const AxParams<double>& P, const double* v, int64_t e, int i, int j, int k) {
-  constexpr int n = N + 1, n2 = n * n, n3 = n2 * n;
-  const double* ue = v + e * n3;
-  const int sG = P.fx.sG[e];
-  auto G = [&](int f, int a, int b, int c) {
-    const int4 x = P.fx.G[(e * 3 + (f >> 1)) * n3 + a + n * b + n2 * c];
-    const int2 y = (f & 1) ? make_int2(x.z, x.w) : make_int2(x.x, x.y);
-    return ldexp(__ll2double_rn(shl(y.y, 32) + y.x), -sG) * (P.fx.wq[a] * P.fx.wq[b] * P.fx.wq[c]);
-  };
-  double out = 0.0;
-#pragma unroll 1
-  for (int d = 0; d < 3; ++d) {
-#pragma unroll 1
-    for (int l = 0; l < n; ++l) {
-      const int a = d == 0 ? l : i, b = d == 1 ? l : j, c = d == 2 ? l : k;
-      double ur = 0.0, us = 0.0, ut = 0.0;
-#pragma unroll 1
-      for (int q = 0; q < n; ++q) {
-        ur += P.D[a * n + q] * ue[q + n * b + n2 * c];
-        us += P.D[b * n + q] * ue[a + n * q + n2 * c];
-        ut += P.D[c * n + q] * ue[a + n * b + n2 * q];
-      }
-      const int f0 = d == 0 ? 0 : d == 1 ? 3 : 4, f1 = d == 0 ? 3 : d == 1 ? 1 : 5, f2 = d == 0 ? 4 : d == 1 ? 5 : 2;
-      const double w = G(f0, a, b, c) * ur + G(f1, a, b, c) * us + G(f2, a, b, c) * ut;
-      out += P.D[l * n + (d == 0 ? i : d == 1 ? j : k)] * w;
-    }
-  }
-  out *= P.h1;
-  const int p = i + n * j + n2 * k;
-  if (P.helm) out += P.h2 * P.B[e * n3 + p] * ue[p];
-  return out;
-}
 
 // h2 B u of a point onto the stiffness part, both without the quadrature weights, in the coarser of the two terms' units.
 // B has 62 bits below the element's largest, h2's mantissa (over kappa) 62, u 60; their product is taken to 59 bits.

@@ -194,21 +194,28 @@ __global__ void k_weights(const uint8_t* __restrict__ wm, double* mult, double* 
 }
 
 // The fixed-point factors of the FP64 operator (FxOp): one CTA per element,
-// first the element's largest exponents of G and B, then the integers.  62
-// bits for G: with fields of 60 bits the three terms of a point's product
-// meet the bound of fx::dot.
+// first the element's largest exponents of G and B and the range of G over its
+// lines, then the integers.  62 bits for G: with fields of 60 bits the three
+// terms of a point's product meet the bound of fx::dot, and factors up to
+// kMaxRange below the largest keep FP64's bits.
+constexpr int kMaxRange = 9;
 __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B, int n,
-                                                 int64_t E, int4* __restrict__ fG, int* __restrict__ sG,
+                                                 int64_t E, int4* __restrict__ fG, int2* __restrict__ sG,
                                                  int2* __restrict__ fB, int* __restrict__ sB, int* bad) {
-  __shared__ int top[2];
-  const int n3 = n * n * n;
+  __shared__ int top[3];
+  __shared__ short point[12 * 12 * 12];
+  const int n2 = n * n, n3 = n2 * n;
   const int64_t e = blockIdx.x;
-  if (threadIdx.x < 2) top[threadIdx.x] = 0;
+  if (threadIdx.x < 3) top[threadIdx.x] = 0;
   __syncthreads();
   int mG = 0, mB = 0;
   for (int p = threadIdx.x; p < n3; p += blockDim.x) {
-    if (G)
-      for (int f = 0; f < 6; ++f) mG = max(mG, __double2hiint(G[(e * 6 + f) * n3 + p]) & 0x7fffffff);
+    if (G) {
+      int hi = 0;
+      for (int f = 0; f < 6; ++f) hi = max(hi, __double2hiint(G[(e * 6 + f) * n3 + p]) & 0x7fffffff);
+      point[p] = (short)fx::expo(hi);
+      mG = max(mG, hi);
+    }
     if (B) mB = max(mB, __double2hiint(B[e * n3 + p]) & 0x7fffffff);
   }
   atomicMax(&top[0], mG);
@@ -216,9 +223,22 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
   __syncthreads();
   // an all-zero B (h2 = 0 at every point of the element) is in range
   const int tG = fx::expo(top[0]), tB = top[1] ? fx::expo(top[1]) : 1023;
+  if (G)
+    for (int q = threadIdx.x; q < 3 * n2; q += blockDim.x) {
+      const int d = q / n2, a = q % n2 % n, b = q % n2 / n;
+      const int first = d == 0 ? n * a + n2 * b : d == 1 ? a + n2 * b : a + n * b, step = d == 0 ? 1 : d == 1 ? n : n2;
+      int line = 0;
+      for (int l = 0; l < n; ++l) line = max(line, (int)point[first + l * step]);
+      atomicMax(&top[2], tG - line);
+    }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    if ((G && abs(tG - 1023) > fx::kOpExp) || (B && abs(tB - 1023) > fx::kOpExp)) atomicExch(bad, 1);
-    if (G) sG[e] = 62 + 1022 - tG;
+    if ((G && (abs(tG - 1023) > fx::kOpExp || top[2] > kMaxRange)) || (B && abs(tB - 1023) > fx::kOpExp))
+      atomicExch(bad, 1);
+    if (G) {
+      sG[e] = make_int2(62 + 1022 - tG, top[2]);
+      if (top[2]) atomicMax(bad + 1, top[2]);
+    }
     if (B) sB[e] = 62 + 1022 - tB;
   }
   if (B)
@@ -234,7 +254,7 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
 
 // ---- launchers ---------------------------------------------------------------
 
-cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int* sG, int2* fB, int* sB,
+cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int2* sG, int2* fB, int* sB,
                            int* bad, cudaStream_t s) {
   if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, n, E, fG, sG, fB, sB, bad);
   return cudaGetLastError();

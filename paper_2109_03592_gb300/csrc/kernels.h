@@ -22,9 +22,9 @@ void launch_coords_pipe(double* xyz, const double* xi, const double* tlev, int n
 // w: the quadrature weights, or ones; G, B and bad may be null
 cudaError_t launch_geometry(const double* xyz, double* G, double* B, const double* D, const double* w, int n,
                             int64_t E, int* bad, cudaStream_t s);
-// FxOp's G and sG from G (not null), its B and sB from B (not null), both made with weights of 1; *bad is set if an
-// element's exponents are out of range.
-cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int* sG, int2* fB, int* sB,
+// FxOp's G and sG from G (not null), its B and sB from B (not null), both made with weights of 1; bad[0] is set if an
+// element's exponents are out of range, bad[1] is the largest sG[].y.
+cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int2* sG, int2* fB, int* sB,
                            int* bad, cudaStream_t s);
 void launch_local_diag(const double* G, double* dK, const double* D, int n, int64_t E, cudaStream_t s);
 void launch_fold_coef(const double* G, const double* B, const double* h1, const double* h2, double* cG, double* cB,
@@ -36,14 +36,15 @@ void launch_weights(const uint8_t* wm, double* mult, double* mask, int64_t m, cu
 // Data of the fixed-point FP64 operator (ax_fx_impl.cuh); G null: not available.
 struct FxOp {
   const int4* G = nullptr;    // [E][3][n^3]: factors (2f, 2f + 1) of a point without the quadrature weights, times 2^sG
-  const int* sG = nullptr;    // [E]
+  const int2* sG = nullptr;   // [E]: sG; the bits from the element's largest factor to the least of its lines' largest
   const int2* B = nullptr;    // [E][n^3]: the mass without them, times 2^sB (both: 62 bits below the element's largest)
   const int* sB = nullptr;    // [E]
   const int2* W = nullptr;    // [n^3]: w_i w_j w_k kappa 2^tw (fx_weights)
   const int* tw = nullptr;    // [n^2]: tw of the t-line (i, j)
   const double* W64 = nullptr; // [n^3]: w_i w_j w_k kappa
   const double* wq = nullptr; // [n]: the weights
-  int direct = 0;             // h1 or h2 outside the exponent range of the integer path
+  int range = 0;              // the largest sG[].y
+  int direct = 0;             // every element in FP64: h1 or h2 outside the exponent range of the integer path
 };
 
 struct NoOp {};

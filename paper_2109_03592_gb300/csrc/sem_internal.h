@@ -112,7 +112,8 @@ struct sem_mesh {
   float* B32 = nullptr;      // [E][n3] round-to-nearest of B64
   float* B32lo = nullptr;    // [E][n3] float(B64 - B32) (double-float only)
   int4* Gfx = nullptr;       // [E][3 n3] the factors in fixed point (FxOp); null where their exponents are out of range
-  int* fx_sG = nullptr;      // [E] FxOp::sG
+  int2* fx_sG = nullptr;     // [E] FxOp::sG
+  int fx_range = 0;          // FxOp::range
   int2* Bfx = nullptr;       // [E][n3] FxOp::B
   int* fx_sB = nullptr;      // [E] FxOp::sB
   int2* fx_W = nullptr;      // [n3] FxOp::W
@@ -145,7 +146,8 @@ struct sem_mesh {
   float* cG32 = nullptr;
   float* cG32lo = nullptr;
   int4* cGfx = nullptr;
-  int* cfx_sG = nullptr;
+  int2* cfx_sG = nullptr;
+  int cfx_range = 0;
   double* cdK = nullptr;
   double* cB64 = nullptr;
   float* cB32 = nullptr;
@@ -168,6 +170,7 @@ struct sem_mesh {
     const int2* b = cB64 ? cBfx : Bfx;
     f.G = b ? g : nullptr;
     f.sG = cG32 ? cfx_sG : fx_sG;
+    f.range = cG32 ? cfx_range : fx_range;
     f.B = b;
     f.sB = cB64 ? cfx_sB : fx_sB;
     f.W = fx_W;
