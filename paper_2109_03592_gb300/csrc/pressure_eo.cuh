@@ -8,9 +8,11 @@
 //   A = sum_l E[I][l] P[l], B = sum_l O[I][l] M[l],  E, O = (X[I][l] +- X[I][l']) / 2,
 //   (Ig v)[I], (Ig v)[I'] = A +- B;   (Dg v)[I], (Dg v)[I'] = B +- A
 // (a middle point, where n or m is odd, has a P of its own and no M), and the
-// transposes alike: half the multiply-adds of the plain form.  (The FP32 gradient's j-
-// and k-stages use the plain form: they are not what bounds it, and the folds' roundings
-// would put its error 10% above the plain form's; as it is E's is 3% below.)  E and O are kernel
+// transposes alike: half the multiply-adds of the plain form.  FP32 uses the plain form
+// where the folds' roundings would put the error above its own: in the gradient's j- and
+// k-stages (not what bounds it; E's error is then 8 to 18% below the plain form's on random
+// elements) and everywhere for N <= 4 and N = 6 (E's error with folds 13 to 33% above at N = 3,
+// 3 to 27% at N = 4, up to 4% at N = 6).  E and O are kernel
 // parameters and every loop over them is unrolled, so they come from constant
 // memory as operands of the multiply-adds; shared memory only carries the lines
 // from one direction to the next.
@@ -98,6 +100,7 @@ template <class A, int N>
 struct Shape {
   static constexpr int n = N + 1, m = N - 1, n2 = n * n, n3 = n2 * n, m2 = m * m, m3 = m2 * m;
   static constexpr int np = (n + 1) / 2, nm = n / 2, mp = (m + 1) / 2, mm = m / 2;  // P and M values of a line
+  static constexpr bool plain = !A::fixed && (N <= 4 || N == 6);
   static constexpr int banks = 128 / (int)sizeof(typename A::V);
   // [K][j][i]: planes padded so that the threads (K, i) of the j-stage meet distinct banks
   static constexpr int sX = n2 + ((n - n2) % banks + banks) % banks;
@@ -196,6 +199,22 @@ __device__ __forceinline__ ll dot2(const int2 (&c)[K], const int2 (&v)[K], int n
   for (int l = 0; l < L; ++l)
     if (l < nd) r = r + (ll)d[l].y * w[l].y;
   return r;
+}
+
+// A row of the matrix times a line, and a column of it: the plain form (FP32).
+template <int L>
+__device__ __forceinline__ float row(const float (&x)[L], const float (&v)[L]) {
+  float s = 0.f;
+#pragma unroll
+  for (int l = 0; l < L; ++l) s = fmaf(x[l], v[l], s);
+  return s;
+}
+template <int M, int L>
+__device__ __forceinline__ float column(const float (&x)[M][L], int l, const float (&v)[M]) {
+  float s = 0.f;
+#pragma unroll
+  for (int r = 0; r < M; ++r) s = fmaf(x[r][l], v[r], s);
+  return s;
 }
 
 template <class A, int L>
@@ -392,9 +411,16 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
 #pragma unroll
         for (int k = 0; k < n; ++k) v[k] = raw[k];
       }
+      V* x = XD(le1) + ji;
+      if constexpr (S::plain) {
+#pragma unroll
+        for (int I = 0; I < m; ++I) {
+          x[I * S::sX] = row(P.dg.x[I], v);
+          x[(m + I) * S::sX] = row(P.ig.x[I], v);
+        }
+      } else {
       C p[S::np], q[imax(S::nm, 1)];
       fold<A, n>(v, p, q);
-      V* x = XD(le1) + ji;
 #pragma unroll
       for (int I = 0; I < S::mp; ++I) {
         const V dA = dot<A>(P.dg.e[I], p, S::np), dB = dot<A>(P.dg.o[I], q, S::nm), iA = dot<A>(P.ig.e[I], p, S::np), iB = dot<A>(P.ig.o[I], q, S::nm);
@@ -405,11 +431,24 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
           x[(2 * m - 1 - I) * S::sX] = iA - iB;
         }
       }
+      }
     }
     if (a < 2) load(a + 1);
     __syncthreads();
     if (a2) {
       const V* x = XD(le2) + K2 * S::sX + i2;
+      V* y = Y0(le2) + K2 * S::sY + i2;
+      if constexpr (S::plain) {
+        V d[n], v[n];
+        load_line<A, n>(x, n, d);
+        load_line<A, n>(x + m * S::sX, n, v);
+#pragma unroll
+        for (int J = 0; J < m; ++J) {
+          y[J * S::rY] = row(P.ig.x[J], d);
+          y[m * S::sY + J * S::rY] = row(P.dg.x[J], v);
+          y[2 * m * S::sY + J * S::rY] = row(P.ig.x[J], v);
+        }
+      } else {
       C pd[S::np], qd[imax(S::nm, 1)], pi[S::np], qi[imax(S::nm, 1)];
       {
         V v[n];
@@ -418,7 +457,6 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
         load_line<A, n>(x + m * S::sX, n, v);
         fold<A, n>(v, pi, qi);
       }
-      V* y = Y0(le2) + K2 * S::sY + i2;
 #pragma unroll
       for (int J = 0; J < S::mp; ++J) {
         const V A0 = dot<A>(P.ig.e[J], pd, S::np), B0 = dot<A>(P.ig.o[J], qd, S::nm);
@@ -433,11 +471,23 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
           y[2 * m * S::sY + (m - 1 - J) * S::rY] = A2 - B2;
         }
       }
+      }
     }
     if (a < 2) put_max(a + 1);
     __syncthreads();
     if (a3) {
       const V* y = Y0(le3) + KJ * S::rY;
+      const C* F = P.F + ((e0 + le3) * 3 + a) * 3 * m3 + KJ;
+      if constexpr (S::plain) {
+        V v[3][n];  // along r, s, t
+#pragma unroll
+        for (int b = 0; b < 3; ++b) load_line<A, n>(y + (2 - b) * m * S::sY, 1, v[b]);
+#pragma unroll
+        for (int I = 0; I < m; ++I)
+          o[I] = fmaf(__ldg(F + 3 * I * m2), row(P.dg.x[I], v[0]),
+                      fmaf(__ldg(F + (3 * I + 1) * m2), row(P.ig.x[I], v[1]),
+                           fmaf(__ldg(F + (3 * I + 2) * m2), row(P.ig.x[I], v[2]), o[I])));
+      } else {
       C p[3][S::np], q[3][imax(S::nm, 1)];
 #pragma unroll
       for (int b = 0; b < 3; ++b) {  // Y2, Y1, Y0: along r, s, t
@@ -445,7 +495,6 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
         load_line<A, n>(y + (2 - b) * m * S::sY, 1, v);
         fold<A, n>(v, p[b], q[b]);
       }
-      const C* F = P.F + ((e0 + le3) * 3 + a) * 3 * m3 + KJ;
       int ex = 0;
       if constexpr (A::fixed) {
         const int ev = element_expo(Max::get(smax[a], le3));
@@ -496,6 +545,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
             o[q_] = fmaf(f0, g0, fmaf(f1, g1, fmaf(f2, g2, o[q_])));
           }
         }
+      }
       }
     }
   }
@@ -582,6 +632,20 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
   for (int a = 0; a < 3; ++a) {
     if (a1) {  // along I -> i: S0 = Dg^T t0, S1 = Ig^T t1, S2 = Ig^T t2, t_b = F[b][a] p
       const C* F = P.F + ((e0 + le1) * 3 + a) * 3 * m3 + KJ;
+      V* s = S0(le1) + KJ * S::rY;
+      if constexpr (S::plain) {
+        V t[3][m];
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+#pragma unroll
+          for (int I = 0; I < m; ++I) t[b][I] = A::factor(__ldg(F + (3 * I + b) * m2), pc[I]);
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+          s[i] = column(P.dg.x, i, t[0]);
+          s[m * S::sY + i] = column(P.ig.x, i, t[1]);
+          s[2 * m * S::sY + i] = column(P.ig.x, i, t[2]);
+        }
+      } else {
       C p[3][S::mp], q[3][imax(S::mm, 1)];
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
@@ -590,7 +654,6 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
         for (int I = 0; I < m; ++I) t[I] = A::factor(__ldg(F + (3 * I + b) * m2), pc[I]);
         fold<A, m>(t, p[b], q[b]);
       }
-      V* s = S0(le1) + KJ * S::rY;
 #pragma unroll
       for (int i = 0; i < S::np; ++i) {
         const V A0 = dot<A>(P.dg.te[i], p[0], S::mp), B0 = dot<A>(P.dg.to[i], q[0], S::mm);
@@ -604,6 +667,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
           s[m * S::sY + n - 1 - i] = A1 - B1;
           s[2 * m * S::sY + n - 1 - i] = A2 - B2;
         }
+      }
       }
     }
     __syncthreads();
