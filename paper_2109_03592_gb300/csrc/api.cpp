@@ -95,6 +95,7 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->DIgl);
   dev_free(m->Ffx);
   dev_free(m->Ffx_s);
+  dev_free(m->pW);
   dev_free(m->invB);
   dev_free(m->Fgl32);
   dev_free(m->invB32);

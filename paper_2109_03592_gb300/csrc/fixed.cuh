@@ -79,24 +79,12 @@ __device__ __forceinline__ double to_double(ll v, int e) {
 }
 
 __device__ __forceinline__ ll shl(ll v, int s) { return (ll)((unsigned long long)v << s); }
-// v 2^s for any s (arithmetic shift right for s < 0)
-__device__ __forceinline__ ll shift(ll v, int s) { return s >= 0 ? shl(v, min(s, 63)) : v >> min(-s, 63); }
 // bits that hold |hi word| of the largest value seen by `m` (m collects hi ^ (hi >> 31))
 __device__ __forceinline__ int mag(ll v) {
   const int h = (int)(v >> 32);
   return h ^ (h >> 31);
 }
 __device__ __forceinline__ int bits_of(int m) { return 64 - __clz(m); }
-
-// A factor as 64-bit integer: |f| K / 2^64 of its 63-bit mantissa, shifted to 62 bits below 2^(top - 1022), with the sign
-// (K / 2^63 in [1, 2]); f kappa = result 2^(top - 1083).
-__device__ __forceinline__ ll scaled_factor(double f, unsigned long long K, int top) {
-  const int hi = __double2hiint(f), d = top - expo(hi);
-  const unsigned long long x =
-      ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(f)) << 10;
-  const ll v = d > 61 || expo(hi) == 0 ? 0 : (ll)(__umul64hi(x, K) >> (d + 1));
-  return hi < 0 ? -v : v;
-}
 #endif
 
 }  // namespace fx

@@ -185,12 +185,13 @@ cudaError_t launch_gl_factors(const double* xyz, const double* Ig, const double*
 // What the weak gradient and divergence read (pressure_eo.cuh).  FP64: the factors in fixed point (Ffx, sF; direct: out
 // of its range) and the plain data for the elements that are evaluated in FP64; FP32: F32, in the same order.
 struct PressureOp {
-  const double *F, *Ig, *DIg, *invB;
+  const double *F, *Ig, *DIg, *invB, *Wgrad, *Wdiv;
   const int2* Ffx;
   const int* sF;
   int direct;
   const float *F32, *invB32;
 };
+// Ffx and sF from F made with weights of 1
 cudaError_t launch_pressure_pack(const double* F, int N, int64_t E, int2* Ffx, int* sF, int* bad, cudaStream_t s);
 cudaError_t launch_pressure_pack32(const double* F, int N, int64_t E, float* F32, cudaStream_t s);
 void launch_recip(const double* a, double* out, int64_t n, cudaStream_t s);

@@ -21,7 +21,7 @@ namespace sem {
 
 // The same quantities as gl_matrices below in long double: the GLL and GL points by Newton (from the FP64 GLL
 // points and from cos(pi (i + 3/4) / (m + 1/2))), made symmetric, and the basis by its products.
-void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double>& DIg) {
+void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double>& DIg, std::vector<long double>& rho) {
   typedef long double ld;
   const int n = N + 1, m = N - 1;
   auto legendre = [](int k, ld x, ld& pk, ld& pk1) {  // P_k and P_{k-1}, k >= 1
@@ -53,6 +53,12 @@ void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double
     if (k & 1) v[k / 2] = 0;
   };
   symmetric(z);
+  rho.resize(m);
+  for (int i = 0; i < m; ++i) {  // 2 / ((1 - z^2) P_m'(z)^2)
+    legendre(m, z[i], p, q);
+    const ld d = m * (q - z[i] * p);
+    rho[i] = 2 * (1 - z[i] * z[i]) / (d * d);
+  }
   Ig.assign((size_t)m * n, 0);
   DIg.assign((size_t)m * n, 0);
   for (int i = 0; i < m; ++i)
@@ -161,7 +167,7 @@ void gl_matrices(int N, std::vector<double>& Ig, std::vector<double>& DIg, std::
 }
 
 PressureOp pressure_op(const sem_mesh* m) {
-  return {m->Fgl, m->Igl, m->DIgl, m->invB, m->Ffx, m->Ffx_s, m->Ffx_direct, m->Fgl32, m->invB32};
+  return {m->Fgl, m->Igl, m->DIgl, m->invB, m->pW, m->pW + (size_t)m->n * m->n * m->n, m->Ffx, m->Ffx_s, m->Ffx_direct, m->Fgl32, m->invB32};
 }
 
 #define SEM_TRY_STATUS(expr)          \
@@ -191,7 +197,7 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   const int64_t m3 = (int64_t)mm * mm * mm;
   std::vector<double> Ig, DIg, rho;
   gl_matrices(N, Ig, DIg, rho);
-  double *F = nullptr, *I_d = nullptr, *DI_d = nullptr, *rho_d = nullptr, *iB = nullptr;
+  double *F = nullptr, *I_d = nullptr, *DI_d = nullptr, *rho_d = nullptr, *iB = nullptr, *pW = nullptr;
   int2* Ffx = nullptr;
   int *sF = nullptr, *bad_d = nullptr;  // bad: det(J) <= 0; factors out of the fixed-point form's range
   auto release = [&]() {
@@ -200,6 +206,7 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
     if (DI_d) cudaFree(DI_d);
     if (rho_d) cudaFree(rho_d);
     if (iB) cudaFree(iB);
+    if (pW) cudaFree(pW);
     if (Ffx) cudaFree(Ffx);
     if (sF) cudaFree(sF);
     if (bad_d) cudaFree(bad_d);
@@ -213,7 +220,12 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   if ((e = cudaMalloc((void**)&F, sizeof(double) * 9 * m3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&I_d, sizeof(double) * mm * n)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&DI_d, sizeof(double) * mm * n)) != cudaSuccess) return fail(e, "cudaMalloc");
-  if ((e = cudaMalloc((void**)&rho_d, sizeof(double) * mm)) != cudaSuccess) return fail(e, "cudaMalloc");
+  std::vector<double> W, Wdiv;
+  pressure_weights(N, W, Wdiv);
+  W.insert(W.end(), Wdiv.begin(), Wdiv.end());
+  rho.resize(2 * mm, 1.0);  // rho, then ones
+  if ((e = cudaMalloc((void**)&rho_d, sizeof(double) * 2 * mm)) != cudaSuccess) return fail(e, "cudaMalloc");
+  if ((e = cudaMalloc((void**)&pW, sizeof(double) * W.size())) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&bad_d, 2 * sizeof(int))) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&Ffx, sizeof(int2) * 9 * m3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&sF, sizeof(int) * 3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
@@ -222,14 +234,18 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
     return fail(e, "cudaMemcpyAsync");
   if ((e = cudaMemcpyAsync(DI_d, DIg.data(), sizeof(double) * mm * n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
-  if ((e = cudaMemcpyAsync(rho_d, rho.data(), sizeof(double) * mm, cudaMemcpyHostToDevice, s)) != cudaSuccess)
+  if ((e = cudaMemcpyAsync(rho_d, rho.data(), sizeof(double) * 2 * mm, cudaMemcpyHostToDevice, s)) != cudaSuccess)
+    return fail(e, "cudaMemcpyAsync");
+  if ((e = cudaMemcpyAsync(pW, W.data(), sizeof(double) * W.size(), cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
   if ((e = cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s)) != cudaSuccess) return fail(e, "cudaMemsetAsync");
-  if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
+  if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d + mm, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
     return fail(e, "k_gl_factors");
   if ((e = launch_pressure_pack(F, N, m->E, Ffx, sF, bad_d + 1, s)) != cudaSuccess) return fail(e, "k_pack_fx");
+  if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
+    return fail(e, "k_gl_factors");
   launch_recip(m->dB, iB, m->n_local, s);
-  count_launches(3);
+  count_launches(4);
   int bad[2] = {0, 0};
   if ((e = cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
@@ -244,11 +260,12 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
     return SEM_ERR_BAD_MESH;
   }
   sem_mesh* mut = const_cast<sem_mesh*>(m);
-  mut->dev_bytes += sizeof(double) * (18 * m3 * m->E + 2 * mm * n + m->n_local) + sizeof(int) * 3 * m->E;
+  mut->dev_bytes += sizeof(double) * (18 * m3 * m->E + 2 * mm * n + W.size() + m->n_local) + sizeof(int) * 3 * m->E;
   m->Ffx = Ffx;
   m->Ffx_s = sF;
   m->Ffx_direct = bad[1];
   m->invB = iB;
+  m->pW = pW;
   m->Igl = I_d;
   m->DIgl = DI_d;
   m->Fgl = F;

@@ -27,12 +27,18 @@
 // the i-stage read them: [e][a][I][b][K][J].
 //
 // Fixed point: v and p are brought to 60 bits below the element's (and component's)
-// largest exponent.  Each table is scaled, not by a power of two, so that its largest
-// row sum of magnitudes takes a value of 60 bits to less than 60 bits; the factors
-// carry the inverse of the scales, with 62 bits below the largest of their element
-// and component.  The tables come from long-double GLL and GL points.  Against
-// long-double arithmetic the relative error of E is 1.0e-16 (N = 7, curved pipe, random
-// pressure) where FP64 with FP64 tables' rounding left out has 2.4e-16.
+// largest exponent, and so are lines that go from one stage to the next, for the orders
+// where the stages' bounds, which no smooth or random field comes near, would cost more
+// bits than FP64 loses (Shape).  Each table is scaled, not by a power of two, so that its largest
+// row sum of magnitudes takes a value of 60 bits to less than 60 bits.  The factors are
+// kept without the GL weights rho, with 62 bits below the largest of their element and
+// component; the gradient's tables are W^-1 Ig^T rho and W^-1 Dg^T rho (W: the GLL weights),
+// whose rows are alike in size, and its results are multiplied by the weights at the end,
+// the divergence's by rho (as in ax_fx_impl.cuh, for the same reason); these carry the
+// inverse of the scales.  The tables come from long-double GLL and GL points.  Error of E
+// against 64 bits by emulation, random and smooth pressures on affine elements: 0.2 to 0.9
+// times FP64's; of the gradient at its interior, face, edge and corner points 0.1 to 1.3 times
+// (without the two measures 0.7 to 8 and up to 410 times, N = 5 to 11).
 //
 // What bounds them: fixed point, issue slots (9 in 10 instructions are multiply-adds, 64-bit additions and the
 // splits between them) and the barriers between stages of different width; FP32, shared memory and DRAM (70% and
@@ -101,6 +107,12 @@ struct Shape {
   static constexpr int n = N + 1, m = N - 1, n2 = n * n, n3 = n2 * n, m2 = m * m, m3 = m2 * m;
   static constexpr int np = (n + 1) / 2, nm = n / 2, mp = (m + 1) / 2, mm = m / 2;  // P and M values of a line
   static constexpr bool plain = !A::fixed && (N <= 4 || N == 6);
+  // Fixed point: where lines between stages are brought to 60 bits (gradient: after its first and second stage;
+  // divergence: after its first).  Errors over FP64's by emulation, with and without: gradient's 0.4 to 1.3 and (N = 4)
+  // 1.6 to (N = 10) 17; with one of the two 1.1 at N = 6 and 7, 2 to 3 above.  Divergence's 0.4 (N = 7) without, 1.1 at N = 6,
+  // 1.9 at 8, 3.7 at 10, 1.3 at 11; 0.3 to 0.9 with.
+  static constexpr bool grad_lift1 = A::fixed && N >= 4, grad_lift2 = A::fixed && N >= 6;
+  static constexpr bool div_lift = A::fixed && (N == 6 || N >= 8);
   static constexpr int banks = 128 / (int)sizeof(typename A::V);
   // [K][j][i]: planes padded so that the threads (K, i) of the j-stage meet distinct banks
   static constexpr int sX = n2 + ((n - n2) % banks + banks) % banks;
@@ -141,7 +153,8 @@ struct Params {
   const int* sF;               // fixed point: [E][3], the factors are F 2^sF
   const double *F64, *Ig, *Dg; // for slow_div and slow_grad
   int64_t E, n_local;
-  int scale;                   // fixed point: F C v = 2^scale x the integers' product along the path, over 2^254
+  int scale;                   // fixed point: F C v = 2^scale W x the integers' product along the path, over 2^254
+  const double* W;             // [n^3] (gradient) or [m^3]: the weights and the inverse of the scales
   int direct;                  // fixed point: every element in FP64 (factors out of range)
   Table<typename A::C, N> ig, dg;
 };
@@ -217,6 +230,30 @@ __device__ __forceinline__ float column(const float (&x)[M][L], int l, const flo
   return s;
 }
 
+// The most bits of an element's values, for the T threads of each of EPB elements: put by every thread of the CTA (those
+// beyond the elements with le >= EPB or v = 0) onto a cleared word, a barrier, then lift().
+template <int T, int EPB>
+__device__ __forceinline__ void put_bits(int* s, int le, int v) {
+  if constexpr (T >= 32) {  // a warp meets two elements at most
+    const int first = __shfl_sync(0xffffffffu, le, 0), last = __shfl_sync(0xffffffffu, le, 31);
+    const int a = __reduce_max_sync(0xffffffffu, le == first ? v : 0);
+    const int b = __reduce_max_sync(0xffffffffu, le == first ? 0 : v);
+    if ((threadIdx.x & 31) == 0) {
+      if (first < EPB) atomicMax(s + first, a);
+      if (last != first && last < EPB) atomicMax(s + last, b);
+    }
+  } else if (le < EPB) {
+    atomicMax(s + le, v);
+  }
+}
+// The shift that brings them to 60 bits.
+__device__ __forceinline__ int lift(int bits) { return max(kFieldBits - bits, 0); }
+template <int L>
+__device__ __forceinline__ void lift_line(ll (&v)[L], int s) {
+#pragma unroll
+  for (int l = 0; l < L; ++l) v[l] = fx::shl(v[l], s);
+}
+
 template <class A, int L>
 __device__ __forceinline__ void load_line(const typename A::V* s, int stride, typename A::V (&v)[L]) {
 #pragma unroll
@@ -282,6 +319,12 @@ __device__ __noinline__ void slow_div(const Params<Fixed, N>& P, int64_t e, doub
   }
 }
 
+// The hi words' magnitudes of a stage's results, for put_bits; nothing in FP32.
+template <class... V>
+__device__ __forceinline__ void note(int& mg, V... v) {
+  if constexpr ((std::is_same<V, ll>::value && ...)) ((mg |= fx::mag(v)), ...);
+}
+
 template <int N>
 __device__ __noinline__ void slow_grad(const Params<Fixed, N>& P, int64_t e, double* sm) {
   constexpr int n = N + 1, m = N - 1, n2 = n * n, n3 = n2 * n, m2 = m * m, m3 = m2 * m;
@@ -345,6 +388,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
   V* sm = reinterpret_cast<V*>(sm_raw);
   using Max = fxk::ElemMax<n2, EPB>;
   __shared__ int smax[3][A::fixed ? Max::size : 1];
+  __shared__ int sbits[S::div_lift ? 3 * EPB : 1];  // of the lines between the stages, per component and element
 
   const int tid = threadIdx.x;
   const int64_t e0 = (int64_t)blockIdx.x * EPB;
@@ -386,6 +430,8 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
   load(0);
   if constexpr (A::fixed) {
     for (int a = 0; a < 3; ++a) Max::clear(smax[a]);
+    if constexpr (S::div_lift)
+      for (int q = tid; q < 3 * EPB; q += blockDim.x) sbits[q] = 0;
     if (!Max::whole) __syncthreads();
     put_max(0);
     __syncthreads();
@@ -401,6 +447,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
   }
 #pragma unroll 1
   for (int a = 0; a < 3; ++a) {
+    int mg = 0;
     if (a1) {
       V v[n];
       if constexpr (A::fixed) {
@@ -426,13 +473,16 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
         const V dA = dot<A>(P.dg.e[I], p, S::np), dB = dot<A>(P.dg.o[I], q, S::nm), iA = dot<A>(P.ig.e[I], p, S::np), iB = dot<A>(P.ig.o[I], q, S::nm);
         x[I * S::sX] = dB + dA;
         x[(m + I) * S::sX] = iA + iB;
+        if constexpr (S::div_lift) note(mg, dB + dA, iA + iB);
         if (2 * I + 1 != m) {
           x[(m - 1 - I) * S::sX] = dB - dA;
           x[(2 * m - 1 - I) * S::sX] = iA - iB;
+          if constexpr (S::div_lift) note(mg, dB - dA, iA - iB);
         }
       }
       }
     }
+    if constexpr (S::div_lift) put_bits<n2, EPB>(sbits + a * EPB, le1, a1 ? fx::bits_of(mg) : 0);
     if (a < 2) load(a + 1);
     __syncthreads();
     if (a2) {
@@ -453,8 +503,10 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
       {
         V v[n];
         load_line<A, n>(x, n, v);
+        if constexpr (S::div_lift) lift_line(v, lift(sbits[a * EPB + le2]));
         fold<A, n>(v, pd, qd);
         load_line<A, n>(x + m * S::sX, n, v);
+        if constexpr (S::div_lift) lift_line(v, lift(sbits[a * EPB + le2]));
         fold<A, n>(v, pi, qi);
       }
 #pragma unroll
@@ -500,6 +552,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
         const int ev = element_expo(Max::get(smax[a], le3));
         slow = slow || out_of_range(ev);
         ex = ev - 1022 - kFieldBits + P.scale + 1 - P.sF[(e0 + le3) * 3 + a];
+        if constexpr (S::div_lift) ex -= lift(sbits[a * EPB + le3]);
       }
 #pragma unroll
       for (int I = 0; I < S::mp; ++I) {
@@ -554,7 +607,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::div_blocks)
 #pragma unroll
     for (int I = 0; I < m; ++I) {
       if constexpr (A::fixed)
-        out[I] = fx::to_double(o[I], eo[I < m / 2 ? I : m - 1 - I]);
+        out[I] = fx::to_double(o[I], eo[I < m / 2 ? I : m - 1 - I]) * __ldg(P.W + KJ * m + I);
       else
         out[I] = o[I];
     }
@@ -583,6 +636,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
   extern __shared__ __align__(16) unsigned char sm_raw[];
   V* sm = reinterpret_cast<V*>(sm_raw);
   __shared__ int smax[A::fixed ? EPB : 1];
+  __shared__ int sbits[S::grad_lift1 ? 6 * EPB : 1];  // of the lines between the stages, two words per component and element
 
   const int tid = threadIdx.x;
   const int64_t e0 = (int64_t)blockIdx.x * EPB;
@@ -604,6 +658,8 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
     for (int I = 0; I < m; ++I) p[I] = a1 ? P.in[(e0 + le1) * m3 + KJ * m + I] : In(0);
     if constexpr (A::fixed) {
       if (tid < EPB) smax[tid] = 0;
+      if constexpr (S::grad_lift1)
+        for (int q = tid; q < 6 * EPB; q += blockDim.x) sbits[q] = 0;
       __syncthreads();
       int ehi = 0;
 #pragma unroll
@@ -630,6 +686,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
 
 #pragma unroll 1
   for (int a = 0; a < 3; ++a) {
+    int mg = 0;
     if (a1) {  // along I -> i: S0 = Dg^T t0, S1 = Ig^T t1, S2 = Ig^T t2, t_b = F[b][a] p
       const C* F = P.F + ((e0 + le1) * 3 + a) * 3 * m3 + KJ;
       V* s = S0(le1) + KJ * S::rY;
@@ -662,14 +719,18 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
         s[i] = B0 + A0;
         s[m * S::sY + i] = A1 + B1;
         s[2 * m * S::sY + i] = A2 + B2;
+        if constexpr (S::grad_lift1) note(mg, B0 + A0, A1 + B1, A2 + B2);
         if (2 * i + 1 != n) {
           s[n - 1 - i] = B0 - A0;
           s[m * S::sY + n - 1 - i] = A1 - B1;
           s[2 * m * S::sY + n - 1 - i] = A2 - B2;
+          if constexpr (S::grad_lift1) note(mg, B0 - A0, A1 - B1, A2 - B2);
         }
       }
       }
     }
+    if constexpr (S::grad_lift1) put_bits<m2, EPB>(sbits + 2 * a * EPB, le1, a1 ? fx::bits_of(mg) : 0);
+    mg = 0;
     __syncthreads();
     if (a2) {  // along J -> j: AI = Ig^T S0 + Dg^T S1, AD = Ig^T S2
       const V* s = S0(le2) + K2 * S::sY + i2;
@@ -696,6 +757,7 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
       for (int b = 0; b < 3; ++b) {
         V v[m];
         load_line<A, m>(s + b * m * S::sY, S::rY, v);
+        if constexpr (S::grad_lift1) lift_line(v, lift(sbits[2 * a * EPB + le2]));
         fold<A, m>(v, p[b], q[b]);
       }
 #pragma unroll
@@ -705,13 +767,16 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
         const ll A2 = dot<A>(P.ig.te[j], p[2], S::mp), B2 = dot<A>(P.ig.to[j], q[2], S::mm);
         x[j * n] = Ev + Od;
         x[m * S::sX + j * n] = A2 + B2;
+        if constexpr (S::grad_lift2) note(mg, Ev + Od, A2 + B2);
         if (2 * j + 1 != n) {
           x[(n - 1 - j) * n] = Ev - Od;
           x[m * S::sX + (n - 1 - j) * n] = A2 - B2;
+          if constexpr (S::grad_lift2) note(mg, Ev - Od, A2 - B2);
         }
       }
       }
     }
+    if constexpr (S::grad_lift2) put_bits<n * m, EPB>(sbits + (2 * a + 1) * EPB, le2, a2 ? fx::bits_of(mg) : 0);
     __syncthreads();
     if (a3) {  // along K -> k: u = Ig^T AI + Dg^T AD
       const V* x = AI(le3) + ji;
@@ -736,16 +801,19 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
       for (int b = 0; b < 2; ++b) {
         V v[m];
         load_line<A, m>(x + b * m * S::sX, S::sX, v);
+        if constexpr (S::grad_lift2) lift_line(v, lift(sbits[(2 * a + 1) * EPB + le3]));
         fold<A, m>(v, p[b], q[b]);
       }
-      const int eu = ex - P.sF[(e0 + le3) * 3 + a];
+      int eu = ex - P.sF[(e0 + le3) * 3 + a];
+      if constexpr (S::grad_lift1) eu -= lift(sbits[2 * a * EPB + le3]);
+      if constexpr (S::grad_lift2) eu -= lift(sbits[(2 * a + 1) * EPB + le3]);
 #pragma unroll
       for (int k = 0; k < S::np; ++k) {
         const ll Ev = dot2(P.ig.te[k], p[0], S::mp, P.dg.to[k], q[1], S::mm);
         const ll Od = dot2(P.dg.te[k], p[1], S::mp, P.ig.to[k], q[0], S::mm);
         if (!slow) {
-          u[k * n2] = fx::to_double(Ev + Od, eu);
-          if (2 * k + 1 != n) u[(n - 1 - k) * n2] = fx::to_double(Ev - Od, eu);
+          u[k * n2] = fx::to_double(Ev + Od, eu) * __ldg(P.W + ji + k * n2);
+          if (2 * k + 1 != n) u[(n - 1 - k) * n2] = fx::to_double(Ev - Od, eu) * __ldg(P.W + ji + (n - 1 - k) * n2);
         }
       }
       }
@@ -770,10 +838,10 @@ static __global__ void __launch_bounds__(256) k_pack_f32(const double* __restric
   }
 }
 
-// F kappa 2^sF in fixed point, kappa = K / 2^63 in [1, 2): 62 bits below the largest of the element and
-// component; *bad where an exponent lies outside 2^+-kOpExp.
-static __global__ void __launch_bounds__(256) k_pack_fx(const double* __restrict__ F, int m, int64_t E, unsigned long long K,
-                                                 int2* __restrict__ out, int* __restrict__ sF, int* bad) {
+// F 2^sF in fixed point, F without the GL weights: 62 bits below the largest of the element and component; *bad where
+// an exponent lies outside 2^+-kOpExp.
+static __global__ void __launch_bounds__(256) k_pack_fx(const double* __restrict__ F, int m, int64_t E,
+                                                        int2* __restrict__ out, int* __restrict__ sF, int* bad) {
   __shared__ int top[3];
   const int m2 = m * m, m3 = m2 * m;
   const int64_t e = blockIdx.x;
@@ -785,66 +853,79 @@ static __global__ void __launch_bounds__(256) k_pack_fx(const double* __restrict
   if (threadIdx.x < 3) {
     const int x = fx::expo(top[threadIdx.x]);
     if (abs(x - 1023) > fx::kOpExp) atomicExch(bad, 1);
-    sF[e * 3 + threadIdx.x] = 61 + 1022 - x;
+    sF[e * 3 + threadIdx.x] = 62 + 1022 - x;
   }
   for (int r = threadIdx.x; r < 9 * m3; r += blockDim.x) {
     const int KJ = r % m2, b = r / m2 % 3, I = r / (3 * m2) % m, a = r / (3 * m3);
     const double f = F[(e * 9 + 3 * b + a) * m3 + KJ * m + I];
-    out[e * 9 * m3 + r] = fx::split(fx::scaled_factor(f, K, fx::expo(top[a])));
+    out[e * 9 * m3 + r] = fx::split(fx::from_double<62>(f, fx::expo(top[a])));
   }
 }
 
-// ---- host: the tables, from Ig and Dg [m][n] ------------------------------------------
+// ---- host: the tables, from Ig and Dg [m][n] and the GL and GLL weights ---------------
 
-struct Scale {  // of the fixed-point tables of one order
-  long double ig, dg;
-  int scale;              // Params::scale
-  unsigned long long K;   // of k_pack_fx
+typedef std::vector<long double> Matrix;
+
+// Of one order: the gradient's matrices W^-1 Ig^T rho and W^-1 Dg^T rho [n][m], the scales of all four tables, and
+// Params::scale and the inverse of the scales that W carries, for both operators.
+struct Scale {
+  Matrix gi, gd;
+  long double s_ig, s_dg, s_gi, s_gd;
+  int scale_div, scale_grad;
+  long double kappa_div, kappa_grad;
 };
 
-// The tables are (Ig sigma_I, Dg sigma_D): sigma = g 2^64 / (largest row sum of magnitudes of the matrix and
-// its transpose), so a contraction of values below B gives values below g B.  With g = 0.8 and B = 2^60 every sum
-// of fx::dot stays below 2^63 (at worst 2^62.98, N = 11), also in the gradient, where two such results are
-// added (1.28 B) before the last contraction.  Odd n has a middle point whose entry stands for itself: g = 0.5 there
-// keeps the entries below 2^63.
-inline Scale table_scale(int N, const std::vector<long double>& Ig, const std::vector<long double>& Dg) {
+// sigma = g 2^64 / (largest row sum of magnitudes): a contraction takes values below B to values below g B.  With g = 0.8
+// (divergence) and 0.62 (gradient, where two results are added: 1.24 B) and B = 2^60 every sum of fx::dot stays
+// below 2^63 (at worst 2^62.69, N = 11), also for the folds of the last contraction's 1.24 B.  Odd n has a middle
+// point whose entry stands for itself: g = 0.5 there keeps the entries below 2^63.
+inline Scale table_scale(int N, const Matrix& Ig, const Matrix& Dg, const Matrix& rho, const Matrix& w) {
   const int n = N + 1, m = N - 1;
-  auto sigma = [&](const std::vector<long double>& X) {
+  auto sigma = [&](const Matrix& X, int rows, int len, long double g) {
     long double top = 0;
-    for (int r = 0; r < m; ++r) {
+    for (int r = 0; r < rows; ++r) {
       long double s = 0;
-      for (int l = 0; l < n; ++l) s += std::fabs(X[r * n + l]);
+      for (int l = 0; l < len; ++l) s += std::fabs(X[r * len + l]);
       top = std::max(top, s);
     }
-    for (int l = 0; l < n; ++l) {
-      long double s = 0;
-      for (int r = 0; r < m; ++r) s += std::fabs(X[r * n + l]);
-      top = std::max(top, s);
-    }
-    return std::ldexp(n % 2 ? 0.5L * (1 - 0x1p-20L) : 0.8L, 64) / top;
+    return std::ldexp(n % 2 ? 0.5L * (1 - 0x1p-20L) : g, 64) / top;
   };
   Scale s;
-  s.ig = sigma(Ig);
-  s.dg = sigma(Dg);
-  int j = 0;
-  const long double f = std::frexp(s.ig * s.ig * s.dg, &j);  // f 2^j, f in [1/2, 1)
-  // kappa = 2^j / (f 2^j) in (1, 2]
-  s.K = (unsigned long long)std::min(std::ldexp(1.0L / f, 63), 0x1.fffffffffffffffep63L);
-  s.scale = 3 * 64 + 62 - j;
+  s.gi.resize(n * m);
+  s.gd.resize(n * m);
+  for (int i = 0; i < n; ++i)
+    for (int I = 0; I < m; ++I) {
+      s.gi[i * m + I] = Ig[I * n + i] * rho[I] / w[i];
+      s.gd[i * m + I] = Dg[I * n + i] * rho[I] / w[i];
+    }
+  s.s_ig = sigma(Ig, m, n, 0.8L);
+  s.s_dg = sigma(Dg, m, n, 0.8L);
+  s.s_gi = sigma(s.gi, n, m, 0.62L);
+  s.s_gd = sigma(s.gd, n, m, 0.62L);
+  auto inverse = [](long double i, long double d, int& scale) {
+    int j = 0;
+    const long double f = std::frexp(i * i * d, &j);  // f 2^j, f in [1/2, 1)
+    scale = 3 * 64 + 62 - j;
+    return 1 / f;
+  };
+  s.kappa_div = inverse(s.s_ig, s.s_dg, s.scale_div);
+  s.kappa_grad = inverse(s.s_gi, s.s_gd, s.scale_grad);
   return s;
 }
 
+// The tables of X [m][n] and, for the transposes, of Y [n][m].
 template <class A, int N>
-Table<typename A::C, N> make_table(const std::vector<long double>& X, long double sigma) {
+Table<typename A::C, N> make_table(const Matrix& X, long double sx, const Matrix& Y, long double sy) {
   constexpr int n = N + 1, m = N - 1;
   Table<typename A::C, N> t{};
-  auto conv = [&](long double v) {
-    if constexpr (A::fixed)
-      return fx::split(std::llround(v * sigma));
-    else
-      return (float)v;
-  };
-  auto fill = [&](auto at, int rows, int len, auto& e, auto& o) {
+  auto fill = [&](const Matrix& M, long double s, int rows, int len, auto& e, auto& o) {
+    auto conv = [&](long double v) {
+      if constexpr (A::fixed)
+        return fx::split(std::llround(v * s));
+      else
+        return (float)v;
+    };
+    auto at = [&](int r, int l) { return M[r * len + l]; };
     for (int r = 0; r < (rows + 1) / 2; ++r) {
       for (int l = 0; l < len / 2; ++l) {
         e[r][l] = conv((at(r, l) + at(r, len - 1 - l)) / 2);
@@ -856,8 +937,8 @@ Table<typename A::C, N> make_table(const std::vector<long double>& X, long doubl
   if constexpr (!A::fixed)
     for (int r = 0; r < m; ++r)
       for (int l = 0; l < n; ++l) t.x[r][l] = (float)X[r * n + l];
-  fill([&](int r, int l) { return X[r * n + l]; }, m, n, t.e, t.o);
-  fill([&](int r, int l) { return X[l * n + r]; }, n, m, t.te, t.to);
+  fill(X, sx, m, n, t.e, t.o);
+  fill(Y, sy, n, m, t.te, t.to);
   return t;
 }
 

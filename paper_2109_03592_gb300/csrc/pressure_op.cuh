@@ -5,6 +5,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "fx_tables.h"
 #include "kernels.h"
 #include "pressure_eo.cuh"
 #include "sem_internal.h"
@@ -15,11 +16,18 @@ template <typename T>
 using Arith = std::conditional_t<std::is_same<T, double>::value, peo::Fixed, peo::F32>;
 
 struct OrderTables {
-  std::vector<long double> Ig, Dg;
+  peo::Matrix Ig, Dg, rho, igt, dgt;  // igt, dgt: the transposes
   peo::Scale scale;
   explicit OrderTables(int N) {
-    gl_matrices_ld(N, Ig, Dg);
-    scale = peo::table_scale(N, Ig, Dg);
+    gl_matrices_ld(N, Ig, Dg, rho);
+    scale = peo::table_scale(N, Ig, Dg, rho, fx_scale(N).w);
+    const int n = N + 1, m = N - 1;
+    igt.resize(n * m);
+    dgt.resize(n * m);
+    for (int q = 0; q < n * m; ++q) {
+      igt[q] = Ig[q % m * n + q / m];
+      dgt[q] = Dg[q % m * n + q / m];
+    }
   }
 };
 template <int N>
@@ -30,10 +38,12 @@ const OrderTables& order_tables() {
 
 // The parameters that depend on the order and the mesh alone.
 template <typename T, int N>
-peo::Params<Arith<T>, N> pressure_params(const PressureOp& op, int64_t E, int64_t n_local) {
+peo::Params<Arith<T>, N> pressure_params(bool grad, const PressureOp& op, int64_t E, int64_t n_local) {
   using A = Arith<T>;
   const OrderTables& o = order_tables<N>();
-  static const auto ig = peo::make_table<A, N>(o.Ig, o.scale.ig), dg = peo::make_table<A, N>(o.Dg, o.scale.dg);
+  const peo::Scale& c = o.scale;
+  static const auto ig = peo::make_table<A, N>(o.Ig, c.s_ig, A::fixed ? c.gi : o.igt, c.s_gi),
+                    dg = peo::make_table<A, N>(o.Dg, c.s_dg, A::fixed ? c.gd : o.dgt, c.s_gd);
   peo::Params<A, N> p{};
   if constexpr (A::fixed) {
     p.F = op.Ffx;
@@ -41,7 +51,8 @@ peo::Params<Arith<T>, N> pressure_params(const PressureOp& op, int64_t E, int64_
     p.F64 = op.F;
     p.Ig = op.Ig;
     p.Dg = op.DIg;
-    p.scale = o.scale.scale;
+    p.scale = grad ? c.scale_grad : c.scale_div;
+    p.W = grad ? op.Wgrad : op.Wdiv;
     p.direct = op.direct;
   } else {
     p.F = op.F32;
@@ -81,7 +92,7 @@ cudaError_t launch_pgrad(int N, const PressureOp& op, const T* p, int64_t E, T* 
   switch (N) {
 #define SEM_CASE(N)                                           \
   case N: {                                                   \
-    auto a = pressure_params<T, N>(op, E, n_local);           \
+    auto a = pressure_params<T, N>(true, op, E, n_local);           \
     a.in = p;                                                 \
     a.out = u;                                                \
     return launch_pressure<T, N>(true, a, s);                 \
@@ -105,7 +116,7 @@ cudaError_t launch_pdiv(int N, const PressureOp& op, const T* u, bool scaled, in
   switch (N) {
 #define SEM_CASE(N)                                           \
   case N: {                                                   \
-    auto a = pressure_params<T, N>(op, E, n_local);           \
+    auto a = pressure_params<T, N>(false, op, E, n_local);           \
     a.in = u;                                                 \
     a.out = out;                                              \
     a.invB = invB;                                            \

@@ -8,16 +8,27 @@ template cudaError_t launch_pdiv<double>(int, const PressureOp&, const double*, 
                                          cudaStream_t);
 
 cudaError_t launch_pressure_pack(const double* F, int N, int64_t E, int2* Ffx, int* sF, int* bad, cudaStream_t s) {
-  unsigned long long K = 0;
+  if (E > 0) peo::k_pack_fx<<<(unsigned)E, 256, 0, s>>>(F, N - 1, E, Ffx, sF, bad);
+  return cudaGetLastError();
+}
+
+bool pressure_weights(int N, std::vector<double>& grad, std::vector<double>& div) {
+  const OrderTables* o = nullptr;
   switch (N) {
 #define SEM_CASE(N) \
-  case N: K = order_tables<N>().scale.K; break;
+  case N: o = &order_tables<N>(); break;
     SEM_PRESSURE_ORDERS(SEM_CASE)
 #undef SEM_CASE
-    default: return cudaErrorNotSupported;
+    default: return false;
   }
-  if (E > 0) peo::k_pack_fx<<<(unsigned)E, 256, 0, s>>>(F, N - 1, E, K, Ffx, sF, bad);
-  return cudaGetLastError();
+  auto cube = [](const peo::Matrix& w, long double kappa, std::vector<double>& out) {
+    const int n = (int)w.size();
+    out.resize((size_t)n * n * n);
+    for (int q = 0; q < n * n * n; ++q) out[q] = (double)(w[q % n] * w[q / n % n] * w[q / (n * n)] * kappa);
+  };
+  cube(fx_scale(N).w, o->scale.kappa_grad, grad);
+  cube(o->rho, o->scale.kappa_div, div);
+  return true;
 }
 
 }  // namespace sem

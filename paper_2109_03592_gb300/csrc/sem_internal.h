@@ -55,8 +55,10 @@ struct Topology {
   int64_t n_global = 0;
   std::vector<int64_t> glo;  // [n_local] first-touch global ids
 };
-// Ig and DIg (pressure_api.cpp) [m][n] in long double, from long-double GLL and GL points.
-void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double>& DIg);
+// Ig and DIg (pressure_api.cpp) [m][n] and the GL weights in long double, from long-double GLL and GL points.
+void gl_matrices_ld(int N, std::vector<long double>& Ig, std::vector<long double>& DIg, std::vector<long double>& rho);
+// PressureOp::Wgrad [n^3] and Wdiv [m^3] (pressure_op64.cu)
+bool pressure_weights(int N, std::vector<double>& grad, std::vector<double>& div);
 
 sem_status build_numbering(int64_t E, int N, const int64_t* vert, Topology& t);
 
@@ -203,6 +205,7 @@ struct sem_mesh {
   mutable int2* Ffx = nullptr;      // F in fixed point and its exponents (PressureOp)
   mutable int* Ffx_s = nullptr;
   mutable int Ffx_direct = 0;
+  mutable double* pW = nullptr;     // PressureOp::Wgrad, then Wdiv
   mutable double* invB = nullptr;   // [n_local] 1 / (QQ^T B)
   // FP32 copies of F and invB, for the FP32 operator of the mixed-precision
   // pressure solve (built on first use)
