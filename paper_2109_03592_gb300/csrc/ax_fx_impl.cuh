@@ -35,6 +35,7 @@
 // through one copy of the code in a loop (no faster at N = 7, 4 to 11% slower above).
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <iterator>
@@ -501,7 +502,7 @@ bool sums_fit(const T& t) {
 }
 
 template <int N, int EPB, bool FUSED>
-cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out) {
+cudaError_t launch_fx_t(const AxParams<double>& user, cudaStream_t s, int* grid_out) {
   constexpr int n = N + 1;
   const size_t smem = sizeof(ll) * (size_t)line_arrays(N) * EPB * LineLayout<n>::size;
   static DeviceOnce once;
@@ -509,6 +510,16 @@ cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out
     return cudaFuncSetAttribute(k_ax_fx<N, EPB, FUSED>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   if (aerr != cudaSuccess) return aerr;
+  // h1 or h2 outside 2^+-100: the operator with both over 2^far, and the results times 2^far by a pass of their own
+  AxParams<double> p = user;
+  int far = 0;
+  const double top = std::max(std::fabs(p.h1), std::fabs(p.h2));
+  if (!p.fx.direct && top != 0.0 && !(top >= 0x1p-100 && top <= 0x1p100)) {
+    far = std::ilogb(top);
+    p.h1 = std::ldexp(p.h1, -far);
+    p.h2 = std::ldexp(p.h2, -far);
+    p.helm = p.h2 != 0.0;
+  }
   const int64_t grid = (p.E + EPB - 1) / EPB;
   if (grid_out) *grid_out = (int)grid;
   if (p.E == 0) return cudaSuccess;
@@ -538,6 +549,8 @@ cudaError_t launch_fx_t(const AxParams<double>& p, cudaStream_t s, int* grid_out
   }
   k_ax_fx<N, EPB, FUSED><<<(unsigned)grid, line_threads(N, EPB), smem, s>>>(q);
   cudaError_t err = cudaGetLastError();
+  if (far && err == cudaSuccess)
+    err = launch_scale_far(p.w, p.E * n * n * n, FUSED ? p.partial : nullptr, (int)grid, far, FUSED ? p.st : nullptr, s);
   if (FUSED && err == cudaSuccess) err = launch_pap_finish(p.partial, (int)grid, p.st, s);
   return err;
 }

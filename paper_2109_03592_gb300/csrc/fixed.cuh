@@ -22,7 +22,7 @@ namespace fx {
 typedef long long ll;
 
 constexpr int kBits = 60;   // magnitudes of fields: at most 2^60
-constexpr int kOpExp = 200;  // exponents of G, B, h1, h2 on the integer path lie within 2^+-200
+constexpr int kOpExp = 200;  // exponents of G and B on the integer path lie within 2^+-200
 
 // A 64-bit value split with a signed low half: v = y 2^32 + x (the register order of v itself).
 __host__ __device__ __forceinline__ int2 split(ll v) {

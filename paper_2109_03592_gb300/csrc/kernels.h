@@ -44,7 +44,7 @@ struct FxOp {
   const double* W64 = nullptr; // [n^3]: w_i w_j w_k kappa
   const double* wq = nullptr; // [n]: the weights
   int range = 0;              // the largest sG[].y
-  int direct = 0;             // every element in FP64: h1 or h2 outside the exponent range of the integer path
+  int direct = 0;             // every element in FP64: h1 or h2 is not finite
 };
 
 struct NoOp {};
@@ -174,6 +174,8 @@ void launch_scale_to_f32(float* r32, const double* r, double sc, int64_t n, cuda
 void launch_accumulate(double* x, const float* d32, double sc, int64_t n, cudaStream_t s);
 void launch_zero_f32(float* a, int64_t n, cudaStream_t s);
 // pAp and alpha from the per-block partials of a fused local operator
+// w [n] and partial [count] (may be null) times 2^e, unless st says that the solve is done
+cudaError_t launch_scale_far(double* w, int64_t n, double* partial, int count, int e, const PcgState* st, cudaStream_t s);
 cudaError_t launch_pap_finish(const double* partial, int count, PcgState* st, cudaStream_t s);
 
 // ---- P_N - P_{N-2} pressure space (pressure.cu) ----

@@ -552,6 +552,16 @@ __global__ void __launch_bounds__(1024) k_pap_finish(const double* __restrict__ 
     }
   }
 }
+__global__ void k_scale_far(double* w, int64_t n, double* partial, int count, int e, const PcgState* st) {
+  if (st && st->done) return;
+  GRID_STRIDE(q, n) w[q] = ldexp(w[q], e);
+  if (partial) GRID_STRIDE(q, count) partial[q] = ldexp(partial[q], e);
+}
+cudaError_t launch_scale_far(double* w, int64_t n, double* partial, int count, int e, const PcgState* st, cudaStream_t s) {
+  k_scale_far<<<vec_blocks(n, 1), kVecThreads, 0, s>>>(w, n, partial, count, e, st);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_pap_finish(const double* partial, int count, PcgState* st, cudaStream_t s) {
   // four partials to a thread and trip, so that few of them do not go through 32 warps' FP64 shuffles (32 partials:
   // 4.7 us with 1024 threads, 3.5 with 32)

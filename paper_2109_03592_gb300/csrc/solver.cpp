@@ -23,7 +23,6 @@
 #include <cstring>
 #include <functional>
 
-#include "fixed.cuh"
 #include "kernels.h"
 #include "sem_internal.h"
 #include "solver.h"
@@ -99,9 +98,7 @@ AxParams<double> ax64_params(const sem_mesh* m, const double* u, double* w, doub
                              double* p, PcgState* st, double* part, double* pout) {
   AxParams<double> a{u, w, m->opG64(), m->opB64(), m->D64, h1, h2, h2 != 0.0, m->E, z, p, st, part, m->dev_err,
                      pout, m->opfx()};
-  const double top = std::ldexp(1.0, fx::kOpExp / 2), low = 1.0 / top;  // NaN is out of range too
-  for (double h : {std::fabs(h1), std::fabs(h2)})
-    if (h != 0.0 && !(h >= low && h <= top)) a.fx.direct = 1;
+  a.fx.direct = !std::isfinite(h1) || !std::isfinite(h2);
   return a;
 }
 
