@@ -166,8 +166,9 @@ sem_status sem_mesh_weights(const sem_mesh* mesh, double* mult_dev, double* mask
  *   h1_eff(q) = h1 * h1_dev[q],  h2_eff(q) = h2 * h2_dev[q]
  * with the scalar h1, h2 that the call passes.  Both NULL restores the
  * constant-coefficient operator.  The factors are stored pre-multiplied
- * (h1 G, h2 B in the forms the chosen kernels read: at most 184 B per local
- * point with both), so the operator kernels read no more bytes than without.
+ * (h1 G, h2 B in the forms the chosen kernels read: 108 B per local point
+ * with both, 136 with the double-float kernels), so the operator kernels read
+ * no more bytes than without.
  * sem_mesh_geometry and sem_rhs keep using the plain G and B.
  * A projection space on the mesh drops its basis at its next solve.
  * Errors: SEM_ERR_INVALID (null mesh; an h1 value <= 0 or an h2 value < 0 or

@@ -151,44 +151,39 @@ void dev_drop(T*& p, size_t count, size_t& tally) {
 sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, CoefArrays& c, cudaStream_t s) {
   const int64_t P = m->n_local;
   const int n = m->n;
+  bool fixed = m->fx_ok && m->ax_var[0] >= kAxFixed && (h1 || h2);
   if (h1) {
     SEM_TRY(dev_alloc(&c.G64, 6 * P, c.bytes));
     SEM_TRY(dev_alloc(&c.G32, 6 * P, c.bytes));
     SEM_TRY(dev_alloc(&c.dK, P, c.bytes));
     if (m->fp64_df) SEM_TRY(dev_alloc(&c.G32lo, 6 * P, c.bytes));
-    if (m->Gfx) {
-      SEM_TRY(dev_alloc(&c.Gfx, 3 * P, c.bytes));
-      SEM_TRY(dev_alloc(&c.fx_sG, m->E, c.bytes));
-    }
+    if (fixed) SEM_TRY(dev_alloc(&c.fx_sG, m->E, c.bytes));
   }
   if (h2) {
     SEM_TRY(dev_alloc(&c.B64, P, c.bytes));
     SEM_TRY(dev_alloc(&c.B32, P, c.bytes));
     SEM_TRY(dev_alloc(&c.dB, P, c.bytes));
     if (m->fp64_df) SEM_TRY(dev_alloc(&c.B32lo, P, c.bytes));
-    if (m->Gfx) {
+    if (fixed) {
       SEM_TRY(dev_alloc(&c.Bfx, P, c.bytes));
       SEM_TRY(dev_alloc(&c.fx_sB, m->E, c.bytes));
     }
   }
   size_t tmp = 0;
-  int* bad_d = nullptr;  // [3]: a bad coefficient; launch_fx_pack's two
+  int* bad_d = nullptr;  // [3]: a bad coefficient; launch_fx_range's two
   SEM_TRY(dev_alloc(&bad_d, 3, tmp));
   std::unique_ptr<int, void (*)(int*)> bad_guard(bad_d, [](int* p) { cudaFree(p); });
   SEM_CUDA(cudaMemsetAsync(bad_d, 0, 3 * sizeof(int), s));
-  if (m->Gfx && (h1 || h2)) {  // the fixed-point factors, from those without quadrature weights
-    SEM_CUDA(launch_geometry(m->xyz, c.G64, c.B64, m->D64, m->wq + n, n, m->E, nullptr, s));
-    launch_fold_coef(c.G64, c.B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
-    SEM_CUDA(launch_fx_pack(c.G64, c.B64, n, m->E, c.Gfx, c.fx_sG, c.Bfx, c.fx_sB, bad_d + 1, s));
-    count_launches(3);
-  }
-  const double* G = m->G64;
-  if (h1 && !G) {  // the plain factors once more
-    SEM_CUDA(launch_geometry(m->xyz, c.G64, nullptr, m->D64, m->wq, n, m->E, nullptr, s));
-    G = c.G64;
+  auto plain = [&]() -> sem_status {  // c.G64 and c.B64
+    if (h1) {
+      SEM_CUDA(launch_geometry(m->xyz, c.G64, nullptr, m->D64, m->wq, n, m->E, nullptr, s));
+      count_launches(1);
+    }
+    launch_fold_coef(c.G64, m->B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
     count_launches(1);
-  }
-  launch_fold_coef(G, m->B64, h1, h2, c.G64, c.B64, n, P, bad_d, s);
+    return SEM_OK;
+  };
+  SEM_TRY(plain());
   if (h1) {
     launch_local_diag(c.G64, c.dK, m->D64, n, m->E, s);
     SEM_CUDA(launch_gs<double>(c.dK, gs_dev(m), 0, nullptr, s));
@@ -199,8 +194,15 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
     SEM_CUDA(launch_gs<double>(c.dB, gs_dev(m), 0, nullptr, s));
     launch_split_f64(c.B64, c.B32, c.B32lo, P, s);
   }
+  double* B1 = reinterpret_cast<double*>(c.Bfx);  // the mass without weights, until it is packed
+  if (fixed) {  // the factors without quadrature weights, in the place of the plain ones
+    SEM_CUDA(launch_geometry(m->xyz, c.G64, B1, m->D64, m->wq + n, n, m->E, nullptr, s));
+    launch_fold_coef(c.G64, B1, h1, h2, c.G64, B1, n, P, bad_d, s);
+    SEM_CUDA(launch_fx_range(c.G64, B1, n, m->E, c.fx_sG, c.fx_sB, bad_d + 1, s));
+    count_launches(3);
+  }
   SEM_CUDA(cudaGetLastError());
-  count_launches(1 + (h1 ? 3 : 0) + (h2 ? 2 : 0));
+  count_launches((h1 ? 3 : 0) + (h2 ? 2 : 0));
   int bad[3] = {0, 0, 0};
   SEM_CUDA(cudaMemcpyAsync(bad, bad_d, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
   SEM_CUDA(cudaStreamSynchronize(s));
@@ -209,26 +211,43 @@ sem_status build_coef(const sem_mesh* m, const double* h1, const double* h2, Coe
                            : "sem_mesh_set_coefficients: need finite h2 >= 0 at every point");
     return SEM_ERR_INVALID;
   }
-  c.fx_range = bad[2];
-  if (bad[1]) {  // coefficients beyond 2^+-200: the kernels on the FP64 pipe take them
-    dev_drop(c.Gfx, 3 * P, c.bytes);
+  if (fixed && !bad[1]) {
+    c.fx_range = bad[2];
+    SEM_CUDA(launch_fx_pack(c.G64, c.fx_sG, B1, c.fx_sB, n, m->E, s));
+    count_launches(1);
+    c.Gfx = reinterpret_cast<int4*>(c.G64);
+    c.G64 = nullptr;
+  } else if (fixed) {  // coefficients beyond 2^+-200, or of too wide a range: the kernels on the FP64 pipe take them
     dev_drop(c.fx_sG, m->E, c.bytes);
     dev_drop(c.Bfx, P, c.bytes);
     dev_drop(c.fx_sB, m->E, c.bytes);
-  } else if (h1 && !m->G64) {
-    dev_drop(c.G64, 6 * P, c.bytes);  // as for the plain factors: no chosen kernel reads it
+    SEM_TRY(plain());
+  }
+  SEM_CUDA(cudaStreamSynchronize(s));
+  return SEM_OK;
+}
+
+}  // namespace
+
+sem_status use_fixed(sem_mesh* m, bool fixed, cudaStream_t s) {
+  if (fixed == (m->Gfx != nullptr)) return SEM_OK;
+  if (fixed) {
+    double* B1 = reinterpret_cast<double*>(m->Bfx);
+    SEM_CUDA(launch_geometry(m->xyz, m->G64, B1, m->D64, m->wq + m->n, m->n, m->E, nullptr, s));
+    SEM_CUDA(launch_fx_pack(m->G64, m->fx_sG, B1, m->fx_sB, m->n, m->E, s));
+    count_launches(2);
+    m->Gfx = reinterpret_cast<int4*>(m->G64);
+    m->G64 = nullptr;
+  } else {
+    m->G64 = reinterpret_cast<double*>(m->Gfx);
+    m->Gfx = nullptr;
+    SEM_CUDA(launch_geometry(m->xyz, m->G64, nullptr, m->D64, m->wq, m->n, m->E, nullptr, s));
+    count_launches(1);
   }
   return SEM_OK;
 }
 
-// The plain FP64 factors, where the tuning freed them (see drop_unused).
-sem_status restore_G64(sem_mesh* m, cudaStream_t s) {
-  if (m->G64) return SEM_OK;
-  SEM_TRY(dev_alloc(&m->G64, 6 * m->n_local, m->dev_bytes));
-  SEM_CUDA(launch_geometry(m->xyz, m->G64, nullptr, m->D64, m->wq, m->n, m->E, nullptr, s));
-  count_launches(1);
-  return SEM_OK;
-}
+namespace {
 
 // Once the kernels are chosen: the factors that none of them reads.
 void drop_unused(sem_mesh* m) {
@@ -237,7 +256,12 @@ void drop_unused(sem_mesh* m) {
     dev_drop(m->G32lo, 6 * P, m->dev_bytes);
     dev_drop(m->B32lo, P, m->dev_bytes);
   }
-  if (m->ax_var[0] >= kAxFixed && m->Gfx) dev_drop(m->G64, 6 * P, m->dev_bytes);
+  if (!m->Gfx && m->fx_ok) {
+    m->fx_ok = false;
+    dev_drop(m->Bfx, P, m->dev_bytes);
+    dev_drop(m->fx_sG, m->E, m->dev_bytes);
+    dev_drop(m->fx_sB, m->E, m->dev_bytes);
+  }
 }
 
 sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
@@ -302,7 +326,6 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
   SEM_TRY(dev_alloc(&m->B64, P, tb));
   SEM_TRY(dev_alloc(&m->G32, 6 * P, tb));
   SEM_TRY(dev_alloc(&m->B32, P, tb));
-  SEM_TRY(dev_alloc(&m->Gfx, 3 * P, tb));
   SEM_TRY(dev_alloc(&m->fx_sG, E, tb));
   SEM_TRY(dev_alloc(&m->Bfx, P, tb));
   SEM_TRY(dev_alloc(&m->fx_sB, E, tb));
@@ -340,7 +363,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
 
   size_t tmp_bytes = 0;
   double *xi_d = nullptr, *tlev_d = nullptr;
-  int* bad_d = nullptr;  // [3]: det J <= 0; launch_fx_pack's two
+  int* bad_d = nullptr;  // [3]: det J <= 0; launch_fx_range's two
   struct Tmp {
     double** a;
     double** c;
@@ -388,9 +411,9 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_CUDA(cudaMemcpyAsync(m->xyz, d.xyz, 3 * P * sizeof(double), cudaMemcpyHostToDevice, s));
   }
   SEM_CUDA(cudaGetLastError());
-  // the fixed-point factors, from those without quadrature weights
+  // the exponents of the fixed-point factors, from those without quadrature weights
   SEM_CUDA(launch_geometry(m->xyz, m->G64, m->B64, m->D64, m->wq + n, n, E, bad_d, s));
-  SEM_CUDA(launch_fx_pack(m->G64, m->B64, n, E, m->Gfx, m->fx_sG, m->Bfx, m->fx_sB, bad_d + 1, s));
+  SEM_CUDA(launch_fx_range(m->G64, m->B64, n, E, m->fx_sG, m->fx_sB, bad_d + 1, s));
   SEM_CUDA(launch_geometry(m->xyz, m->G64, m->B64, m->D64, m->wq, n, E, bad_d, s));
   // assembled diagonals for the Jacobi preconditioner: dK = QQ^T diag(stiffness), dB = QQ^T B
   launch_local_diag(m->G64, m->dK, m->D64, n, E, s);
@@ -409,8 +432,8 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     return SEM_ERR_BAD_MESH;
   }
   m->fx_range = bad[2];
+  m->fx_ok = !bad[1];
   if (bad[1]) {
-    dev_drop(m->Gfx, 3 * P, tb);
     dev_drop(m->fx_sG, E, tb);
     dev_drop(m->Bfx, P, tb);
     dev_drop(m->fx_sB, E, tb);
@@ -529,8 +552,9 @@ sem_status sem_mesh_set_coefficients(sem_mesh* m, const double* h1_dev, const do
   std::lock_guard<std::mutex> lk(m->ws_mutex);
   CoefArrays c;
   sem_status st = build_coef(m, h1_dev, h2_dev, c, s);
-  // h2 out of the fixed-point range: the kernels on the FP64 pipe read the plain factors
-  if (st == SEM_OK && h2_dev && !h1_dev && !c.Bfx && m->Gfx) st = restore_G64(m, s);
+  // h2 alone out of the fixed-point range: the kernels on the FP64 pipe read the plain factors
+  if (st == SEM_OK && m->fx_ok) st = use_fixed(m, !(h2_dev && !h1_dev && !c.Bfx), s);
+  if (st == SEM_OK && cudaStreamSynchronize(s) != cudaSuccess) st = cuda_fail(cudaGetLastError(), "sem_mesh_set_coefficients");
   if (st != SEM_OK) {
     cudaStreamSynchronize(s);
     c.release();

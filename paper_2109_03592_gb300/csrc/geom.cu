@@ -193,15 +193,13 @@ __global__ void k_weights(const uint8_t* __restrict__ wm, double* mult, double* 
   }
 }
 
-// The fixed-point factors of the FP64 operator (FxOp): one CTA per element,
-// first the element's largest exponents of G and B and the range of G over its
-// lines, then the integers.  62 bits for G: with fields of 60 bits the three
-// terms of a point's product meet the bound of fx::dot, and factors up to
-// kMaxRange below the largest keep FP64's bits.
+// The exponents of the fixed-point factors of the FP64 operator (FxOp), one CTA per
+// element: the largest of G and of B, and the range of G over the element's lines.
+// Factors have 62 bits: with fields of 60 bits the three terms of a point's product meet
+// the bound of fx::dot, and factors up to kMaxRange below the largest keep FP64's bits.
 constexpr int kMaxRange = 9;
-__global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, const double* __restrict__ B, int n,
-                                                 int64_t E, int4* __restrict__ fG, int2* __restrict__ sG,
-                                                 int2* __restrict__ fB, int* __restrict__ sB, int* bad) {
+__global__ void __launch_bounds__(256) k_fx_range(const double* __restrict__ G, const double* __restrict__ B, int n,
+                                                  int64_t E, int2* __restrict__ sG, int* __restrict__ sB, int* bad) {
   __shared__ int top[3];
   __shared__ short point[12 * 12 * 12];
   const int n2 = n * n, n3 = n2 * n;
@@ -241,22 +239,53 @@ __global__ void __launch_bounds__(256) k_fx_pack(const double* __restrict__ G, c
     }
     if (B) sB[e] = 62 + 1022 - tB;
   }
-  if (B)
-    for (int p = threadIdx.x; p < n3; p += blockDim.x) fB[e * n3 + p] = fx::split(fx::from_double<62>(B[e * n3 + p], tB));
+}
+
+// G [6][n^3] and B of an element as integers, each in the place of the doubles: a mesh keeps one form of them.
+__global__ void __launch_bounds__(256) k_fx_pack(double* G, const int2* __restrict__ sG, double* B,
+                                                 const int* __restrict__ sB, int n, int64_t E) {
+  constexpr int kMost = (12 * 12 * 12 + 255) / 256;
+  const int n3 = n * n * n;
+  const int64_t e = blockIdx.x;
+  if (B) {
+    const int tB = 62 + 1022 - sB[e];
+    for (int p = threadIdx.x; p < n3; p += blockDim.x) {
+      const int2 v = fx::split(fx::from_double<62>(B[e * n3 + p], tB));
+      reinterpret_cast<int2*>(B)[e * n3 + p] = v;
+    }
+  }
   if (!G) return;
-  for (int q = threadIdx.x; q < 3 * n3; q += blockDim.x) {
-    const int p = q % n3, f = 2 * (q / n3);  // factors f and f + 1 of point p
-    const int2 x = fx::split(fx::from_double<62>(G[(e * 6 + f) * n3 + p], tG));
-    const int2 y = fx::split(fx::from_double<62>(G[(e * 6 + f + 1) * n3 + p], tG));
-    fG[e * 3 * n3 + q] = make_int4(x.x, x.y, y.x, y.y);
+  const int tG = 62 + 1022 - sG[e].x;
+  for (int f = 0; f < 3; ++f) {  // factors 2f and 2f + 1 of a point side by side
+    int4 v[kMost];
+#pragma unroll
+    for (int r = 0; r < kMost; ++r) {
+      const int p = threadIdx.x + 256 * r;
+      if (p < n3) {
+        const int2 x = fx::split(fx::from_double<62>(G[(e * 6 + 2 * f) * n3 + p], tG));
+        const int2 y = fx::split(fx::from_double<62>(G[(e * 6 + 2 * f + 1) * n3 + p], tG));
+        v[r] = make_int4(x.x, x.y, y.x, y.y);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kMost; ++r) {
+      const int p = threadIdx.x + 256 * r;
+      if (p < n3) reinterpret_cast<int4*>(G)[(e * 3 + f) * n3 + p] = v[r];
+    }
   }
 }
 
 // ---- launchers ---------------------------------------------------------------
 
-cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int2* sG, int2* fB, int* sB,
-                           int* bad, cudaStream_t s) {
-  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, B, n, E, fG, sG, fB, sB, bad);
+cudaError_t launch_fx_range(const double* G, const double* B, int n, int64_t E, int2* sG, int* sB, int* bad,
+                            cudaStream_t s) {
+  if (E > 0) k_fx_range<<<(unsigned)E, 256, 0, s>>>(G, B, n, E, sG, sB, bad);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fx_pack(double* G, const int2* sG, double* B, const int* sB, int n, int64_t E, cudaStream_t s) {
+  if (E > 0) k_fx_pack<<<(unsigned)E, 256, 0, s>>>(G, sG, B, sB, n, E);
   return cudaGetLastError();
 }
 

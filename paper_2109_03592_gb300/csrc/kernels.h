@@ -22,10 +22,11 @@ void launch_coords_pipe(double* xyz, const double* xi, const double* tlev, int n
 // w: the quadrature weights, or ones; G, B and bad may be null
 cudaError_t launch_geometry(const double* xyz, double* G, double* B, const double* D, const double* w, int n,
                             int64_t E, int* bad, cudaStream_t s);
-// FxOp's G and sG from G (not null), its B and sB from B (not null), both made with weights of 1; bad[0] is set if an
-// element's exponents are out of range, bad[1] is the largest sG[].y.
-cudaError_t launch_fx_pack(const double* G, const double* B, int n, int64_t E, int4* fG, int2* sG, int2* fB, int* sB,
-                           int* bad, cudaStream_t s);
+// FxOp's sG of G and sB of B (either may be null), both made with weights of 1; bad[0] is set if an element's exponents
+// are out of range, bad[1] is the largest sG[].y.  launch_fx_pack turns them into FxOp's G and B in place.
+cudaError_t launch_fx_range(const double* G, const double* B, int n, int64_t E, int2* sG, int* sB, int* bad,
+                            cudaStream_t s);
+cudaError_t launch_fx_pack(double* G, const int2* sG, double* B, const int* sB, int n, int64_t E, cudaStream_t s);
 void launch_local_diag(const double* G, double* dK, const double* D, int n, int64_t E, cudaStream_t s);
 void launch_fold_coef(const double* G, const double* B, const double* h1, const double* h2, double* cG, double* cB,
                       int n, int64_t P, int* bad, cudaStream_t s);

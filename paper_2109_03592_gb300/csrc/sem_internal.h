@@ -107,16 +107,17 @@ struct sem_mesh {
 
   // device arrays (library-owned)
   double* xyz = nullptr;     // [E][3][n3]
-  double* G64 = nullptr;     // [E][6][n3]; freed after the tuning where no chosen kernel reads it
+  double* G64 = nullptr;     // [E][6][n3]; null while the factors are in fixed point, in the same memory (use_fixed)
   double* B64 = nullptr;     // [E][n3]
   float* G32 = nullptr;      // [E][6][n3] round-to-nearest of G64 (the "hi" part)
   float* G32lo = nullptr;    // [E][6][n3] float(G64 - G32): G64 ~ G32 + G32lo to 2^-48 (double-float only)
   float* B32 = nullptr;      // [E][n3] round-to-nearest of B64
   float* B32lo = nullptr;    // [E][n3] float(B64 - B32) (double-float only)
-  int4* Gfx = nullptr;       // [E][3 n3] the factors in fixed point (FxOp); null where their exponents are out of range
+  int4* Gfx = nullptr;       // [E][3 n3] the factors in fixed point (FxOp)
+  bool fx_ok = false;        // their exponents are in its range
   int2* fx_sG = nullptr;     // [E] FxOp::sG
   int fx_range = 0;          // FxOp::range
-  int2* Bfx = nullptr;       // [E][n3] FxOp::B
+  int2* Bfx = nullptr;       // [E][n3] FxOp::B, where Gfx is set
   int* fx_sB = nullptr;      // [E] FxOp::sB
   int2* fx_W = nullptr;      // [n3] FxOp::W
   int* fx_tw = nullptr;      // [n2] FxOp::tw

@@ -66,10 +66,14 @@ int64_t local_points(const sem_mesh_desc& d) {
   return E * n * n * n;
 }
 
-// Device bytes one request holds while it runs: mesh arrays (~137 B per
-// local point, ~228 B while they are built), solver workspace (~96 B), the request's f, b, x (24 B) and the
-// set-up scratch (8 B), plus a fixed allowance.
-size_t estimate_bytes(const sem_mesh_desc& d) { return (size_t)local_points(d) * 272 + (64u << 20); }
+// Device bytes one request holds while it runs: mesh arrays (~137 B per local point), solver workspace (~96 B), the
+// request's f, b, x (24 B) and the set-up scratch (8 B), plus a fixed allowance; 28 B more for the factors of the
+// double-float kernels, which only the environment chooses on meshes in the fixed-point range.
+size_t estimate_bytes(const sem_mesh_desc& d) {
+  const char* k = std::getenv("SEM_FP64_KERNEL");
+  const bool df = (k && !std::strcmp(k, "df")) || std::getenv("SEM_FP64_DF_VARIANT");
+  return (size_t)local_points(d) * (df ? 300 : 272) + (64u << 20);
+}
 
 }  // namespace
 

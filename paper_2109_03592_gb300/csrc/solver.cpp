@@ -206,9 +206,9 @@ static bool ensure_lo(sem_mesh* m, cudaStream_t s) {
 
 static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
   const size_t n = (size_t)m->n_local;
-  const bool df = ax_df_available(m->N) && ensure_lo(m, s);
   double* w = nullptr;
   SEM_CUDA(cudaMalloc((void**)&w, n * sizeof(double)));
+  const bool df = ax_df_available(m->N) && ensure_lo(m, s);  // without them where memory is short
   cudaEvent_t a, b;
   cudaEventCreate(&a);
   cudaEventCreate(&b);
@@ -220,6 +220,11 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
     for (int v = 0; v < ax_num_variants(); ++v) {
       cudaError_t err = cudaSuccess;
       float total = 0.f;
+      if (kind == 0 && v >= kAxFixed) {
+        if (!m->fx_ok) break;
+        status = use_fixed(m, true, s);
+        if (status != SEM_OK) break;
+      }
       for (int rep = 0; rep <= reps && err == cudaSuccess; ++rep) {
         cudaEventRecord(a, s);
         if (kind == 0) {
@@ -268,9 +273,15 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
     cudaError_t err = cudaMalloc((void**)&p, n * sizeof(double));
     if (err == cudaSuccess) err = cudaMalloc((void**)&part, ((size_t)m->E + 1) * sizeof(double));
     if (err == cudaSuccess) err = cudaMalloc((void**)&st, sizeof(PcgState));
-    if (err == cudaSuccess) err = cudaMemsetAsync(p, 0, n * sizeof(double), s);
+    const bool room = err == cudaSuccess;
+    if (!room) {  // no memory for the trial: the plain form's variant
+      cudaGetLastError();
+      err = cudaSuccess;
+    } else {
+      err = cudaMemsetAsync(p, 0, n * sizeof(double), s);
+    }
     float bestf = 1e30f;
-    for (int v = 0; v < ax_num_variants() && err == cudaSuccess; ++v) {
+    for (int v = 0; room && v < ax_num_variants() && err == cudaSuccess; ++v) {
       float total = 0.f;
       cudaError_t e2 = cudaSuccess;
       for (int rep = 0; rep <= reps && e2 == cudaSuccess; ++rep) {
@@ -319,7 +330,7 @@ static sem_status autotune_measure(sem_mesh* m, cudaStream_t s) {
 sem_status autotune_mesh(sem_mesh* m, cudaStream_t s) {
   int lg = 0;
   while ((1LL << (lg + 1)) <= m->E) ++lg;
-  const TuneKey key{m->N, lg, m->Gfx != nullptr};
+  const TuneKey key{m->N, lg, m->fx_ok};
   {
     std::lock_guard<std::mutex> lk(g_tune_mutex);
     for (auto& kv : g_tune)
@@ -349,7 +360,7 @@ forced:
   }
   if (const char* f = std::getenv("SEM_FP64_VARIANT")) {  // of the native operator; 4 and 5 are fixed point
     const int v = std::atoi(f);
-    if (v >= 0 && v < ax_num_variants() && m->ax_ms[0][v] > 0.f && (v < kAxFixed || m->Gfx)) {
+    if (v >= 0 && v < ax_num_variants() && m->ax_ms[0][v] > 0.f && (v < kAxFixed || m->fx_ok)) {
       m->ax_var[0] = v;
       m->fp64_df = 0;
     }
@@ -366,11 +377,15 @@ forced:
       m->fp64_df = 1;
     }
   }
-  if (m->fp64_df && !ensure_lo(m, s)) {
-    set_error("out of memory for the double-float factors");
-    return SEM_ERR_OOM;
+  if (m->fp64_df && !m->G32lo) {
+    sem_status st = use_fixed(m, false, s);
+    if (st != SEM_OK) return st;
+    if (!ensure_lo(m, s)) {
+      set_error("out of memory for the double-float factors");
+      return SEM_ERR_OOM;
+    }
   }
-  return SEM_OK;
+  return use_fixed(m, m->fx_ok && m->ax_var[0] >= kAxFixed, s);
 }
 
 // ---- CG chunks ---------------------------------------------------------------------

@@ -43,6 +43,8 @@ cudaError_t ax32(const sem_mesh* m, const float* u, float* w, double h1, double 
 AxParams<double> ax64_params(const sem_mesh* m, const double* u, double* w, double h1, double h2, const double* z,
                              double* p, PcgState* st, double* part, double* pout = nullptr);
 int ax64_variant(const sem_mesh* m);
+// The FP64 factors in the form that the fixed-point kernels read, or that of the others (api.cpp).
+sem_status use_fixed(sem_mesh* m, bool fixed, cudaStream_t s);
 cudaError_t ax64(const sem_mesh* m, const double* u, double* w, double h1, double h2, bool fused, const double* z,
                  double* p, PcgState* st, double* part, cudaStream_t s, double* pout = nullptr);
 // Write a fresh PcgState (tol, maxit, done) to ws->st / read it back (both synchronise ws->s).
