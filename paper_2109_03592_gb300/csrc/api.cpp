@@ -25,6 +25,7 @@ void set_error(const std::string& msg) { g_last_error = msg; }
 
 sem_status cuda_fail(cudaError_t err, const char* what) {
   set_error(std::string(what) + ": " + cudaGetErrorName(err) + " (" + cudaGetErrorString(err) + ")");
+  cudaGetLastError();  // reported here: not again by the next call's check
   return err == cudaErrorMemoryAllocation ? SEM_ERR_OOM : SEM_ERR_CUDA;
 }
 

@@ -59,3 +59,18 @@ def test_build_needs_little_more_than_the_mesh(monkeypatch):
     finally:
         del hold
         torch.cuda.empty_cache()
+
+
+def test_an_allocation_failure_is_reported_once(monkeypatch):
+    import torch
+    import paper_2109_03592_gb300 as sem
+    _mesh(monkeypatch, None, 2)
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (1 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(sem.SemError):
+            _mesh(monkeypatch, None, 40)  # 4.5 GB
+        _mesh(monkeypatch, None, 4)  # the next call knows nothing of it
+    finally:
+        del hold
+        torch.cuda.empty_cache()
