@@ -90,12 +90,12 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->cdB);
   dev_free(m->cBfx);
   dev_free(m->cfx_sB);
-  dev_free(m->Fgl);
+  dev_free(m->pF);
+  dev_free(m->pF_s);
+  dev_free(m->prho);
   dev_free(m->pdinv);
   dev_free(m->Igl);
   dev_free(m->DIgl);
-  dev_free(m->Ffx);
-  dev_free(m->Ffx_s);
   dev_free(m->pW);
   dev_free(m->invB);
   dev_free(m->Fgl32);

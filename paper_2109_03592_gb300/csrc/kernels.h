@@ -185,18 +185,23 @@ cudaError_t launch_pap_finish(const double* partial, int count, PcgState* st, cu
 size_t gl_factors_smem(int n, int m);
 cudaError_t launch_gl_factors(const double* xyz, const double* Ig, const double* DIg, const double* rho, int n, int m,
                               int64_t E, double* F, int* bad, cudaStream_t s);
-// What the weak gradient and divergence read (pressure_eo.cuh).  FP64: the factors in fixed point (Ffx, sF; direct: out
-// of its range) and the plain data for the elements that are evaluated in FP64; FP32: F32, in the same order.
-struct PressureOp {
-  const double *F, *Ig, *DIg, *invB, *Wgrad, *Wdiv;
-  const int2* Ffx;
-  const int* sF;
+// The factors F[b][a] of the pressure operators, in one form: fixed point, int2 [E][3 (a)][m (I)][3 (b)][m (K)][m (J)]
+// without the GL weights and times 2^sF; or, where an exponent is out of its range (direct), double [E][3 (b)][3 (a)][m^3].
+struct PressureFactors {
+  const void* data;
+  const int* sF;      // [E][3]
+  const double* rho;  // [m] the weights
   int direct;
+};
+// What the weak gradient and divergence read (pressure_eo.cuh); FP32: F32, in the order of the fixed-point form.
+struct PressureOp {
+  PressureFactors f;
+  const double *Ig, *DIg, *invB, *Wgrad, *Wdiv;
   const float *F32, *invB32;
 };
-// Ffx and sF from F made with weights of 1
-cudaError_t launch_pressure_pack(const double* F, int N, int64_t E, int2* Ffx, int* sF, int* bad, cudaStream_t s);
-cudaError_t launch_pressure_pack32(const double* F, int N, int64_t E, float* F32, cudaStream_t s);
+// F, made with weights of 1, into its fixed-point form in place; *bad where an exponent is out of range
+cudaError_t launch_pressure_pack(void* F, int N, int64_t E, int* sF, int* bad, cudaStream_t s);
+cudaError_t launch_pressure_pack32(const PressureFactors& F, int N, int64_t E, float* F32, cudaStream_t s);
 void launch_recip(const double* a, double* out, int64_t n, cudaStream_t s);
 // T = double or float
 template <typename T>
@@ -217,7 +222,7 @@ int pressure_red_blocks();
 cudaError_t launch_pdot(const double* a, const double* b, int64_t n, double* partial, double* out, cudaStream_t s);
 // out [E m^3] = diag(E), or 1 / diag(E) with recip (the pressure operator's
 // diagonal; wm's Dirichlet bit is the velocity mask, dB the assembled mass)
-cudaError_t launch_pdiag(const double* F, const double* Ig, const double* DIg, const uint8_t* wm, const double* dB,
+cudaError_t launch_pdiag(const PressureFactors& F, const double* Ig, const double* DIg, const uint8_t* wm, const double* dB,
                         int n, int m, int64_t E, double* out, int recip, cudaStream_t s);
 // Device-resident pressure CG steps (state in a PcgState, see pressure.cu):
 // sigma and alpha; the update with the stop / pause tests; the direction.

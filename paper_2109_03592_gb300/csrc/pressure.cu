@@ -15,6 +15,7 @@
 // contractions of whole lines held in registers, several elements per CTA,
 // in FP32 or in fixed point.
 #include "kernels.h"
+#include "pressure_factors.cuh"
 
 namespace sem {
 
@@ -83,7 +84,7 @@ __global__ void k_gl_factors(const double* __restrict__ xyz, const double* __res
     C[2][1] = J[0][2] * J[1][0] - J[0][0] * J[1][2];
     C[2][2] = J[0][0] * J[1][1] - J[0][1] * J[1][0];
     const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
-    if (!(det > 0.0)) atomicExch(bad, 1);
+    if (bad && !(det > 0.0)) atomicExch(bad, 1);
     const double w = rho[i] * rho[j] * rho[k];
     double* Fe = F + e * 9 * m3 + q;
     for (int b = 0; b < 3; ++b)
@@ -360,7 +361,7 @@ __global__ void k_presidual_keep(const double* __restrict__ g, double cg, const 
 // DIg*DIg (elementwise) along each direction, by how many of b, b' are that
 // direction.  Shared memory: X [3][m][n], wgt [n^3], T1 [n][n][m],
 // T2 [n][m][m], S [6][m^3].
-__global__ void k_pdiag(const double* __restrict__ F, const double* __restrict__ Ig, const double* __restrict__ DIg,
+__global__ void k_pdiag(const PressureFactors F, const double* __restrict__ Ig, const double* __restrict__ DIg,
                         const uint8_t* __restrict__ wm, const double* __restrict__ dB, int n, int m, int64_t E,
                         double* __restrict__ out, int recip) {
   extern __shared__ double sm[];
@@ -414,10 +415,10 @@ __global__ void k_pdiag(const double* __restrict__ F, const double* __restrict__
     __syncthreads();
   }
   for (int q = threadIdx.x; q < m3; q += blockDim.x) {
-    const double* Fe = F + e * 9 * m3 + q;
     double d = 0.0;
     for (int a = 0; a < 3; ++a) {
-      const double f0 = Fe[(0 + a) * m3], f1 = Fe[(3 + a) * m3], f2 = Fe[(6 + a) * m3];
+      const double f0 = pressure_factor(F, m, e, 0, a, q), f1 = pressure_factor(F, m, e, 1, a, q),
+                   f2 = pressure_factor(F, m, e, 2, a, q);
       d += f0 * f0 * S[q] + f1 * f1 * S[m3 + q] + f2 * f2 * S[2 * m3 + q] +
            2.0 * (f0 * f1 * S[3 * m3 + q] + f0 * f2 * S[4 * m3 + q] + f1 * f2 * S[5 * m3 + q]);
     }
@@ -475,7 +476,7 @@ cudaError_t launch_pdot(const double* a, const double* b, int64_t n, double* par
   return cudaGetLastError();
 }
 
-cudaError_t launch_pdiag(const double* F, const double* Ig, const double* DIg, const uint8_t* wm, const double* dB,
+cudaError_t launch_pdiag(const PressureFactors& F, const double* Ig, const double* DIg, const uint8_t* wm, const double* dB,
                         int n, int m, int64_t E, double* out, int recip, cudaStream_t s) {
   const size_t smem = sizeof(double) * (3 * m * n + n * n * n + n * n * m + n * m * m + 6 * m * m * m);
   cudaError_t err = cudaFuncSetAttribute(k_pdiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -166,8 +166,10 @@ void gl_matrices(int N, std::vector<double>& Ig, std::vector<double>& DIg, std::
     }
 }
 
+PressureFactors pressure_factors(const sem_mesh* m) { return {m->pF, m->pF_s, m->prho, m->pF_direct}; }
+
 PressureOp pressure_op(const sem_mesh* m) {
-  return {m->Fgl, m->Igl, m->DIgl, m->invB, m->pW, m->pW + (size_t)m->n * m->n * m->n, m->Ffx, m->Ffx_s, m->Ffx_direct, m->Fgl32, m->invB32};
+  return {pressure_factors(m), m->Igl, m->DIgl, m->invB, m->pW, m->pW + (size_t)m->n * m->n * m->n, m->Fgl32, m->invB32};
 }
 
 #define SEM_TRY_STATUS(expr)          \
@@ -191,14 +193,13 @@ sem_status check_mesh(const sem_mesh* m, const char* who) {
 // Build the mesh's GL-point data once (under its p_mutex).
 sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   std::lock_guard<std::mutex> lk(m->p_mutex);
-  if (m->Fgl) return SEM_OK;
+  if (m->pF) return SEM_OK;
   SEM_CUDA(cudaSetDevice(m->device));
   const int N = m->N, n = N + 1, mm = N - 1;
   const int64_t m3 = (int64_t)mm * mm * mm;
   std::vector<double> Ig, DIg, rho;
   gl_matrices(N, Ig, DIg, rho);
   double *F = nullptr, *I_d = nullptr, *DI_d = nullptr, *rho_d = nullptr, *iB = nullptr, *pW = nullptr;
-  int2* Ffx = nullptr;
   int *sF = nullptr, *bad_d = nullptr;  // bad: det(J) <= 0; factors out of the fixed-point form's range
   auto release = [&]() {
     if (F) cudaFree(F);
@@ -207,7 +208,6 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
     if (rho_d) cudaFree(rho_d);
     if (iB) cudaFree(iB);
     if (pW) cudaFree(pW);
-    if (Ffx) cudaFree(Ffx);
     if (sF) cudaFree(sF);
     if (bad_d) cudaFree(bad_d);
   };
@@ -227,7 +227,6 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   if ((e = cudaMalloc((void**)&rho_d, sizeof(double) * 2 * mm)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&pW, sizeof(double) * W.size())) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&bad_d, 2 * sizeof(int))) != cudaSuccess) return fail(e, "cudaMalloc");
-  if ((e = cudaMalloc((void**)&Ffx, sizeof(int2) * 9 * m3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&sF, sizeof(int) * 3 * m->E)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&iB, sizeof(double) * m->n_local)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMemcpyAsync(I_d, Ig.data(), sizeof(double) * mm * n, cudaMemcpyHostToDevice, s)) != cudaSuccess)
@@ -241,34 +240,35 @@ sem_status ensure_pressure(const sem_mesh* m, cudaStream_t s) {
   if ((e = cudaMemsetAsync(bad_d, 0, 2 * sizeof(int), s)) != cudaSuccess) return fail(e, "cudaMemsetAsync");
   if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d + mm, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
     return fail(e, "k_gl_factors");
-  if ((e = launch_pressure_pack(F, N, m->E, Ffx, sF, bad_d + 1, s)) != cudaSuccess) return fail(e, "k_pack_fx");
-  if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
-    return fail(e, "k_gl_factors");
+  if ((e = launch_pressure_pack(F, N, m->E, sF, bad_d + 1, s)) != cudaSuccess) return fail(e, "k_pack_fx");
   launch_recip(m->dB, iB, m->n_local, s);
-  count_launches(4);
+  count_launches(3);
   int bad[2] = {0, 0};
   if ((e = cudaMemcpyAsync(bad, bad_d, 2 * sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
     return fail(e, "cudaMemcpyAsync");
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "cudaStreamSynchronize");
-  cudaFree(rho_d);
-  rho_d = nullptr;
-  cudaFree(bad_d);
-  bad_d = nullptr;
   if (bad[0]) {
     release();
     set_error("mesh has an element with det(J) <= 0 at a GL point");
     return SEM_ERR_BAD_MESH;
   }
+  if (bad[1]) {  // out of the fixed-point form's range: as doubles
+    if ((e = launch_gl_factors(m->xyz, I_d, DI_d, rho_d, n, mm, m->E, F, bad_d, s)) != cudaSuccess)
+      return fail(e, "k_gl_factors");
+    count_launches(1);
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "cudaStreamSynchronize");
+  }
+  cudaFree(bad_d);
   sem_mesh* mut = const_cast<sem_mesh*>(m);
-  mut->dev_bytes += sizeof(double) * (18 * m3 * m->E + 2 * mm * n + W.size() + m->n_local) + sizeof(int) * 3 * m->E;
-  m->Ffx = Ffx;
-  m->Ffx_s = sF;
-  m->Ffx_direct = bad[1];
+  mut->dev_bytes += sizeof(double) * (9 * m3 * m->E + 2 * mm * n + 2 * mm + W.size() + m->n_local) + sizeof(int) * 3 * m->E;
+  m->pF_s = sF;
+  m->pF_direct = bad[1];
+  m->prho = rho_d;
   m->invB = iB;
   m->pW = pW;
   m->Igl = I_d;
   m->DIgl = DI_d;
-  m->Fgl = F;
+  m->pF = F;
   return SEM_OK;
 }
 
@@ -294,7 +294,7 @@ sem_status ensure_pressure32(const sem_mesh* m, cudaStream_t s) {
   cudaError_t e;
   if ((e = cudaMalloc((void**)&F, sizeof(float) * nF)) != cudaSuccess) return fail(e, "cudaMalloc");
   if ((e = cudaMalloc((void**)&iB, sizeof(float) * m->n_local)) != cudaSuccess) return fail(e, "cudaMalloc");
-  if ((e = launch_pressure_pack32(m->Fgl, N, m->E, F, s)) != cudaSuccess) return fail(e, "k_pack_f32");
+  if ((e = launch_pressure_pack32(pressure_factors(m), N, m->E, F, s)) != cudaSuccess) return fail(e, "k_pack_f32");
   launch_recip_f32(m->dB, iB, m->n_local, s);
   count_launches(2);
   if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail(e, "pressure FP32 copies");
@@ -316,7 +316,7 @@ sem_status ensure_pdiag(const sem_mesh* m, cudaStream_t s) {
   double* d = nullptr;
   cudaError_t e = cudaMalloc((void**)&d, sizeof(double) * np);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc");
-  e = launch_pdiag(m->Fgl, m->Igl, m->DIgl, m->wm, m->dB, m->n, mm, m->E, d, 1, s);
+  e = launch_pdiag(pressure_factors(m), m->Igl, m->DIgl, m->wm, m->dB, m->n, mm, m->E, d, 1, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     cudaStreamSynchronize(s);
@@ -634,8 +634,9 @@ sem_status sem_pressure_factors(const sem_mesh* m, double* F_dev, void* stream) 
   cudaStream_t s = (cudaStream_t)stream;
   st = ensure_pressure(m, s);
   if (st != SEM_OK) return st;
-  const int64_t mm = m->N - 1;
-  SEM_CUDA(cudaMemcpyAsync(F_dev, m->Fgl, sizeof(double) * 9 * mm * mm * mm * m->E, cudaMemcpyDeviceToDevice, s));
+  // not kept: the same kernel on the same coordinates gives the same factors
+  SEM_CUDA(launch_gl_factors(m->xyz, m->Igl, m->DIgl, m->prho, m->n, m->N - 1, m->E, F_dev, nullptr, s));
+  count_launches(1);
   return SEM_OK;
 }
 
@@ -721,7 +722,7 @@ sem_status sem_pressure_diag(const sem_mesh* m, double* d_dev, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   st = ensure_pressure(m, s);
   if (st != SEM_OK) return st;
-  SEM_CUDA(launch_pdiag(m->Fgl, m->Igl, m->DIgl, m->wm, m->dB, m->n, m->N - 1, m->E, d_dev, 0, s));
+  SEM_CUDA(launch_pdiag(pressure_factors(m), m->Igl, m->DIgl, m->wm, m->dB, m->n, m->N - 1, m->E, d_dev, 0, s));
   count_launches(1);
   return SEM_OK;
 }

@@ -57,6 +57,7 @@
 
 #include "fixed.cuh"
 #include "fx_common.cuh"
+#include "pressure_factors.cuh"
 
 namespace sem {
 namespace peo {
@@ -151,7 +152,8 @@ struct Params {
   const typename A::In* invB;  // reciprocal assembled mass (divergence), or null
   const typename A::C* F;
   const int* sF;               // fixed point: [E][3], the factors are F 2^sF
-  const double *F64, *Ig, *Dg; // for slow_div and slow_grad
+  PressureFactors f;           // for slow_div and slow_grad, with the matrices
+  const double *Ig, *Dg;
   int64_t E, n_local;
   int scale;                   // fixed point: F C v = 2^scale W x the integers' product along the path, over 2^254
   const double* W;             // [n^3] (gradient) or [m^3]: the weights and the inverse of the scales
@@ -311,8 +313,8 @@ __device__ __noinline__ void slow_div(const Params<Fixed, N>& P, int64_t e, doub
         g1 += P.Ig[I * n + i] * Y1[KJ * n + i];
         g2 += P.Ig[I * n + i] * Y0[KJ * n + i];
       }
-      const double* F = P.F64 + e * 9 * m3 + q;
-      const double v = F[a * m3] * g0 + F[(3 + a) * m3] * g1 + F[(6 + a) * m3] * g2;
+      const double v = pressure_factor(P.f, m, e, 0, a, q) * g0 + pressure_factor(P.f, m, e, 1, a, q) * g1 +
+                       pressure_factor(P.f, m, e, 2, a, q) * g2;
       double* o = P.out + e * m3 + q;
       *o = a == 0 ? v : *o + v;
     }
@@ -338,10 +340,9 @@ __device__ __noinline__ void slow_grad(const Params<Fixed, N>& P, int64_t e, dou
 #pragma unroll 1
       for (int I = 0; I < m; ++I) {
         const double p = P.in[e * m3 + KJ * m + I];
-        const double* F = P.F64 + e * 9 * m3 + KJ * m + I;
-        s0 += P.Dg[I * n + i] * (F[a * m3] * p);
-        s1 += P.Ig[I * n + i] * (F[(3 + a) * m3] * p);
-        s2 += P.Ig[I * n + i] * (F[(6 + a) * m3] * p);
+        s0 += P.Dg[I * n + i] * (pressure_factor(P.f, m, e, 0, a, KJ * m + I) * p);
+        s1 += P.Ig[I * n + i] * (pressure_factor(P.f, m, e, 1, a, KJ * m + I) * p);
+        s2 += P.Ig[I * n + i] * (pressure_factor(P.f, m, e, 2, a, KJ * m + I) * p);
       }
       S0[q] = s0;
       S1[q] = s1;
@@ -828,27 +829,29 @@ __global__ void __launch_bounds__(Shape<A, N>::threads, Shape<A, N>::grad_blocks
   }
 }
 
-// The factors F[b][a](q) as the kernels read them.
-static __global__ void __launch_bounds__(256) k_pack_f32(const double* __restrict__ F, int m, int64_t E, float* __restrict__ out) {
+// The factors F[b][a](q) in FP32, as the kernels read them.
+static __global__ void __launch_bounds__(256) k_pack_f32(const PressureFactors F, int m, int64_t E, float* __restrict__ out) {
   const int m2 = m * m, m3 = m2 * m;
   const int64_t e = blockIdx.x;
   for (int r = threadIdx.x; r < 9 * m3; r += blockDim.x) {
     const int KJ = r % m2, b = r / m2 % 3, I = r / (3 * m2) % m, a = r / (3 * m3);
-    out[e * 9 * m3 + r] = (float)F[(e * 9 + 3 * b + a) * m3 + KJ * m + I];
+    out[e * 9 * m3 + r] = (float)pressure_factor(F, m, e, b, a, KJ * m + I);
   }
 }
 
-// F 2^sF in fixed point, F without the GL weights: 62 bits below the largest of the element and component; *bad where
-// an exponent lies outside 2^+-kOpExp.
-static __global__ void __launch_bounds__(256) k_pack_fx(const double* __restrict__ F, int m, int64_t E,
-                                                        int2* __restrict__ out, int* __restrict__ sF, int* bad) {
+// F [3 (b)][3 (a)][m^3] of an element, without the GL weights, into its fixed-point form in place: 62 bits below the
+// largest of the element and component; *bad where an exponent lies outside 2^+-kOpExp.
+static __global__ void __launch_bounds__(256) k_pack_fx(double* F, int m, int64_t E, int* __restrict__ sF, int* bad) {
+  extern __shared__ double f[];  // [9 m^3]
   __shared__ int top[3];
   const int m2 = m * m, m3 = m2 * m;
   const int64_t e = blockIdx.x;
   if (threadIdx.x < 3) top[threadIdx.x] = 0;
   __syncthreads();
-  for (int r = threadIdx.x; r < 9 * m3; r += blockDim.x)
-    atomicMax(top + r / m3 % 3, __double2hiint(F[e * 9 * m3 + r]) & 0x7fffffff);
+  for (int r = threadIdx.x; r < 9 * m3; r += blockDim.x) {
+    f[r] = F[e * 9 * m3 + r];
+    atomicMax(top + r / m3 % 3, __double2hiint(f[r]) & 0x7fffffff);
+  }
   __syncthreads();
   if (threadIdx.x < 3) {
     const int x = fx::expo(top[threadIdx.x]);
@@ -857,8 +860,7 @@ static __global__ void __launch_bounds__(256) k_pack_fx(const double* __restrict
   }
   for (int r = threadIdx.x; r < 9 * m3; r += blockDim.x) {
     const int KJ = r % m2, b = r / m2 % 3, I = r / (3 * m2) % m, a = r / (3 * m3);
-    const double f = F[(e * 9 + 3 * b + a) * m3 + KJ * m + I];
-    out[e * 9 * m3 + r] = fx::split(fx::from_double<62>(f, fx::expo(top[a])));
+    reinterpret_cast<int2*>(F)[e * 9 * m3 + r] = fx::split(fx::from_double<62>(f[(3 * b + a) * m3 + KJ * m + I], fx::expo(top[a])));
   }
 }
 

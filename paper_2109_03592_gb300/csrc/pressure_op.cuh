@@ -46,14 +46,14 @@ peo::Params<Arith<T>, N> pressure_params(bool grad, const PressureOp& op, int64_
                     dg = peo::make_table<A, N>(o.Dg, c.s_dg, A::fixed ? c.gd : o.dgt, c.s_gd);
   peo::Params<A, N> p{};
   if constexpr (A::fixed) {
-    p.F = op.Ffx;
-    p.sF = op.sF;
-    p.F64 = op.F;
+    p.F = static_cast<const int2*>(op.f.data);
+    p.sF = op.f.sF;
+    p.f = op.f;
     p.Ig = op.Ig;
     p.Dg = op.DIg;
     p.scale = grad ? c.scale_grad : c.scale_div;
     p.W = grad ? op.Wgrad : op.Wdiv;
-    p.direct = op.direct;
+    p.direct = op.f.direct;
   } else {
     p.F = op.F32;
   }

@@ -7,8 +7,12 @@ template cudaError_t launch_pgrad<double>(int, const PressureOp&, const double*,
 template cudaError_t launch_pdiv<double>(int, const PressureOp&, const double*, bool, int64_t, double*, int64_t,
                                          cudaStream_t);
 
-cudaError_t launch_pressure_pack(const double* F, int N, int64_t E, int2* Ffx, int* sF, int* bad, cudaStream_t s) {
-  if (E > 0) peo::k_pack_fx<<<(unsigned)E, 256, 0, s>>>(F, N - 1, E, Ffx, sF, bad);
+cudaError_t launch_pressure_pack(void* F, int N, int64_t E, int* sF, int* bad, cudaStream_t s) {
+  const int m = N - 1;
+  const size_t smem = sizeof(double) * 9 * m * m * m;
+  cudaError_t err = cudaFuncSetAttribute(peo::k_pack_fx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  if (E > 0) peo::k_pack_fx<<<(unsigned)E, 256, smem, s>>>(static_cast<double*>(F), m, E, sF, bad);
   return cudaGetLastError();
 }
 

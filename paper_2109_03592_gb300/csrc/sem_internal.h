@@ -200,12 +200,12 @@ struct sem_mesh {
   // 3 b + a) and the GLL basis values / derivatives at the GL points [m][n]
   mutable std::mutex p_mutex;
   mutable double* pdinv = nullptr;  // [E m^3] 1 / diag(E), the pressure CG's Jacobi preconditioner
-  mutable double* Fgl = nullptr;
+  mutable void* pF = nullptr;
+  mutable int* pF_s = nullptr;      // (PressureFactors)
+  mutable int pF_direct = 0;
+  mutable double* prho = nullptr;   // [2 m] GL weights, then ones
   mutable double* Igl = nullptr;
   mutable double* DIgl = nullptr;
-  mutable int2* Ffx = nullptr;      // F in fixed point and its exponents (PressureOp)
-  mutable int* Ffx_s = nullptr;
-  mutable int Ffx_direct = 0;
   mutable double* pW = nullptr;     // PressureOp::Wgrad, then Wdiv
   mutable double* invB = nullptr;   // [n_local] 1 / (QQ^T B)
   // FP32 copies of F and invB, for the FP32 operator of the mixed-precision

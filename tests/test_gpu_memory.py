@@ -61,6 +61,20 @@ def test_build_needs_little_more_than_the_mesh(monkeypatch):
         torch.cuda.empty_cache()
 
 
+def test_one_form_of_the_pressure_factors(monkeypatch):
+    import torch
+    m = _mesh(monkeypatch, None, 12, 5)
+    small = 64 * m.E + (1 << 20)
+    base, points = _bytes(m), m.pressure_size()
+    p = torch.ones(m.pressure_shape, dtype=torch.float64, device="cuda")
+    m.pressure_apply(p, torch.empty_like(p))
+    assert _bytes(m) <= base + 72 * points + 8 * m.n_local + small
+    m.pressure_diag(torch.empty_like(p))
+    assert _bytes(m) <= base + 80 * points + 8 * m.n_local + small
+    m.pressure_apply_f32(p.float(), torch.empty(m.pressure_shape, dtype=torch.float32, device="cuda"))
+    assert _bytes(m) <= base + 116 * points + 12 * m.n_local + small
+
+
 def test_an_allocation_failure_is_reported_once(monkeypatch):
     import torch
     import paper_2109_03592_gb300 as sem
