@@ -116,17 +116,19 @@ __device__ __forceinline__ void line_contract(const T* __restrict__ S, const T (
   }
 }
 
-// Lines per thread, Q: two in FP32 where n is a multiple of 4 (vector row reads), (a, b) and
-// (a, b + n / 2), so that a matrix row read from shared memory serves both: the matrices'
-// rows were half of the shared-memory reads that bound the kernel.  One application at E =
-// 32,768, N = 7: 315 us, 326 with one line.  For other n the rows are scalar reads that the
-// compiler keeps in registers (168 at n = 10 with two lines).  Meshes of fewer than
-// kFdmPairElements keep one line: they do not fill the GPU (32 elements per SM, twice), and
-// two lines are twice the chain (a whole application on a small mesh 28.7 us, 27.7 with one).
+// Lines per thread, Q: two in FP32 at N = 7, (a, b) and (a, b + n / 2), so that a matrix row read
+// from shared memory serves both: the matrices' rows were half of the shared-memory reads that
+// bound the kernel.  One application at E = 32,768: 315 us, 326 with one line; on boxes of 19,683
+// elements 222 and 230, of 9261 214 and 217.  Meshes of fewer than kFdmPairElements keep one line:
+// they do not fill the GPU (32 elements per SM, twice), and two lines are twice the chain (4913
+// elements 94.2 and 94.4, 2197 45.7 and 43.6).  Other orders keep one line: two are no faster at
+// N = 3 (64,000 elements 195.3 and 195.4, 32,768 155.5 and 153.6, 4096 58.3 and 56.2) and slower
+// at N = 11 (9261 elements 360 and 354, 2197 78.3 and 76.8), and where n is no multiple of 4 the rows
+// are scalar reads that the compiler keeps in registers (168 at n = 10 with two lines).
 constexpr int64_t kFdmPairElements = 2 * 32 * 152;
 template <int N, typename T>
 __host__ __device__ constexpr int fdm_lines() {
-  return (N + 1) % 4 == 0 && sizeof(T) == 4 ? 2 : 1;
+  return N == 7 && sizeof(T) == 4 ? 2 : 1;
 }
 
 // (With the 1D matrices hoisted into registers, 110 registers at N = 7 in
