@@ -42,8 +42,8 @@
 //
 // What bounds them: fixed point, issue slots (9 in 10 instructions are multiply-adds, 64-bit additions and the
 // splits between them) and the barriers between stages of different width; FP32, shared memory and DRAM (70% and
-// 50% busy).  E = 32,768, N = 7: gradient 512 us, divergence 621 us, E in FP64 1.36 ms (0.28 TB/s of p, u and
-// factors) against 8.76 ms on the FP64 pipe; E in FP32 350 us against 604 us for plain contractions with the
+// 50% busy).  E = 32,768, N = 7: E in FP64 1.38 ms (0.28 TB/s of p, u and factors; 1.32 before the weights and the
+// lines' lifts) against 8.76 ms on the FP64 pipe; E in FP32 350 us against 604 us for plain contractions with the
 // matrices in shared memory.
 //
 // An element whose input is not finite, or whose exponents lie outside 2^+-500, is
@@ -140,8 +140,9 @@ struct Shape {
   static constexpr int threads = (EPB * n2 + 31) / 32 * 32;
   static constexpr size_t smem = sizeof(typename A::V) * (size_t)EPB * elem;
   // Resident threads per SM.  Fixed point, N = 7: the gradient 530 us with 512, 515 with 640; the divergence 622
-  // and 654 (its spills).
-  static constexpr int grad_blocks = imax((A::fixed ? 640 : 1024) / threads, 1);
+  // and 654 (its spills).  The gradient of N = 2 and 3 fits 1152 (E at N = 2, 155,392 elements: 240 us, 264 with what the
+  // compiler takes).
+  static constexpr int grad_blocks = imax((A::fixed ? (N <= 3 ? 1152 : 640) : 1024) / threads, 1);
   static constexpr int div_blocks = imax((A::fixed ? 512 : 1024) / threads, 1);
 };
 
