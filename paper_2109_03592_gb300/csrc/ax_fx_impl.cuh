@@ -29,8 +29,9 @@
 //
 // What bounds it: issue, of multiply-adds and of the additions between them (integer pipe 57% busy, multiply pipe
 // 35%, DRAM 46%).  One thread per 2x2x2 octant instead of per line needed twice the shared-memory reads and splits
-// (N = 7, E = 32,768: 361 us; this kernel 274, 4.9 TB/s of u, G and w; even-odd FP32 pairs 407, the FP64 pipe 1900;
-// odd n, column threads without the fold, N = 8, E = 22,528: 660; this kernel 312).  The Helmholtz term, from B in fixed point loaded ahead of the
+// (N = 7, E = 32,768: 361 us; this kernel 274 with the weights in the factors and without the checks of small values, 285
+// with both as they are, 3.8 TB/s of u, G and w; even-odd FP32 pairs 407, the FP64 pipe 1900; odd n, column threads
+// without the fold, N = 8, E = 22,528: 660; this kernel 312 and 327).  The Helmholtz term, from B in fixed point loaded ahead of the
 // stores of w, adds 12% (308 us; converted from FP64 at each use, 25%).  Not kept: the r- and s-lines
 // through one copy of the code in a loop (no faster at N = 7, 4 to 11% slower above).
 #pragma once

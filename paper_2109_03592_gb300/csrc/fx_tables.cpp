@@ -32,7 +32,7 @@ void gll_points_ld(int N, std::vector<long double>& x) {
 namespace {
 
 // d = g 2^64 / (largest row sum of magnitudes): a contraction takes values below B to values below g B.  g = 0.8 keeps
-// the sums of fx::dot below 2^63 for values of 60 bits (at worst 2^62.66, N = 11, for these tables; a caller that scales
+// the sums of fx::dot below 2^63 for values of 60 bits (at worst 2^62.68, N = 9, for these tables; a caller that scales
 // them checks the sums again); an odd n has a middle point whose
 // entry stands for itself, and g = 0.5 keeps the entries below 2^63.
 FxScale build(int N) {
