@@ -8,7 +8,6 @@
 #include <memory>
 #include <string>
 
-#include "fixed.cuh"
 #include "fx_tables.h"
 #include "kernels.h"
 #include "sem_internal.h"
@@ -62,8 +61,6 @@ void free_mesh_arrays(sem_mesh* m) {
   dev_free(m->fx_sG);
   dev_free(m->Bfx);
   dev_free(m->fx_sB);
-  dev_free(m->fx_W);
-  dev_free(m->fx_tw);
   dev_free(m->fx_W64);
   dev_free(m->wq);
   dev_free(m->dK);
@@ -346,19 +343,9 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
     SEM_TRY(dev_alloc(&m->eodf, eodf.size(), tb));
   }
 
-  std::vector<long long> W;
-  std::vector<int> tw;
-  fx_weights(N, W, tw);
-  std::vector<int2> Wsplit(W.size());
-  std::vector<double> W64(W.size());
-  for (size_t q = 0; q < W.size(); ++q) {
-    Wsplit[q] = fx::split(W[q]);
-    W64[q] = std::ldexp((double)W[q], -tw[q % (n * n)]);
-  }
+  const std::vector<double> W64 = fx_weights(N);
   std::vector<double> w1(w);
   w1.resize(2 * n, 1.0);
-  SEM_TRY(dev_alloc(&m->fx_W, W.size(), tb));
-  SEM_TRY(dev_alloc(&m->fx_tw, tw.size(), tb));
   SEM_TRY(dev_alloc(&m->fx_W64, W64.size(), tb));
   SEM_TRY(dev_alloc(&m->wq, 2 * n, tb));
 
@@ -380,9 +367,7 @@ sem_status build_mesh(const sem_mesh_desc& d, cudaStream_t s, sem_mesh* m) {
 
   SEM_CUDA(cudaMemcpyAsync(xi_d, xi.data(), n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->wq, w1.data(), 2 * n * sizeof(double), cudaMemcpyHostToDevice, s));
-  SEM_CUDA(cudaMemcpyAsync(m->fx_W, Wsplit.data(), Wsplit.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->fx_W64, W64.data(), W64.size() * sizeof(double), cudaMemcpyHostToDevice, s));
-  SEM_CUDA(cudaMemcpyAsync(m->fx_tw, tw.data(), tw.size() * sizeof(int), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D64, D.data(), n * n * sizeof(double), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32, D32.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));
   SEM_CUDA(cudaMemcpyAsync(m->D32lo, D32lo.data(), n * n * sizeof(float), cudaMemcpyHostToDevice, s));

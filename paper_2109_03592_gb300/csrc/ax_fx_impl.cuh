@@ -27,8 +27,8 @@
 // that the shifts are written for (2^-500 .. 2^500), or whose small values stand
 // alone beside large ones (line_state) is evaluated in FP64 (element_fp64).
 //
-// What bounds it: issue, of multiply-adds and of the additions between them (integer pipe 57% busy, multiply pipe
-// 35%, DRAM 46%).  One thread per 2x2x2 octant instead of per line needed twice the shared-memory reads and splits
+// What bounds it: issue, of multiply-adds and of the additions between them (integer pipe 50% busy, multiply pipe
+// 35%, FP64 19%, DRAM 49%).  One thread per 2x2x2 octant instead of per line needed twice the shared-memory reads and splits
 // (N = 7, E = 32,768: 361 us; this kernel 274 with the weights in the factors and without the checks of small values, 285
 // with both as they are, 3.8 TB/s of u, G and w; even-odd FP32 pairs 407, the FP64 pipe 1900; odd n, column threads
 // without the fold, N = 8, E = 22,528: 660; this kernel 312 and 327).  The Helmholtz term, from B in fixed point loaded ahead of the
@@ -412,33 +412,19 @@ __global__ void __launch_bounds__(line_threads(N, EPB), line_blocks(N, EPB))
       mt.down = eo - em;
       if (helm) eo = max(eo, em);
     }
-    if (FUSED) eo += 64 - P.fx.tw[line];
-    // The weights: in FP64, whose pipe is idle, or for <p, A p> in integers, o W kept to 2^(64 - wb): |o| < 3 g 2^60 + 2^59
-    // (g: fx_tables.cpp) and W <= 2^62, so that stays below 2^63.  (Integers for both: 2697 us a plain apply at N = 7,
-    // E = 262,144.)
-    constexpr int wb = n % 2 ? 4 : 3;
-    ll ph = 0, pm = 0;
+    const double* v = FUSED ? (P.pout ? P.pout : P.p) : P.u;
 #pragma unroll
     for (int k = 0; k < n; ++k) {
       const int at = L::idx(x, y, k);
       ll o = wt[k] + R[at] + S[at];
       if (helm) o = mt.add(o, B[k], split(U[at]));
-      if (!FUSED) {
-        P.w[base + k * n2] = to_double(o, eo) * __ldg(P.fx.W64 + line + k * n2);
-      } else {
-        const int2 c = __ldg(P.fx.W + line + k * n2), v = split(o);
-        const ll m = mad(mad(0, c.x, v.y), c.y, v.x), h = (ll)c.y * v.y;
-        P.w[base + k * n2] = to_double(shl(h, wb) + ((m + (1ll << (31 - wb))) >> (32 - wb)), eo - wb);
-        // o W / 2^64 to nearest (a floor has the same sign in every line); two bits of p, which only scale it
-        const int2 a = split(U[at] >> 2), b = split(h + ((m + (1ll << 31)) >> 32));
-        ph = mad(ph, a.y, b.y);
-        pm = mad(mad(pm + __mulhi(a.x, b.x), a.x, b.y), a.y, b.x);  // (inside an element b is small: 2^-10 of its bound)
-      }
+      // The weights and <p, A p> in FP64, whose pipe is idle.  (In integers, a CG iteration at N = 7, E = 32,768: 661 to 669 us,
+      // 655 so; with p from its integers 661; a plain apply at E = 262,144 with the weights in integers 2697, 2667 so.)
+      const double w = to_double(o, eo) * __ldg(P.fx.W64 + line + k * n2);
+      if (FUSED) pw = fma(v[base + k * n2], w, pw);
+      P.w[base + k * n2] = w;
     }
-    // the lines' sums cancel in <p, A p> (smooth p: to 1e-4 of them and less), so their low halves count
-    if (FUSED) pw = ldexp(fma(__ll2double_rn(pm), 0x1p-32, __ll2double_rn(ph)), 64 + 2 + eo + eu);
     if (mass64) {
-      const double* v = FUSED ? (P.pout ? P.pout : P.p) : P.u;
 #pragma unroll 1
       for (int k = 0; k < n; ++k) {
         const double u = v[base + k * n2], t = P.h2 * P.B[base + k * n2] * u;

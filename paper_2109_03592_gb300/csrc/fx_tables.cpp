@@ -94,19 +94,12 @@ const FxScale& fx_scale(int N) {
   return table[N];
 }
 
-void fx_weights(int N, std::vector<long long>& W, std::vector<int>& tw) {
+std::vector<double> fx_weights(int N) {
   const FxScale& f = fx_scale(N);
   const int n = N + 1;
-  const long double wmax = *std::max_element(f.w.begin(), f.w.end());
-  W.resize((size_t)n * n * n);
-  tw.resize((size_t)n * n);
-  for (int ij = 0; ij < n * n; ++ij) {
-    const long double c = f.w[ij % n] * f.w[ij / n] * f.kappa;
-    int top = 0;
-    std::frexp(c * wmax, &top);
-    tw[ij] = 62 - top;
-    for (int k = 0; k < n; ++k) W[(size_t)k * n * n + ij] = std::llround(std::ldexp(c * f.w[k], tw[ij]));
-  }
+  std::vector<double> W((size_t)n * n * n);
+  for (int q = 0; q < n * n * n; ++q) W[q] = (double)(f.w[q % n] * f.w[q / n % n] * f.w[q / (n * n)] * f.kappa);
+  return W;
 }
 
 }  // namespace sem

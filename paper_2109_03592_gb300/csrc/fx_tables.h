@@ -15,9 +15,8 @@ struct FxScale {
 };
 const FxScale& fx_scale(int N);  // N = 1 .. 11; built once per order
 
-// w_i w_j w_k kappa of the points (FxOp::W) as integers of at most 62 bits, below the largest of their t-line (i, j) by
-// 2^-tw: W [n^3], tw [n^2].
-void fx_weights(int N, std::vector<long long>& W, std::vector<int>& tw);
+// w_i w_j w_k kappa of the points (FxOp::W64), [n^3].
+std::vector<double> fx_weights(int N);
 
 // GLL points of order N in long double.
 void gll_points_ld(int N, std::vector<long double>& x);

@@ -40,8 +40,6 @@ struct FxOp {
   const int2* sG = nullptr;   // [E]: sG; the bits from the element's largest factor to the least of its lines' largest
   const int2* B = nullptr;    // [E][n^3]: the mass without them, times 2^sB (both: 62 bits below the element's largest)
   const int* sB = nullptr;    // [E]
-  const int2* W = nullptr;    // [n^3]: w_i w_j w_k kappa 2^tw (fx_weights)
-  const int* tw = nullptr;    // [n^2]: tw of the t-line (i, j)
   const double* W64 = nullptr; // [n^3]: w_i w_j w_k kappa
   const double* wq = nullptr; // [n]: the weights
   int range = 0;              // the largest sG[].y

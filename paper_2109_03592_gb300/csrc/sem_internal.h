@@ -119,8 +119,6 @@ struct sem_mesh {
   int fx_range = 0;          // FxOp::range
   int2* Bfx = nullptr;       // [E][n3] FxOp::B, where Gfx is set
   int* fx_sB = nullptr;      // [E] FxOp::sB
-  int2* fx_W = nullptr;      // [n3] FxOp::W
-  int* fx_tw = nullptr;      // [n2] FxOp::tw
   double* fx_W64 = nullptr;  // [n3] FxOp::W64
   double* wq = nullptr;      // [2 n] GLL weights, then ones
   double* dK = nullptr;      // [n_local] QQ^T diag of the stiffness (h1 = 1, h2 = 0)
@@ -176,8 +174,6 @@ struct sem_mesh {
     f.range = cG32 ? cfx_range : fx_range;
     f.B = b;
     f.sB = cB64 ? cfx_sB : fx_sB;
-    f.W = fx_W;
-    f.tw = fx_tw;
     f.W64 = fx_W64;
     f.wq = wq;
     return f;
